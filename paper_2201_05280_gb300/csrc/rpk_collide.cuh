@@ -95,7 +95,10 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 ? 5 : 1)
   u_out[p] = m.j[0] * m.inv_rho;
   u_out[npts + p] = m.j[1] * m.inv_rho;
   u_out[2 * npts + p] = m.j[2] * m.inv_rho;
-  kap_out[p] = K.kapc * m.rho * (K.theta0 + m.dth);
+  if constexpr (kPaper)
+    kap_out[p] = K.kapc * m.rho * fmad(fmad(K.delta, m.dR, Real(3) * m.dT), K.inv_3pd, K.theta0);
+  else
+    kap_out[p] = K.kapc * m.rho * (K.theta0 + m.dth);
   if constexpr (kPaper) tt_out[p] = m.dT;  // paper mode: theta_T(f) - theta0 of time t
   flag_moments(m, K.theta0, status);
 }
@@ -124,7 +127,6 @@ __device__ __forceinline__ void flag_moments2(const Mom<F2>& m, float theta0, un
 // points per thread on a periodic grid with nx even, FP32 arithmetic in
 // packed FP32x2 form (the one-point kernel's FP32 arithmetic to rounding, half
 // the arithmetic instructions; pair words halve the loads and stores).
-// Thread (blockIdx.x * blockDim.x + threadIdx.x) owns x0 = 2 * that index.
 // kPaper: the paper's theta_R solver (the state holds theta_R - theta0; the
 // time-t theta_T(f) - theta0 goes to tt_out), as in k_collide.
 template <typename Store, bool kPaper = false>
@@ -135,14 +137,11 @@ __global__ void __launch_bounds__(128, sizeof(Store) == 4 ? 3 : 4)
                    float* __restrict__ tt_out) {
   using IO = PairIO<Store>;
   using Word = typename IO::Word;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (K.nx >> 1)) return;
-  const int y = blockIdx.y;
-  const int s = blockIdx.z / K.nz;
-  const int z = blockIdx.z - s * K.nz;
-  const int64_t n3p = K.n3 >> 1;                                     // pairs per sublattice
-  const int64_t cellp = ((((int64_t)z * K.ny + y) * K.nx) >> 1) + i;  // pair of the cell
-  const int64_t pp = (int64_t)s * n3p + cellp;                        // pair in a field plane
+  int s, i, y, z;
+  int64_t cellp;  // pair of the cell
+  if (!pair_from_block(K, s, i, y, z, cellp)) return;
+  const int64_t n3p = K.n3 >> 1;                // pairs per sublattice
+  const int64_t pp = (int64_t)s * n3p + cellp;  // pair in a field plane
   F2 h[kQ];
   gather_pair<Store>(reinterpret_cast<const Word*>(pin), K, s, i, y, z, h);
   Mom<F2> m;
@@ -177,13 +176,10 @@ __global__ void __launch_bounds__(128, kPaper ? 4 : 5)
                      float* __restrict__ tt_out) {
   static_assert(std::is_same<Store, __half>::value, "the word-holding collision serves FP16 storage");
   using IO = PairIO<Store>;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (K.nx >> 1)) return;
-  const int y = blockIdx.y;
-  const int s = blockIdx.z / K.nz;
-  const int z = blockIdx.z - s * K.nz;
+  int s, i, y, z;
+  int64_t cellp;
+  if (!pair_from_block(K, s, i, y, z, cellp)) return;
   const int64_t n3p = K.n3 >> 1;
-  const int64_t cellp = ((((int64_t)z * K.ny + y) * K.nx) >> 1) + i;
   const int64_t pp = (int64_t)s * n3p + cellp;
   unsigned hw[kQ];
   gather_pair_words<Store>(reinterpret_cast<const unsigned*>(pin), K, s, i, y, z, hw);

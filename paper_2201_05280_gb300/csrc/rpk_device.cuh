@@ -61,9 +61,23 @@ __device__ __forceinline__ void static_for(F&& f) {
 // ---------------------------------------------------------------------------
 // per-launch constants (host fills them in double, then casts)
 
+// Division of a 32-bit index by a launch constant: n / d = (umulhi(m, n) + n) >> l
+// for n < 2^31 (m = floor(2^32 (2^l - d) / d) + 1, l = ceil(log2 d)).
+struct FastDiv {
+  unsigned m, l;
+  FastDiv() = default;
+  explicit FastDiv(unsigned d) {
+    l = 0;
+    while ((1ull << l) < d) ++l;
+    m = (unsigned)(((1ull << 32) * ((1ull << l) - d)) / d + 1);
+  }
+  __device__ __forceinline__ unsigned div(unsigned n) const { return (__umulhi(m, n) + n) >> l; }
+};
+
 template <typename Real>
 struct StepConst {
   int nx, ny, nz;
+  FastDiv by_nx, by_ny, by_nxp;  // division by nx, ny and nx / 2
   int64_t n3;     // nx*ny*nz
   Real theta0;
   Real c_keep;    // 1 - 2 beta*
@@ -307,14 +321,35 @@ struct PointIdx {
   int64_t cell;  // (z*ny + y)*nx + x
 };
 
+// Point of a thread: consecutive threads take consecutive cells of sublattice
+// blockIdx.y, across the ends of rows, so every thread of every block but the
+// last has a point whatever nx is (n3 < 2^31: the populations of more cells
+// would not fit any device).
 template <typename Real>
 __device__ __forceinline__ bool point_from_block(const StepConst<Real>& K, PointIdx& P) {
-  P.x = blockIdx.x * blockDim.x + threadIdx.x;
-  P.y = blockIdx.y;
-  P.s = blockIdx.z / K.nz;
-  P.z = blockIdx.z - P.s * K.nz;
-  if (P.x >= K.nx) return false;
-  P.cell = ((int64_t)P.z * K.ny + P.y) * K.nx + P.x;
+  const unsigned c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= (unsigned)K.n3) return false;
+  const unsigned row = K.by_nx.div(c), z = K.by_ny.div(row);
+  P.s = blockIdx.y;
+  P.x = (int)(c - row * K.nx);
+  P.y = (int)(row - z * K.ny);
+  P.z = (int)z;
+  P.cell = c;
+  return true;
+}
+
+// As point_from_block for pairs of x-adjacent points (nx even): pair c of the sublattice
+// is column i of row (y, z).
+__device__ __forceinline__ bool pair_from_block(const StepConst<float>& K, int& s, int& i, int& y, int& z,
+                                                int64_t& cellp) {
+  const unsigned c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= (unsigned)(K.n3 >> 1)) return false;
+  const unsigned row = K.by_nxp.div(c), zz = K.by_ny.div(row);
+  s = blockIdx.y;
+  i = (int)(c - row * (unsigned)(K.nx >> 1));
+  y = (int)(row - zz * K.ny);
+  z = (int)zz;
+  cellp = c;
   return true;
 }
 

@@ -652,7 +652,7 @@ __device__ __forceinline__ void init_point(const StepConst<Real>& K, Real half_d
   // E_R = delta rho theta_R/2 as a deviation from delta theta0/2 (paper mode:
   // the state is theta_R - theta0)
   e = K.paper ? dR
-              : Real(0.5) * K.delta * (rho * dR + K.theta0 * drho) -
+              : Real(0.5) * K.delta * fmad(K.theta0, drho, rho * dR) -
                     half_dt_over_tau1 * Real(0.5) * K.delta * rho * (dth - dR);
 }
 

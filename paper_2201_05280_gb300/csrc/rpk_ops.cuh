@@ -24,6 +24,9 @@ static StepConst<Real> make_step_const(const rpk_relax& r, int nsub, int nx, int
   K.ny = ny;
   K.nz = nz;
   K.n3 = (int64_t)nx * ny * nz;
+  K.by_nx = FastDiv((unsigned)nx);
+  K.by_ny = FastDiv((unsigned)ny);
+  K.by_nxp = FastDiv((unsigned)std::max(1, nx / 2));
   K.theta0 = Real(kTheta0);
   K.c_keep = Real(1.0 - 2.0 * beta);
   K.c_relax = Real(2.0 * beta);
@@ -54,10 +57,21 @@ static StepConst<Real> make_const(const rpk_lattice* L) {
   return make_step_const<Real>(L->relax, L->nsub, L->grid.nx, L->grid.ny, L->grid.nz, L->rot_mode);
 }
 
-static inline dim3 point_grid(const rpk_lattice* L, int bx) {
-  return dim3((unsigned)((L->grid.nx + bx - 1) / bx), (unsigned)L->grid.ny,
-              (unsigned)(2 * L->grid.nz));
+// Threads per block for n points or pairs per sublattice: 128, or fewer (down
+// to one warp) while the two sublattices' blocks would leave SMs without one.
+static inline int block_for(const rpk_lattice* L, int64_t n) {
+  int b = 128;
+  while (b > 32 && 2 * ((n + b - 1) / b) < L->sms) b /= 2;
+  return b;
 }
+
+// Launch shape of a kernel with one point (n = n3) or pair (n = n3 / 2) per thread.
+struct PointLaunch {
+  dim3 grid;
+  int block;
+  PointLaunch(const rpk_lattice* L, int64_t n)
+      : grid((unsigned)((n + block_for(L, n) - 1) / block_for(L, n)), 2), block(block_for(L, n)) {}
+};
 
 static inline rpk_status check_launch(const char* what) {
   cudaError_t err = cudaGetLastError();
@@ -97,26 +111,26 @@ static rpk_status collide_launch(rpk_lattice* L, const StepConst<Real>& K) {
   Store* pout = static_cast<Store*>(L->pop[L->cur ^ 1]);
   Real* ucur = static_cast<Real*>(L->u[L->steps & 1]);
   const Real* wcol = static_cast<const Real*>(L->wrho);
+  const PointLaunch pt(L, L->n3);
   if (L->rot_mode) {
     if constexpr (kPull && kBC == 0 && sizeof(Real) == 4) {
       if (L->grid.nx % 2 == 0) {
         // two x-adjacent points per thread, packed FP32x2 arithmetic
-        const dim3 grid((unsigned)((L->grid.nx / 2 + 127) / 128), (unsigned)L->grid.ny,
-                        (unsigned)(2 * L->grid.nz));
+        const PointLaunch at(L, L->n3 / 2);
         if constexpr (std::is_same<Store, __half>::value)
-          k_collide_pair_w<Store, true><<<grid, 128, 0, L->stream>>>(
+          k_collide_pair_w<Store, true><<<at.grid, at.block, 0, L->stream>>>(
               K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
               static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status,
               static_cast<Real*>(L->thbuf));
         else
-          k_collide_pair<Store, true><<<grid, 128, 0, L->stream>>>(
+          k_collide_pair<Store, true><<<at.grid, at.block, 0, L->stream>>>(
               K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
               static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status,
               static_cast<Real*>(L->thbuf));
         return check_launch("k_collide_pair");
       }
     }
-    k_collide<Store, Real, kPull, kBC, true><<<point_grid(L, 128), 128, 0, L->stream>>>(
+    k_collide<Store, Real, kPull, kBC, true><<<pt.grid, pt.block, 0, L->stream>>>(
         K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
         static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap),
         static_cast<const Real*>(L->ghost), L->status, static_cast<Real*>(L->thbuf), wcol);
@@ -125,21 +139,20 @@ static rpk_status collide_launch(rpk_lattice* L, const StepConst<Real>& K) {
   if constexpr (kPull && kBC == 0 && sizeof(Real) == 4) {
     if (L->grid.nx % 2 == 0) {
       // two x-adjacent points per thread, packed FP32x2 arithmetic
-      const dim3 grid((unsigned)((L->grid.nx / 2 + 127) / 128), (unsigned)L->grid.ny,
-                      (unsigned)(2 * L->grid.nz));
+      const PointLaunch at(L, L->n3 / 2);
       // FP16 storage holds the pair words, not their FP32 values, across the collision
       if constexpr (std::is_same<Store, __half>::value)
-        k_collide_pair_w<Store, false><<<grid, 128, 0, L->stream>>>(
+        k_collide_pair_w<Store, false><<<at.grid, at.block, 0, L->stream>>>(
             K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
             static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status, nullptr);
       else
-        k_collide_pair<Store, false><<<grid, 128, 0, L->stream>>>(
+        k_collide_pair<Store, false><<<at.grid, at.block, 0, L->stream>>>(
             K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
             static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status, nullptr);
       return check_launch("k_collide_pair");
     }
   }
-  k_collide<Store, Real, kPull, kBC, false><<<point_grid(L, 128), 128, 0, L->stream>>>(
+  k_collide<Store, Real, kPull, kBC, false><<<pt.grid, pt.block, 0, L->stream>>>(
       K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
       static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap),
       static_cast<const Real*>(L->ghost), L->status, nullptr, wcol);
@@ -148,7 +161,7 @@ static rpk_status collide_launch(rpk_lattice* L, const StepConst<Real>& K) {
 
 template <typename Real, int kBC>
 static rpk_status transport_launch(rpk_lattice* L, const StepConst<Real>& K) {
-  const dim3 grid = point_grid(L, 128);
+  const PointLaunch pt(L, L->n3);
   const Real* ucur = static_cast<const Real*>(L->u[L->steps & 1]);
   const Real* uprev = static_cast<const Real*>(L->u[(L->steps + 1) & 1]);
   const Real* gh = static_cast<const Real*>(L->ghost);
@@ -217,7 +230,7 @@ static rpk_status transport_launch(rpk_lattice* L, const StepConst<Real>& K) {
   Real* src = dst;
   for (int k = 1; k < L->nsub; ++k) {
     dst = (k == L->nsub - 1) ? e : (src == ea ? eb : ea);
-    k_ftcs<Real, kBC><<<grid, 128, 0, L->stream>>>(K, src, drho, kap, dst, gh);
+    k_ftcs<Real, kBC><<<pt.grid, pt.block, 0, L->stream>>>(K, src, drho, kap, dst, gh);
     src = dst;
   }
   RPK_CUDA(timing_end(L, RPK_KC_TRANSPORT, 2 + L->nsub));
@@ -273,7 +286,8 @@ rpk_status Ops<Store, Real>::init(rpk_lattice* L, const double* rho, const doubl
   L->cur = 0;
   unsigned long long* check = reinterpret_cast<unsigned long long*>(L->diag_out);
   RPK_CUDA(cudaMemsetAsync(check, 0, 2 * sizeof(unsigned long long), L->stream));
-  k_init<Store, Real><<<point_grid(L, 128), 128, 0, L->stream>>>(
+  const PointLaunch pt(L, L->n3);
+  k_init<Store, Real><<<pt.grid, pt.block, 0, L->stream>>>(
       K, hdt, rho, u, T, R, static_cast<Store*>(L->pop[0]), static_cast<Real*>(L->e),
       static_cast<Real*>(L->u[0]), static_cast<Real*>(L->u[1]), check);
   return check_launch("k_init");
@@ -322,25 +336,25 @@ rpk_status Ops<Store, Real>::moments(rpk_lattice* L, double* rho, double* u, dou
   const Real* e = static_cast<const Real*>(L->e);
   const Real* gh = static_cast<const Real*>(L->ghost);
   const Real* wcol = static_cast<const Real*>(L->wrho);
-  const dim3 grid = point_grid(L, 128);
+  const PointLaunch pt(L, L->n3);
   const bool res = L->grid.bc_x == RPK_BC_RESERVOIR;
   const int wm = wall_mask(L);
   if (L->streamed) {
-    k_moments<Store, Real, false, 0><<<grid, 128, 0, L->stream>>>(K, pin, e, gh, rho, u, T, R, E, wcol);
+    k_moments<Store, Real, false, 0><<<pt.grid, pt.block, 0, L->stream>>>(K, pin, e, gh, rho, u, T, R, E, wcol);
   } else if (wm) {
     rpk_status st = wall_launch<Store, Real>(L, K);
     if (st != RPK_OK) return st;
     if (wm == kWallY)
-      k_moments<Store, Real, true, kWallY><<<grid, 128, 0, L->stream>>>(K, pin, e, gh, rho, u, T, R, E, wcol);
+      k_moments<Store, Real, true, kWallY><<<pt.grid, pt.block, 0, L->stream>>>(K, pin, e, gh, rho, u, T, R, E, wcol);
     else if (wm == kWallX)
-      k_moments<Store, Real, true, kWallX><<<grid, 128, 0, L->stream>>>(K, pin, e, gh, rho, u, T, R, E, wcol);
+      k_moments<Store, Real, true, kWallX><<<pt.grid, pt.block, 0, L->stream>>>(K, pin, e, gh, rho, u, T, R, E, wcol);
     else
-      k_moments<Store, Real, true, kWallY | kWallX><<<grid, 128, 0, L->stream>>>(K, pin, e, gh, rho, u, T, R,
+      k_moments<Store, Real, true, kWallY | kWallX><<<pt.grid, pt.block, 0, L->stream>>>(K, pin, e, gh, rho, u, T, R,
                                                                                 E, wcol);
   } else if (res) {
-    k_moments<Store, Real, true, 1><<<grid, 128, 0, L->stream>>>(K, pin, e, gh, rho, u, T, R, E, wcol);
+    k_moments<Store, Real, true, 1><<<pt.grid, pt.block, 0, L->stream>>>(K, pin, e, gh, rho, u, T, R, E, wcol);
   } else {
-    k_moments<Store, Real, true, 0><<<grid, 128, 0, L->stream>>>(K, pin, e, gh, rho, u, T, R, E, wcol);
+    k_moments<Store, Real, true, 0><<<pt.grid, pt.block, 0, L->stream>>>(K, pin, e, gh, rho, u, T, R, E, wcol);
   }
   return check_launch("k_moments");
 }
