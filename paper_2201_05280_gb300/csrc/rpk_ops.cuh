@@ -159,6 +159,34 @@ static rpk_status collide_launch(rpk_lattice* L, const StepConst<Real>& K) {
   return check_launch("k_collide");
 }
 
+// Transport of a quasi-1-D lattice: nsub sub-steps in equal parts of at most
+// kLineSub, the first part with the MacCormack passes; returns the launches.
+// Tiles of 64 points while that leaves no more tiles than SMs (FP64 issues two
+// lanes per cycle and SM, so narrow tiles on every SM beat wide ones on a
+// few), else 128.
+template <typename Real, int kBC>
+static int line_launches(rpk_lattice* L, const StepConst<Real>& K, const Real* es, const Real* ucur,
+                         const Real* uprev, const Real* drho, const Real* kap, Real* e, Real* ea, Real* eb,
+                         const Real* gh) {
+  const int parts = (L->nsub + kLineSub - 1) / kLineSub;
+  const Real* src = es;
+  for (int i = 0, done = 0; i < parts; ++i) {
+    const int m = (L->nsub - done + parts - i - 1) / (parts - i);
+    const int halo = 2 * (m + (i == 0 ? 1 : 0));
+    const int tile = 2 * ((L->grid.nx + 63 - halo) / (64 - halo)) <= L->sms ? 64 : 128;
+    const dim3 grid((unsigned)((L->grid.nx + tile - halo - 1) / (tile - halo)), 2);
+    const size_t smem = 2 * tile * sizeof(Real);
+    Real* dst = i == parts - 1 ? e : (src == ea ? eb : ea);
+    if (i == 0)
+      k_line_transport<Real, kBC, true><<<grid, tile, smem, L->stream>>>(K, src, ucur, uprev, drho, kap, dst, gh, m);
+    else
+      k_line_transport<Real, kBC, false><<<grid, tile, smem, L->stream>>>(K, src, ucur, uprev, drho, kap, dst, gh, m);
+    src = dst;
+    done += m;
+  }
+  return parts;
+}
+
 template <typename Real, int kBC>
 static rpk_status transport_launch(rpk_lattice* L, const StepConst<Real>& K) {
   const PointLaunch pt(L, L->n3);
@@ -208,6 +236,13 @@ static rpk_status transport_launch(rpk_lattice* L, const StepConst<Real>& K) {
     }
     RPK_CUDA(timing_end(L, RPK_KC_TRANSPORT, 2 + L->nsub));
     return check_launch("rotational transport (paper mode)");
+  }
+  if constexpr (kBC == 0 || kBC == 1) {
+    if (L->grid.ny == 1 && L->grid.nz == 1) {
+      const int n = line_launches<Real, kBC>(L, K, es, ucur, uprev, drho, kap, e, ea, eb, gh);
+      RPK_CUDA(timing_end(L, RPK_KC_TRANSPORT, n));
+      return check_launch("rotational transport (line)");
+    }
   }
   // predictor, corrector and the first FTCS sub-step; further sub-steps end in e
   Real* dst = L->nsub == 1 ? e : ea;
