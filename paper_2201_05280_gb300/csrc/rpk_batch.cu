@@ -49,12 +49,97 @@ __device__ __forceinline__ PointIdx tube_point(int nx, int p) {
   return P;
 }
 
-template <typename Store, typename Real, int kThreads>
+// FTCS sub-steps of a tube's two sublattice lines, several per block barrier.
+// A warp takes a piece of a line, kP consecutive points per lane, in
+// registers: neighbours inside a lane are registers, those of the next lane
+// one shuffle each side, so m <= kP sub-steps need no barrier; lanes 0 and 31
+// are halo (recomputed by the neighbouring pieces) and the 30 lanes between
+// are written. kP is odd: 32 lanes reading with stride kP hit 32 banks.
+// Bound: the FP32 pipes (theta, the face difference, two products and the update
+// of every point and sub-step) and the chain of one sub-step. Arithmetic in the
+// order of the lattice's FTCS kernels, so results are those of one barrier per
+// sub-step bit for bit.
+// With a block barrier and 10 shared loads per point and sub-step it took 0.8
+// us a sub-step for the largest tubes (1500 cells, FTCS_OLDNEW).
+template <typename Real>
+struct FtcsLine {
+  const Real* a;     // theta_R - theta0 = a e + c
+  const Real* c;
+  const Real* face;  // K of the face below each point
+  const Real* last;  // and of the face above the last point, per line
+  const Real* th0;   // theta_R - theta0 of the corrector, for the first sub-step
+  int nx;
+  Real h;             // dt / nsub
+  Real th_lo, th_hi;  // reservoir values
+};
+
+template <int kP, typename Real>
+__device__ __forceinline__ void ftcs_pass(const FtcsLine<Real>& L, const Real* ein, Real* eout, int m,
+                                          int nwarps, bool first) {
+  const int lane = threadIdx.x & 31;
+  const int nx = L.nx, pieces = (nx + 30 * kP - 1) / (30 * kP);
+  for (int w = threadIdx.x >> 5; w < 2 * pieces; w += nwarps) {
+    const int s = w >= pieces, x0 = (w - s * pieces) * 30 * kP + (lane - 1) * kP;
+    const int off = s * nx;
+    Real e[kP], a[kP], c[kP], f[kP + 1], th[kP];
+#pragma unroll
+    for (int i = 0; i < kP; ++i) {
+      const int x = x0 + i;
+      const bool in = x >= 0 && x < nx;
+      // beyond an end: theta stays the reservoir's (a = 0)
+      e[i] = in ? ein[off + x] : Real(0);
+      a[i] = in ? L.a[off + x] : Real(0);
+      c[i] = in ? L.c[off + x] : (x < 0 ? L.th_lo : L.th_hi);
+      f[i] = in ? L.face[off + x] : (x == nx ? L.last[s] : Real(0));
+    }
+    f[kP] = __shfl_down_sync(0xffffffffu, f[0], 1);
+#pragma unroll
+    for (int i = 0; i < kP; ++i)
+      th[i] = first && x0 + i >= 0 && x0 + i < nx ? L.th0[off + x0 + i] : fmad(a[i], e[i], c[i]);
+    for (int k = 0; k < m; ++k) {
+      const Real lo = __shfl_up_sync(0xffffffffu, th[kP - 1], 1);
+      const Real hi = __shfl_down_sync(0xffffffffu, th[0], 1);
+      Real d = th[0] - lo;
+#pragma unroll
+      for (int i = 0; i < kP; ++i) {
+        const Real dn = (i + 1 < kP ? th[i + 1] : hi) - th[i];
+        e[i] = fmad(L.h, fmad(f[i + 1], dn, -(f[i] * d)), e[i]);
+        d = dn;
+      }
+#pragma unroll
+      for (int i = 0; i < kP; ++i) th[i] = fmad(a[i], e[i], c[i]);
+    }
+    if (lane > 0 && lane < 31) {
+#pragma unroll
+      for (int i = 0; i < kP; ++i)
+        if (x0 + i < nx) eout[off + x0 + i] = e[i];
+    }
+  }
+}
+
+// Points per lane of ftcs_pass: the fewest point slots per warp over the
+// rounds that a tube's pieces take; among equals the widest (fewest barriers).
+template <typename Real>
+__device__ __forceinline__ int ftcs_width(int nx, int nwarps) {
+  if (sizeof(Real) == 8) return 5;
+  int best = 5, cost = 1 << 30;
+  for (int w = 5; w <= 13; w += (w < 9 ? 2 : 4)) {
+    const int pieces = 2 * ((nx + 30 * w - 1) / (30 * w));
+    const int c = (pieces + nwarps - 1) / nwarps * w;
+    if (c <= cost) {
+      cost = c;
+      best = w;
+    }
+  }
+  return best;
+}
+
+template <typename Store, typename Real, int kThreads, bool kImplicit>
 __global__ void __launch_bounds__(kThreads)
     k_batch(TubeDev<Real>* __restrict__ tubes, const int* __restrict__ order, int ntubes,
             int* __restrict__ counter, Store* __restrict__ pop0, Store* __restrict__ pop1,
             Real* __restrict__ e_state, Real* __restrict__ ux_state, float* __restrict__ snaps,
-            int save_every, int max_np, int implicit, unsigned* __restrict__ status) {
+            int save_every, int max_np, unsigned* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* sE = reinterpret_cast<Real*>(smem_raw);  // auxiliary E_R (state), then corrector
   Real* sS = sE + max_np;                        // e* after exchange, then theta_R
@@ -64,6 +149,7 @@ __global__ void __launch_bounds__(kThreads)
   Real* sK = sD + max_np;                        // kappa_R
   Real* sP = sK + max_np;                        // predictor
   __shared__ int s_slot;
+  __shared__ Real s_last[2];  // K of each line's last face
   const int tid = threadIdx.x;
   for (;;) {
     __syncthreads();
@@ -160,7 +246,7 @@ __global__ void __launch_bounds__(kThreads)
         sS[p] = (Real(2) * val - t0d * dr) / (K.delta * (Real(1) + dr));
       }
       __syncthreads();
-      if (implicit) {
+      if constexpr (kImplicit) {
         // 4'. backward-Euler variant: per sublattice line solve
         //     (delta rho / 2) phi - dt [K+ (phi_+ - phi) - K- (phi - phi_-)] = e - delta theta0 D / 2
         //     for phi = theta_R - theta0 by cyclic reduction in shared memory:
@@ -237,55 +323,45 @@ __global__ void __launch_bounds__(kThreads)
         }
         __syncthreads();
       } else {
-        // 4. FTCS sub-steps: e += h sum_faces K_face (theta_nb - theta). The first
-        //    uses theta_R of the corrector (sS) and updates e in place; later ones
-        //    use theta_R = a e + c with a = 2/(delta(1 + D)), c = -delta theta0 D/(delta(1 + D))
-        //    (affine in e at fixed rho), ping-ponging e between sE and sS with one
-        //    barrier per sub-step.
+        // 4. FTCS sub-steps, e += h sum_faces K_face (theta_nb - theta) with
+        //    theta_R = a e + c, a = 2/(delta(1 + D)), c = -delta theta0 D/(delta(1 + D))
+        //    (affine in e at fixed rho; the first sub-step takes the corrector's
+        //    theta_R): a -> sP, c -> sD, K of every point's low face -> the u(t-1)
+        //    slot (dead until the next step's u), e between sE and sK.
+        Real* face = (t & 1) ? sU0 : sU1;
         for (int p = tid; p < np; p += kThreads) {
           const int s = p >= nx, x = p - s * nx;
-          const Real thp = sS[p], kp = sK[p];
-          const Real thm = x == 0 ? thGl : sS[p - 1], km = x == 0 ? gl[kGhKap] : sK[p - 1];
-          const Real thq = x + 1 >= nx ? thGh : sS[p + 1], kq = x + 1 >= nx ? gh[kGhKap] : sK[p + 1];
-          Real acc = Real(0);
-          acc += Real(0.5) * (kp + km) * (thm - thp);
-          acc += Real(0.5) * (kp + kq) * (thq - thp);
-          sE[p] = sE[p] + K.hsub * acc;
+          const Real dr = sD[p], kp = sK[p];
+          const Real inv = Real(1) / (K.delta * (Real(1) + dr));
+          sP[p] = Real(2) * inv;
+          sD[p] = -t0d * dr * inv;
+          face[p] = Real(0.5) * (kp + (x == 0 ? gl[kGhKap] : sK[p - 1]));
+          if (x == nx - 1) s_last[s] = Real(0.5) * (kp + gh[kGhKap]);
         }
         __syncthreads();
-        if (nsub > 1) {
-          for (int p = tid; p < np; p += kThreads) {
-            const Real dr = sD[p];
-            const Real inv = Real(1) / (K.delta * (Real(1) + dr));
-            sP[p] = Real(2) * inv;    // a
-            sD[p] = -t0d * dr * inv;  // c
+        const FtcsLine<Real> FL{sP, sD, face, s_last, sS, nx, K.hsub, thGl, thGh};
+        Real* ein = sE;
+        Real* eout = sK;
+        const int width = ftcs_width<Real>(nx, kThreads / 32);
+        for (int k = 0; k < nsub;) {
+          const int m = min(nsub - k, width);
+          if constexpr (sizeof(Real) == 8) {
+            ftcs_pass<5>(FL, ein, eout, m, kThreads / 32, k == 0);
+          } else {
+            if (width == 5) ftcs_pass<5>(FL, ein, eout, m, kThreads / 32, k == 0);
+            else if (width == 7) ftcs_pass<7>(FL, ein, eout, m, kThreads / 32, k == 0);
+            else if (width == 9) ftcs_pass<9>(FL, ein, eout, m, kThreads / 32, k == 0);
+            else ftcs_pass<13>(FL, ein, eout, m, kThreads / 32, k == 0);
           }
+          k += m;
           __syncthreads();
-          Real* ein = sE;
-          Real* eout = sS;
-          for (int k = 1; k < nsub; ++k) {
-            for (int p = tid; p < np; p += kThreads) {
-              const int s = p >= nx, x = p - s * nx;
-              const Real ep = ein[p];
-              const Real thp = sP[p] * ep + sD[p], kp = sK[p];
-              const Real thm = x == 0 ? thGl : sP[p - 1] * ein[p - 1] + sD[p - 1];
-              const Real km = x == 0 ? gl[kGhKap] : sK[p - 1];
-              const Real thq = x + 1 >= nx ? thGh : sP[p + 1] * ein[p + 1] + sD[p + 1];
-              const Real kq = x + 1 >= nx ? gh[kGhKap] : sK[p + 1];
-              Real acc = Real(0);
-              acc += Real(0.5) * (kp + km) * (thm - thp);
-              acc += Real(0.5) * (kp + kq) * (thq - thp);
-              eout[p] = ep + K.hsub * acc;
-            }
-            __syncthreads();
-            Real* tmp = ein;
-            ein = eout;
-            eout = tmp;
-          }
-          if (ein != sE) {
-            for (int p = tid; p < np; p += kThreads) sE[p] = ein[p];
-            __syncthreads();
-          }
+          Real* tmp = ein;
+          ein = eout;
+          eout = tmp;
+        }
+        if (ein != sE) {
+          for (int p = tid; p < np; p += kThreads) sE[p] = ein[p];
+          __syncthreads();
         }
       }
       cur ^= 1;
@@ -468,14 +544,20 @@ namespace {
 
 template <typename Store, typename Real>
 struct BatchOps {
-  static void* kernel(int threads) {
+  // one kernel per thread count and diffusion, so that neither form's registers
+  // bind the other
+  template <bool kImplicit>
+  static void* kernel_of(int threads) {
     switch (threads) {
-      case 128: return (void*)k_batch<Store, Real, 128>;
-      case 256: return (void*)k_batch<Store, Real, 256>;
-      case 384: return (void*)k_batch<Store, Real, 384>;
-      case 512: return (void*)k_batch<Store, Real, 512>;
+      case 128: return (void*)k_batch<Store, Real, 128, kImplicit>;
+      case 256: return (void*)k_batch<Store, Real, 256, kImplicit>;
+      case 384: return (void*)k_batch<Store, Real, 384, kImplicit>;
+      case 512: return (void*)k_batch<Store, Real, 512, kImplicit>;
       default: return nullptr;
     }
+  }
+  static void* kernel(int threads, int implicit) {
+    return implicit ? kernel_of<true>(threads) : kernel_of<false>(threads);
   }
 };
 
@@ -555,7 +637,7 @@ rpk_status upload_tubes(rpk_batch* B) {
 // Shared-memory limit of the kernel variant (outside any stream capture).
 template <typename Store, typename Real>
 rpk_status prepare_batch(rpk_batch* B, int threads) {
-  void* kfn = BatchOps<Store, Real>::kernel(threads);
+  void* kfn = BatchOps<Store, Real>::kernel(threads, B->implicit);
   if (!kfn) return fail(RPK_ERR_ARG, "unsupported thread count");
   RPK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)batch_smem(B)));
@@ -575,20 +657,11 @@ rpk_status launch_batch(rpk_batch* B, cudaStream_t stream, int threads, int ctas
   Real* es = static_cast<Real*>(B->e_state);
   Real* us = static_cast<Real*>(B->ux_state);
   const int max_np = 2 * B->max_nx;
-  switch (threads) {
-#define RPK_LAUNCH(NT)                                                                         \
-  case NT:                                                                                     \
-    k_batch<Store, Real, NT><<<grid, NT, smem, stream>>>(tubes, B->order_dev, B->ntubes,       \
-                                                         B->counter, p0, p1, es, us, B->snaps, \
-                                                         B->save_every, max_np, B->implicit,   \
-                                                         B->status);                           \
-    break;
-    RPK_LAUNCH(128)
-    RPK_LAUNCH(256)
-    RPK_LAUNCH(384)
-    RPK_LAUNCH(512)
-#undef RPK_LAUNCH
-  }
+  void* kfn = BatchOps<Store, Real>::kernel(threads, B->implicit);
+  int ntubes = B->ntubes, save_every = B->save_every;
+  void* args[] = {&tubes, &B->order_dev, &ntubes, &B->counter, &p0,         &p1,
+                  &es,    &us,           &B->snaps, &save_every, (void*)&max_np, &B->status};
+  RPK_CUDA(cudaLaunchKernel(kfn, dim3(grid), dim3(threads), args, smem, stream));
   RPK_CUDA(cudaGetLastError());
   return RPK_OK;
 }
