@@ -38,6 +38,27 @@ __device__ __forceinline__ V collide_relax(const StepConst<Real>& K, Mom<V>& m, 
     return fmad(K.exc * m.rho, m.dth - m.dR, e);
 }
 
+// The same with the shell-wise sums and targets: about 470 operations a point
+// instead of 690 (FP64: 760 to 530 instructions of its pipe).
+template <typename Real, bool kPaper, typename V, typename Emit>
+__device__ __forceinline__ V collide_shells(const StepConst<Real>& K, const V (&h)[kQ], V e, Emit&& emit,
+                                            Mom<V>& m) {
+  raw_moments_shells(h, m);
+  recover<Real, kPaper, true>(m, e, K);
+  Herm<V> H;
+  mix_coeffs(m, K, H);
+  herm_scale(H, K.c_relax);
+  emit(0, fmad(K.c_keep, h[0], H.e0));
+  herm_shells(H, [&](int k, V ev, V od) {
+    emit(2 * k + 1, fmad(K.c_keep, h[2 * k + 1], ev + od));
+    emit(2 * k + 2, fmad(K.c_keep, h[2 * k + 2], ev - od));
+  });
+  if constexpr (kPaper)
+    return fmad(K.ra_keep, m.dR, K.ra_t * m.dT);
+  else
+    return fmad(K.exc * m.rho, m.dth - m.dR, e);
+}
+
 template <typename Real, bool kPaper = false, typename V, typename Emit>
 __device__ __forceinline__ V collide_emit(const StepConst<Real>& K, const V (&h)[kQ], V e, Emit&& emit,
                                           Mom<V>& m) {
@@ -50,8 +71,11 @@ template <typename Store, typename Real, bool kPaper = false>
 __device__ __forceinline__ Real collide_point(const StepConst<Real>& K, const Real (&h)[kQ], Real e,
                                               Store* __restrict__ out, Mom<Real>& m) {
   const int64_t n3 = K.n3;
-  return collide_emit<Real, kPaper>(
-      K, h, e, [&](int q, Real v) { out[(int64_t)q * n3] = from_real<Store, Real>(v); }, m);
+  auto put = [&](int q, Real v) { out[(int64_t)q * n3] = from_real<Store, Real>(v); };
+  if constexpr (kShells<Store>)
+    return collide_shells<Real, kPaper>(K, h, e, put, m);
+  else
+    return collide_emit<Real, kPaper>(K, h, e, put, m);
 }
 
 // Device status flags: 1 non-finite moment, 2 rho <= 0, 4 theta_T or theta_R <= 0.

@@ -93,6 +93,7 @@ struct StepConst {
   Real exc;       // dt delta / (2 tau1)
   Real kapc;      // k_r 5 tau / (2 B), kappa_R = kapc * rho * theta
   Real E0;        // delta theta0 / 2
+  Real inv_delta; // 1 / delta
   Real dt;
   Real hsub;      // dt / nsub
   // paper mode of the rotational solver (Sec. 5, four steps on theta_R):
@@ -160,6 +161,65 @@ __device__ __forceinline__ void raw_moments(const V (&h)[kQ], Mom<V>& m) {
   m.dP[3] = pxy; m.dP[4] = pxz; m.dP[5] = pyz;
 }
 
+// The same sums shell by shell: the weight of a shell multiplies the shell's
+// sums once instead of every pair, and the sign patterns of the (1, 1, 1) and
+// (1/2, 1/2, 1/2) pairs, (+++), (++-), (+-+), (+--), are one 4-point butterfly for
+// the even and one for the odd parts: 138 operations instead of 214. For
+// storage of 32 bits and more (another order of rounding flips last bits of
+// 16-bit values).
+template <typename V>
+__device__ __forceinline__ void raw_moments_shells(const V (&h)[kQ], Mom<V>& m) {
+  using S = scalar_t<V>;
+  constexpr S w1 = S(pair_weight(0)), w2 = S(pair_weight(3)), wf = S(pair_weight(6)), wc = S(pair_weight(12)),
+              wh = S(pair_weight(16));
+  constexpr S w2j = S(2 * pair_weight(3)), w2p = S(4 * pair_weight(3)), whj = S(0.5 * pair_weight(16)),
+              whp = S(0.25 * pair_weight(16));
+  auto ev = [&](int k) { return h[2 * k + 1] + h[2 * k + 2]; };
+  auto od = [&](int k) { return h[2 * k + 1] - h[2 * k + 2]; };
+  // axes
+  const V s0 = ev(0), s1 = ev(1), s2 = ev(2), s3 = ev(3), s4 = ev(4), s5 = ev(5);
+  // face diagonals: planes xy, xz, yz
+  const V ap = ev(6), am = ev(7), bp = ev(8), bm = ev(9), cp = ev(10), cm = ev(11);
+  const V A = ap + am, B = bp + bm, C = cp + cm;
+  const V oap = od(6), oam = od(7), obp = od(8), obm = od(9), ocp = od(10), ocm = od(11);
+  // space diagonals: even sums (all, xy, xz, yz) and odd sums (x, y, z)
+  auto butterfly = [](V p, V q, V r, V t, V (&o)[4]) {
+    const V pq = p + q, rt = r + t, d = p - q, e = r - t;
+    o[0] = pq + rt;
+    o[1] = pq - rt;
+    o[2] = d + e;
+    o[3] = d - e;
+  };
+  V ce[4], co[4], he[4], ho[4];
+  butterfly(ev(12), ev(13), ev(14), ev(15), ce);
+  butterfly(od(12), od(13), od(14), od(15), co);
+  butterfly(ev(16), ev(17), ev(18), ev(19), he);
+  butterfly(od(16), od(17), od(18), od(19), ho);
+  V d = S(kWeightRest) * h[0];
+  d = fmad(w1, s0 + s1 + s2, d);
+  d = fmad(w2, s3 + s4 + s5, d);
+  d = fmad(wf, A + B + C, d);
+  d = fmad(wc, ce[0], d);
+  d = fmad(wh, he[0], d);
+  m.drho = d;
+  m.rho = S(1) + d;
+  m.inv_rho = S(1) / m.rho;
+  m.j[0] = fmad(whj, ho[0], fmad(wc, co[0], fmad(wf, (oap + oam) + (obp + obm), fmad(w2j, od(3), w1 * od(0)))));
+  m.j[1] = fmad(whj, ho[1], fmad(wc, co[1], fmad(wf, (oap - oam) + (ocp + ocm), fmad(w2j, od(4), w1 * od(1)))));
+  m.j[2] = fmad(whj, ho[2], fmad(wc, co[2], fmad(wf, (obp - obm) + (ocp - ocm), fmad(w2j, od(5), w1 * od(2)))));
+  const V diag = fmad(whp, he[0], wc * ce[0]);
+  m.dP[0] = fmad(w1, s0, fmad(w2p, s3, fmad(wf, A + B, diag)));
+  m.dP[1] = fmad(w1, s1, fmad(w2p, s4, fmad(wf, A + C, diag)));
+  m.dP[2] = fmad(w1, s2, fmad(w2p, s5, fmad(wf, B + C, diag)));
+  m.dP[3] = fmad(whp, he[1], fmad(wc, ce[1], wf * (ap - am)));
+  m.dP[4] = fmad(whp, he[2], fmad(wc, ce[2], wf * (bp - bm)));
+  m.dP[5] = fmad(whp, he[3], fmad(wc, ce[3], wf * (cp - cm)));
+}
+
+// Storage whose one-point kernels use the factored sums and targets.
+template <typename Store>
+constexpr bool kShells = sizeof(Store) > 2;
+
 // f-level moments from g (Sec. 5, g/f relations) and the stored auxiliary
 // rotational energy e (deviation) -- or, in paper mode, the stored theta_R:
 // then theta_T(f) = (theta_T(g) + a theta_R)/(1 + a) inverts the printed
@@ -170,7 +230,7 @@ __device__ __forceinline__ void raw_moments(const V (&h)[kQ], Mom<V>& m) {
 //   D = (theta_T(g) - Rt)/(1 + dt/(2 tau1)) = theta_T(f) - theta_R
 //   theta_T(f) = theta + delta D/(3 + delta),  theta_R = theta - 3 D/(3 + delta)
 //   sigma(f) = (P - jj/rho - rho theta_T(g) I)/(1 + dt/(2 tau*) - b dt/(2 tau))
-template <typename Real, bool kPaper = false, typename V>
+template <typename Real, bool kPaper = false, bool kInv = false, typename V>
 __device__ __forceinline__ void recover(Mom<V>& m, V e, const StepConst<Real>& K) {
   using S = scalar_t<V>;
   const S t0 = K.theta0;
@@ -183,7 +243,11 @@ __device__ __forceinline__ void recover(Mom<V>& m, V e, const StepConst<Real>& K
     m.dT = fmad(K.pa, m.dR, m.dTg) * K.inv_1pa;
     m.dth = fmad(K.delta, m.dR, S(3) * m.dT) * K.inv_3pd;
   } else {
-    const V dRt = (S(2) * e - K.delta * t0 * m.drho) * m.inv_rho / K.delta;
+    V dRt = (S(2) * e - K.delta * t0 * m.drho) * m.inv_rho;
+    if constexpr (kInv)  // a product where the last bit is free
+      dRt = dRt * K.inv_delta;
+    else
+      dRt = dRt / K.delta;
     m.dth = fmad(K.delta, dRt, S(3) * m.dTg) * K.inv_3pd;
     const V D = (m.dTg - dRt) * K.inv_d;
     m.dT = fmad(K.delta * K.inv_3pd, D, m.dth);
@@ -294,6 +358,61 @@ __device__ __forceinline__ V herm_odd(const Herm<V>& H) {
   if constexpr (VY * VZ != 0) r = fmad(S(cz * cz * cy), H.ozzy, fmad(S(cy * cy * cz), H.oyyz, r));
   if constexpr (VX * VY * VZ != 0) r = fmad(S(cx * cy * cz), H.oxyz, r);
   return r;
+}
+
+// herm_even and herm_odd of all pairs, shell by shell: sums shared between the
+// axis, face and space diagonals, and butterflies over the sign patterns (160
+// operations instead of 224 for the 20 pairs). emit(k, even, odd).
+template <typename V, typename Emit>
+__device__ __forceinline__ void herm_shells(const Herm<V>& H, Emit&& emit) {
+  using S = scalar_t<V>;
+  const V ex = H.e0 + H.exx, ey = H.e0 + H.eyy, ez = H.e0 + H.ezz;
+  const V ox = H.ox + H.oxxx, oy = H.oy + H.oyyy, oz = H.oz + H.ozzz;
+  emit(0, ex, ox);
+  emit(1, ey, oy);
+  emit(2, ez, oz);
+  emit(3, fmad(S(4), H.exx, H.e0), fmad(S(8), H.oxxx, S(2) * H.ox));
+  emit(4, fmad(S(4), H.eyy, H.e0), fmad(S(8), H.oyyy, S(2) * H.oy));
+  emit(5, fmad(S(4), H.ezz, H.e0), fmad(S(8), H.ozzz, S(2) * H.oz));
+  const V xy = ex + H.eyy, xz = ex + H.ezz, yz = ey + H.ezz;
+  const V xa = ox + H.oyyx, ya = oy + H.oxxy;  // plane xy
+  const V xb = ox + H.ozzx, zb = oz + H.oxxz;  // plane xz
+  const V yc = oy + H.ozzy, zc = oz + H.oyyz;  // plane yz
+  emit(6, xy + H.exy, xa + ya);
+  emit(7, xy - H.exy, xa - ya);
+  emit(8, xz + H.exz, xb + zb);
+  emit(9, xz - H.exz, xb - zb);
+  emit(10, yz + H.eyz, yc + zc);
+  emit(11, yz - H.eyz, yc - zc);
+  const V n1 = H.exz + H.eyz, n2 = H.exz - H.eyz;
+  {
+    const V b = xy + H.ezz, m1 = b + H.exy, m2 = b - H.exy;
+    const V X = xa + H.ozzx, Y = ya + H.ozzy, Z = zb + H.oyyz;
+    const V a = X + Y, c = X - Y, f = Z + H.oxyz, g = Z - H.oxyz;
+    emit(12, m1 + n1, a + f);
+    emit(13, m1 - n1, a - f);
+    emit(14, m2 + n2, c + g);
+    emit(15, m2 - n2, c - g);
+    // half velocities: second-order terms times 1/4, third-order times 1/8
+    // (X holds the first-order term once: 1/8 + 3/8 = 1/2)
+    const V hb = fmad(S(0.25), H.exx + H.eyy + H.ezz, H.e0);
+    const V h1 = fmad(S(0.25), H.exy, hb), h2 = fmad(S(-0.25), H.exy, hb);
+    const V hX = fmad(S(0.125), X, S(0.375) * H.ox), hY = fmad(S(0.125), Y, S(0.375) * H.oy);
+    const V hZ = fmad(S(0.125), Z, S(0.375) * H.oz);
+    const V ha = hX + hY, hc = hX - hY, hf = fmad(S(0.125), H.oxyz, hZ), hg = fmad(S(-0.125), H.oxyz, hZ);
+    emit(16, fmad(S(0.25), n1, h1), ha + hf);
+    emit(17, fmad(S(-0.25), n1, h1), ha - hf);
+    emit(18, fmad(S(0.25), n2, h2), hc + hg);
+    emit(19, fmad(S(-0.25), n2, h2), hc - hg);
+  }
+}
+
+// H times the scalar c.
+template <typename V>
+__device__ __forceinline__ void herm_scale(Herm<V>& H, scalar_t<V> c) {
+  V* v = reinterpret_cast<V*>(&H);
+#pragma unroll
+  for (int i = 0; i < (int)(sizeof(Herm<V>) / sizeof(V)); ++i) v[i] = v[i] * c;
 }
 
 // Hermite coefficients of f^mix = tau*(f^ES/tau + f^Eq/tau1) (Sec. 5): both

@@ -821,11 +821,14 @@ __global__ void __launch_bounds__(128)
   Real h[kQ];
   gather<Store, Real, kPull, kBC>(pin, ghost, K, P, h, wcol);
   Mom<Real> m;
-  raw_moments(h, m);
-  if (K.paper)
-    recover<Real, true>(m, e_in[p], K);
+  if constexpr (kShells<Store>)
+    raw_moments_shells(h, m);
   else
-    recover<Real, false>(m, e_in[p], K);
+    raw_moments(h, m);
+  if (K.paper)
+    recover<Real, true, kShells<Store>>(m, e_in[p], K);
+  else
+    recover<Real, false, kShells<Store>>(m, e_in[p], K);
   if (rho_o) rho_o[p] = 1.0 + (double)m.drho;
   if (u_o) {
     u_o[p] = (double)(m.j[0] * m.inv_rho);

@@ -41,6 +41,7 @@ static StepConst<Real> make_step_const(const rpk_relax& r, int nsub, int nx, int
   K.exc = Real(r.dt * r.delta / (2.0 * r.tau1));
   K.kapc = Real(r.k_r * 5.0 * r.tau / (2.0 * B));
   K.E0 = Real(0.5 * r.delta * kTheta0);
+  K.inv_delta = Real(1.0 / r.delta);
   K.dt = Real(r.dt);
   K.hsub = Real(r.dt / std::max(1, nsub));
   const double X = 3.0 * r.dt / (2.0 * r.tau1 * (3.0 + r.delta));
