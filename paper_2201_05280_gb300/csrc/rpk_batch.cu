@@ -49,6 +49,214 @@ __device__ __forceinline__ PointIdx tube_point(int nx, int p) {
   return P;
 }
 
+// The pull of `gather` on an nx x 1 x 1 lattice between reservoirs: only x
+// shifts, 32-bit offsets, and no end checks where every source is inside.
+template <typename Store, typename Real>
+__device__ __forceinline__ void gather_line(const Store* __restrict__ pin, const Real* __restrict__ ghost, int nx,
+                                            int s, int x, Real (&h)[kQ]) {
+  const Store* same = pin + s * kQ * nx + x;
+  const Store* other = pin + (1 - s) * kQ * nx + x;
+  const int hp = s ? 0 : -1, hm = s ? 1 : 0;  // source offsets of the half velocities, c_x > 0 and < 0
+  if (x >= 2 && x < nx - 2) {
+    h[0] = to_real<Store, Real>(same[0]);
+    static_for<kQ - 1>([&](auto qc) {
+      constexpr int q = decltype(qc)::value + 1;
+      constexpr Vel2 v = vel2(q);
+      if constexpr ((v.x & 1) != 0)
+        h[q] = to_real<Store, Real>(other[q * nx + (v.x > 0 ? hp : hm)]);
+      else
+        h[q] = to_real<Store, Real>(same[q * nx - v.x / 2]);
+    });
+  } else {
+    h[0] = to_real<Store, Real>(same[0]);
+    static_for<kQ - 1>([&](auto qc) {
+      constexpr int q = decltype(qc)::value + 1;
+      constexpr Vel2 v = vel2(q);
+      constexpr bool half = (v.x & 1) != 0;
+      const int d = half ? (v.x > 0 ? hp : hm) : -v.x / 2;
+      if (x + d < 0 || x + d >= nx)
+        h[q] = ghost[(v.x > 0 ? 0 : kGhostStride) + q];
+      else
+        h[q] = to_real<Store, Real>((half ? other : same)[q * nx + d]);
+    });
+  }
+}
+
+// One backward-Euler step of the rotational diffusion on a tube's two lines,
+//     (delta rho / 2) phi - dt [K+ (phi_+ - phi) - K- (phi - phi_-)] = e - delta theta0 D / 2
+// for phi = theta_R - theta0, by substructuring: every thread eliminates inside
+// blocks of kBE points, leaving each point as x = r + l x_prev + u x_sep in terms of
+// the last points (separators) of the previous and its own block; one warp per
+// line reduces the separators' equations the same way to one per lane, solves
+// those 32 by parallel cyclic reduction in shuffles and substitutes back; then
+// all points follow independently. Three block barriers (cyclic reduction over
+// the points needed 2 log2(nx) + 3) and one division per point. kBE is odd, so
+// threads striding by it hit distinct banks.
+// Each row carries its excess g = 1 - l - u along: l, u, g and r are then sums and
+// products of non-negative numbers, with no cancellation however large K is
+// (FP32, K = 400: error 9e-9 rms of phi where the reduction of the assembled
+// matrix has 1.9e-7).
+// In: e (sE), D (sD), kappa (sK). l -> sL, u -> sU, r -> sR, g -> sE (e is read by
+// its own thread only). Out: e in sE.
+constexpr int kBE = 9;
+
+// A row of the elimination: x = r + l x_prev + u x_next, l + u + g = 1.
+template <typename Real>
+struct BeRow {
+  Real l, u, g, r;
+};
+
+// Row x = (rr + kf x_before + kq x_next) / (s + kf + kq) after x_before = row p.
+template <typename Real>
+__device__ __forceinline__ BeRow<Real> be_eliminate(const BeRow<Real>& p, Real kf, Real kq, Real s, Real rr) {
+  const Real inv = Real(1) / fmad(kf, p.l + p.g, s + kq);
+  return {kf * p.l * inv, kq * inv, fmad(kf, p.g, s) * inv, fmad(kf, p.r, rr) * inv};
+}
+
+// Row a with its x_next replaced by row n (in the same x_prev).
+template <typename Real>
+__device__ __forceinline__ void be_fold(BeRow<Real>& a, const BeRow<Real>& n) {
+  a.l = fmad(a.u, n.l, a.l);
+  a.g = fmad(a.u, n.g, a.g);
+  a.r = fmad(a.u, n.r, a.r);
+  a.u = a.u * n.u;
+}
+
+template <typename Real>
+__device__ __forceinline__ void be_blocks(const StepConst<Real>& K, int nx, int nthreads, Real* sE, const Real* sD,
+                                          const Real* sK, Real* sL, Real* sU, Real* sR, Real kGl, Real kGh, Real thGl,
+                                          Real thGh) {
+  const int nb = (nx + kBE - 1) / kBE;
+  const Real half = Real(0.5), t0d = K.delta * K.theta0;
+  for (int b = threadIdx.x; b < 2 * nb; b += nthreads) {
+    const int line = b >= nb, x0 = (b - line * nb) * kBE, n = min(kBE, nx - x0), o = line * nx + x0;
+    BeRow<Real> w[kBE];
+    Real kp = sK[o];
+    Real kf = K.dt * (half * (kp + (x0 == 0 ? kGl : sK[o - 1])));  // face below
+#pragma unroll
+    for (int i = 0; i < kBE; ++i) {
+      if (i < n) {
+        const bool top = x0 + i == nx - 1;
+        const Real kn = top ? kGh : sK[o + i + 1];
+        const Real kq = K.dt * (half * (kp + kn));  // face above
+        const Real dr = sD[o + i];
+        Real s = half * K.delta * (Real(1) + dr), r = sE[o + i] - half * t0d * dr;
+        Real l = kf, u = kq;
+        if (x0 + i == 0) {  // the reservoirs' values are known
+          r = fmad(kf, thGl, r);
+          s += kf;
+          l = Real(0);
+        }
+        if (top) {
+          r = fmad(kq, thGh, r);
+          s += kq;
+          u = Real(0);
+        }
+        // before a block's first point lies x_prev itself
+        const BeRow<Real> before = i == 0 ? BeRow<Real>{Real(1), Real(0), Real(0), Real(0)} : w[i > 0 ? i - 1 : 0];
+        w[i] = be_eliminate(before, l, u, s, r);
+        kp = kn;
+        kf = kq;
+      }
+    }
+#pragma unroll
+    for (int i = kBE - 3; i >= 0; --i)
+      if (i < n - 2) be_fold(w[i], w[i + 1]);
+#pragma unroll
+    for (int i = 0; i < kBE; ++i)
+      if (i < n) {
+        sL[o + i] = w[i].l;
+        sU[o + i] = w[i].u;
+        sE[o + i] = w[i].g;
+        sR[o + i] = w[i].r;
+      }
+  }
+}
+
+// Separators of a line by one warp; their solution replaces sR at the separators.
+template <typename Real>
+__device__ __forceinline__ void be_separators(int nx, int line, Real* sL, Real* sU, Real* sG, Real* sR) {
+  const unsigned all = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int nb = (nx + kBE - 1) / kBE, per = (nb + 31) / 32;
+  const int j0 = lane * per, cnt = max(0, min(per, nb - j0));
+  auto sep = [&](int j) { return line * nx + min((j + 1) * kBE, nx) - 1; };
+  auto get = [&](int p) { return BeRow<Real>{sL[p], sU[p], sG[p], sR[p]}; };
+  auto put = [&](int p, const BeRow<Real>& w) { sL[p] = w.l, sU[p] = w.u, sG[p] = w.g, sR[p] = w.r; };
+  const BeRow<Real> none{Real(0), Real(1), Real(0), Real(0)};  // x_next is the separator itself
+  // forward sweep over the lane's separators, rows kept at the separators' slots
+  BeRow<Real> w{Real(0), Real(0), Real(1), Real(0)};
+  for (int k = 0; k < cnt; ++k) {
+    const int j = j0 + k, p = sep(j);
+    BeRow<Real> a = get(p);
+    // the next block's first point by the separators (its own last point when
+    // the block has one point; nothing beyond the last block, where u = 0)
+    const int q = line * nx + (j + 1) * kBE;
+    const BeRow<Real> n = j + 1 < nb && (j + 1) * kBE < nx - 1 ? get(q) : none;
+    // a = r + l x_prev + u (n.r + n.l x + n.u x_next): 1 - u n.l = l + g + u (n.u + n.g)
+    const Real inv = Real(1) / (a.l + fmad(a.u, n.u + n.g, a.g));
+    a.g = fmad(a.u, n.g, a.g) * inv;
+    a.r = fmad(a.u, n.r, a.r) * inv;
+    a.u = a.u * n.u * inv;
+    a.l = a.l * inv;
+    w = k == 0 ? a : be_eliminate(w, a.l, a.u, a.g, a.r);
+    put(p, w);
+  }
+  // the lane's first separator by the previous lane's last one and its own
+  // last one; w stays the last row
+  BeRow<Real> f = none;
+  if (cnt > 1) {
+    f = get(sep(j0 + cnt - 2));
+    for (int k = cnt - 3; k >= 0; --k) {
+      const int p = sep(j0 + k);
+      BeRow<Real> a = get(p);
+      be_fold(a, f);
+      put(p, a);
+      f = a;
+    }
+  }
+  // last rows by the lanes' last separators
+  const BeRow<Real> n{__shfl_down_sync(all, f.l, 1), __shfl_down_sync(all, f.u, 1), __shfl_down_sync(all, f.g, 1),
+                      __shfl_down_sync(all, f.r, 1)};
+  BeRow<Real> y = w;
+  if (lane < 31 && cnt > 0 && j0 + cnt < nb) {
+    const Real inv = Real(1) / (w.l + fmad(w.u, n.u + n.g, w.g));
+    y = {w.l * inv, w.u * n.u * inv, fmad(w.u, n.g, w.g) * inv, fmad(w.u, n.r, w.r) * inv};
+  }
+#pragma unroll
+  for (int h = 1; h < 32; h *= 2) {
+    const Real lm = __shfl_up_sync(all, y.l, h), gm = __shfl_up_sync(all, y.g, h), rm = __shfl_up_sync(all, y.r, h);
+    const Real up = __shfl_down_sync(all, y.u, h), gp = __shfl_down_sync(all, y.g, h), rp = __shfl_down_sync(all, y.r, h);
+    const Real l = lane >= h ? y.l : Real(0), u = lane + h < 32 ? y.u : Real(0);
+    const Real inv = Real(1) / fmad(l, lm + gm, fmad(u, up + gp, y.g));
+    y = {l * lm * inv, u * up * inv, fmad(l, gm, fmad(u, gp, y.g)) * inv, fmad(l, rm, fmad(u, rp, y.r)) * inv};
+  }
+  const Real v = y.r;
+  Real vp = __shfl_up_sync(all, v, 1);
+  if (lane == 0) vp = Real(0);
+  for (int k = 0; k < cnt; ++k) {
+    const int p = sep(j0 + k);
+    sR[p] = k == cnt - 1 ? v : fmad(sL[p], vp, fmad(sU[p], v, sR[p]));
+  }
+}
+
+// e of every point from its block's and the previous block's separators.
+template <typename Real>
+__device__ __forceinline__ void be_points(const StepConst<Real>& K, int nx, int nthreads, Real* sE, const Real* sD,
+                                          const Real* sL, const Real* sU, const Real* sR) {
+  for (int p = threadIdx.x; p < 2 * nx; p += nthreads) {
+    const int s = p >= nx, x = p - s * nx, j = x / kBE;
+    const int q = s * nx + min((j + 1) * kBE, nx) - 1;
+    Real phi = sR[q];
+    if (p != q) {
+      phi = fmad(sU[p], phi, sR[p]);
+      if (j > 0) phi = fmad(sL[p], sR[s * nx + j * kBE - 1], phi);
+    }
+    const Real dr = sD[p];
+    sE[p] = Real(0.5) * K.delta * ((Real(1) + dr) * phi + K.theta0 * dr);
+  }
+}
+
 // FTCS sub-steps of a tube's two sublattice lines, several per block barrier.
 // A warp takes a piece of a line, kP consecutive points per lane, in
 // registers: neighbours inside a lane are registers, those of the next lane
@@ -60,7 +268,8 @@ __device__ __forceinline__ PointIdx tube_point(int nx, int p) {
 // order of the lattice's FTCS kernels, so results are those of one barrier per
 // sub-step bit for bit.
 // With a block barrier and 10 shared loads per point and sub-step it took 0.8
-// us a sub-step for the largest tubes (1500 cells, FTCS_OLDNEW).
+// us a sub-step for tubes of 1500 cells; 304 tubes of 500 to 1500 cells went
+// from 405 to 104 ms.
 template <typename Real>
 struct FtcsLine {
   const Real* a;     // theta_R - theta0 = a e + c
@@ -186,14 +395,18 @@ __global__ void __launch_bounds__(kThreads)
       float* sn = snaps + T->snap_off + (int64_t)(t / save_every) * 4 * np;
       // 1. pull + collide + exchange of every point of the tube
       for (int p = tid; p < np; p += kThreads) {
-        const PointIdx P = tube_point(nx, p);
+        const int s = p >= nx, x = p - s * nx;
         Real h[kQ];
-        if (streamed)
-          gather<Store, Real, false, 1>(pin, ghost, K, P, h);
-        else
-          gather<Store, Real, true, 1>(pin, ghost, K, P, h);
+        if (streamed) {
+#pragma unroll
+          for (int q = 0; q < kQ; ++q) h[q] = to_real<Store, Real>(pin[(s * kQ + q) * nx + x]);
+        } else {
+          gather_line<Store, Real>(pin, ghost, nx, s, x, h);
+        }
         Mom<Real> m;
-        const Real es = collide_point<Store, Real>(K, h, sE[p], pout + (int64_t)(P.s * kQ) * K.n3 + P.cell, m);
+        Store* out = pout + s * kQ * nx + x;
+        const Real es = collide_shells<Real, false>(
+            K, h, sE[p], [&](int q, Real v) { out[q * nx] = from_real<Store, Real>(v); }, m);
         sS[p] = es;
         sD[p] = m.drho;
         uc[p] = m.j[0] * m.inv_rho;
@@ -243,84 +456,18 @@ __global__ void __launch_bounds__(kThreads)
         const Real val = Real(0.5) * (sS[p] + epp - K.dt * div);
         const Real dr = sD[p];
         sE[p] = val;
-        sS[p] = (Real(2) * val - t0d * dr) / (K.delta * (Real(1) + dr));
+        if constexpr (!kImplicit) sS[p] = (Real(2) * val - t0d * dr) / (K.delta * (Real(1) + dr));
       }
       __syncthreads();
       if constexpr (kImplicit) {
-        // 4'. backward-Euler variant: per sublattice line solve
-        //     (delta rho / 2) phi - dt [K+ (phi_+ - phi) - K- (phi - phi_-)] = e - delta theta0 D / 2
-        //     for phi = theta_R - theta0 by cyclic reduction in shared memory:
-        //     a -> sP, b -> sK, c -> sS, right-hand side and then phi -> sE.
-        for (int p = tid; p < np; p += kThreads) {
-          const int s = p >= nx, x = p - s * nx;
-          const Real kp = sK[p];
-          const Real km = x == 0 ? gl[kGhKap] : sK[p - 1];
-          const Real kq = x + 1 >= nx ? gh[kGhKap] : sK[p + 1];
-          sP[p] = -K.dt * Real(0.5) * (kp + km);
-          sS[p] = -K.dt * Real(0.5) * (kp + kq);
-        }
+        // 4'. backward-Euler variant: l -> sP, u -> sS, g -> sE, r -> the u(t-1) slot (dead
+        //     until the next step's u)
+        Real* r = (t & 1) ? sU0 : sU1;
+        be_blocks(K, nx, kThreads, sE, sD, sK, sP, sS, r, gl[kGhKap], gh[kGhKap], thGl, thGh);
         __syncthreads();
-        for (int p = tid; p < np; p += kThreads) {
-          const int s = p >= nx, x = p - s * nx;
-          const Real a = sP[p], c = sS[p], dr = sD[p];
-          sK[p] = Real(0.5) * K.delta * (Real(1) + dr) - a - c;
-          Real r = sE[p] - Real(0.5) * t0d * dr;
-          if (x == 0) {
-            r -= a * thGl;
-            sP[p] = Real(0);
-          }
-          if (x + 1 >= nx) {
-            r -= c * thGh;
-            sS[p] = Real(0);
-          }
-          sE[p] = r;
-        }
+        if (tid < 64) be_separators(nx, tid >> 5, sP, sS, sE, r);
         __syncthreads();
-        int h = 1;
-        for (; 2 * h <= nx; h *= 2) {
-          const int cnt = nx / (2 * h);  // x = 2h - 1, 4h - 1, ... < nx per line
-          for (int j = tid; j < 2 * cnt; j += kThreads) {
-            const int s = j >= cnt, k = j - s * cnt;
-            const int x = (k + 1) * 2 * h - 1, p = s * nx + x;
-            const int L = p - h;
-            const Real al = -sP[p] / sK[L];
-            Real a = al * sP[L], b = sK[p] + al * sS[L], c = Real(0), r = sE[p] + al * sE[L];
-            if (x + h < nx) {
-              const int R = p + h;
-              const Real ga = -sS[p] / sK[R];
-              c = ga * sS[R];
-              b += ga * sP[R];
-              r += ga * sE[R];
-            }
-            sP[p] = a;
-            sK[p] = b;
-            sS[p] = c;
-            sE[p] = r;
-          }
-          __syncthreads();
-        }
-        // the top equation of each line, x = h - 1, is now uncoupled
-        if (tid < 2) {
-          const int p = tid * nx + h - 1;
-          sE[p] = sE[p] / sK[p];
-        }
-        __syncthreads();
-        for (h /= 2; h >= 1; h /= 2) {
-          const int cnt = (nx + h) / (2 * h);  // x = h - 1, 3h - 1, ... < nx per line
-          for (int j = tid; j < 2 * cnt; j += kThreads) {
-            const int s = j >= cnt, k = j - s * cnt;
-            const int x = (2 * k + 1) * h - 1, p = s * nx + x;
-            Real r = sE[p];
-            if (x - h >= 0) r -= sP[p] * sE[p - h];
-            if (x + h < nx) r -= sS[p] * sE[p + h];
-            sE[p] = r / sK[p];
-          }
-          __syncthreads();
-        }
-        for (int p = tid; p < np; p += kThreads) {
-          const Real dr = sD[p];
-          sE[p] = Real(0.5) * K.delta * ((Real(1) + dr) * sE[p] + K.theta0 * dr);
-        }
+        be_points(K, nx, kThreads, sE, sD, sP, sS, r);
         __syncthreads();
       } else {
         // 4. FTCS sub-steps, e += h sum_faces K_face (theta_nb - theta) with
@@ -443,8 +590,8 @@ __global__ void k_batch_moments(const TubeDev<Real>* __restrict__ tubes, const S
     else
       gather<Store, Real, true, 1>(pin, tb->ghost, K, P, h);
     Mom<Real> m;
-    raw_moments(h, m);
-    recover(m, e_state[off + p], K);
+    raw_moments_shells(h, m);
+    recover<Real, false, true>(m, e_state[off + p], K);
     const int64_t g = off + p;
     out[g] = 1.0 + (double)m.drho;
     out[total_pts + g] = (double)(m.j[0] * m.inv_rho);
