@@ -545,6 +545,190 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv_tc(TcArgs P) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_COLS) : "memory");
 }
 
+// ---------------------------------------------------------------------------
+// Weight and bias gradients of all residual-block convolutions in one launch
+// (tcgen05; Co = Ci = 128, 5 taps, ReLU inputs):
+//   dW[o][t][i] += sum_q dY[q][o] relu(X[q + t - 2][i]),  db[o] += sum_q dY[q][o].
+// The reduction runs over positions, so both operands are MN-major: a tile of
+// 128 positions is staged as in k_conv_tc (8-channel chunks, rows 16 bytes
+// apart), which read with channels as M or N and rows as K is the no-swizzle
+// MN-major layout (SBO = chunk stride, LBO = 128 bytes between groups of 8
+// rows), and the tap shift is again a start-address offset of 16 bytes a row.
+// A CTA owns (layer, half of the input channels, share of the tiles): M 128, N
+// 64 per tap, 5 x 64 TMEM columns. All 512 threads stage tile i (loads, ReLU,
+// BF16, stores) while the 40 MMAs of tile i - 1 run from the other buffer; the
+// accumulators are added to dW once per CTA by 16-byte atomics, and the bias
+// gradient is the FP32 column sums of dY on their way to shared memory.
+// Bound: reading dY and X (FP32) once per half. One launch after the whole
+// input-gradient chain fills the chip where a layer alone gave 10 x 2 x 29 small
+// tiles re-staged by every block: 12 launches of 99 us (mma.sync) and 12 of
+// 22.5 us (bias) for 32 crops of 1024 points became one of 41 us.
+constexpr int DW_N = 64;                                    // input channels per CTA
+constexpr uint32_t DW_A_STRIDE = (TC_N + 1) * 16;           // dY: bytes between 8-channel chunks
+constexpr uint32_t DW_B_STRIDE = (TC_ROWS + 1) * 16;        // X
+constexpr uint32_t DW_A_BYTES = (TC_M / 8) * DW_A_STRIDE;   // 33024
+constexpr uint32_t DW_B_BYTES = (DW_N / 8) * DW_B_STRIDE;   // 17024
+constexpr uint32_t DW_BUF = DW_A_BYTES + DW_B_BYTES;
+constexpr uint32_t DW_BAR_OFF = 2 * DW_BUF;
+constexpr uint32_t DW_SMEM = DW_BAR_OFF + 64;
+constexpr int DW_COLS = 512;                                // 5 x 64 accumulator columns, a power of two
+constexpr uint32_t DW_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
+                              ((uint32_t)(DW_N >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
+
+struct DwTcArgs {
+  const float* dY;    // layer l's output gradient at dY + l * stride
+  const float* h;     // even layers' inputs: block b's at h + b * stride
+  const float* z;     // odd layers' inputs
+  float* g;           // layer l's weight gradient at g + l * gstride, then its bias gradient
+  int64_t stride, gstride;
+  int ntiles, tiles_per_seq, seq_len, splits;
+  unsigned* error;
+};
+
+__global__ void __launch_bounds__(TC_THREADS, 1) k_dw_tc(DwTcArgs P) {
+  extern __shared__ __align__(1024) unsigned char tc_smem[];
+  uint64_t* bars = reinterpret_cast<uint64_t*>(tc_smem + DW_BAR_OFF);  // MMAs of buffer 0, 1 done
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tc_smem + DW_BAR_OFF + 32);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int split = blockIdx.x % P.splits, part = blockIdx.x / P.splits;
+  const int half = part & 1, layer = part >> 1;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(DW_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == 0) {
+    for (int b = 0; b < 2; ++b)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bars + b)), "r"(1) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot, bar0 = smem_u32(bars), base = smem_u32(tc_smem);
+  const float* dY = P.dY + layer * P.stride;
+  const float* X = ((layer & 1) ? P.z : P.h) + (layer >> 1) * P.stride + half * DW_N;
+  constexpr int kA = TC_N * (TC_M / 8) / TC_THREADS;                              // 4 dY elements per thread
+  constexpr int kB = (TC_ROWS * (DW_N / 8) + TC_THREADS - 1) / TC_THREADS;        // 3 X elements
+  float bsum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  bool ok = true;
+  int n = 0;  // tiles issued
+  for (int tile = split; tile < P.ntiles; tile += P.splits, ++n) {
+    const int sq = tile / P.tiles_per_seq, part0 = (tile - sq * P.tiles_per_seq) * TC_N;
+    const int lo = sq * P.seq_len, q0 = lo + part0, cnt = min(TC_N, P.seq_len - part0);
+    float4 a[kA][2], b[kB][2];
+#pragma unroll
+    for (int u = 0; u < kA; ++u) {
+      const int e = tid + u * TC_THREADS, r = e / (TC_M / 8), c = e % (TC_M / 8);
+      a[u][0] = a[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r < cnt) {
+        const float4* src = reinterpret_cast<const float4*>(dY + (int64_t)(q0 + r) * TC_M + 8 * c);
+        a[u][0] = src[0];
+        a[u][1] = src[1];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kB; ++u) {
+      const int e = tid + u * TC_THREADS, r = e / (DW_N / 8), c = e % (DW_N / 8);
+      const int q = q0 - 2 + r;
+      b[u][0] = b[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r < TC_ROWS && q >= lo && q < lo + P.seq_len) {
+        const float4* src = reinterpret_cast<const float4*>(X + (int64_t)q * TC_KC + 8 * c);
+        b[u][0] = src[0];
+        b[u][1] = src[1];
+      }
+    }
+    const int buf = n & 1;
+    if (n >= 2) ok = mbar_wait(bar0 + 8 * buf, ((n >> 1) - 1) & 1);
+    ok = __syncthreads_and(ok);
+    if (!ok) break;
+    unsigned char* sA = tc_smem + buf * DW_BUF;
+    unsigned char* sB = sA + DW_A_BYTES;
+#pragma unroll
+    for (int u = 0; u < kA; ++u) {
+      const int e = tid + u * TC_THREADS, r = e / (TC_M / 8), c = e % (TC_M / 8);
+      const float4 f = a[u][0], g = a[u][1];
+      bsum[0] += f.x, bsum[1] += f.y, bsum[2] += f.z, bsum[3] += f.w;
+      bsum[4] += g.x, bsum[5] += g.y, bsum[6] += g.z, bsum[7] += g.w;
+      *reinterpret_cast<uint4*>(sA + c * DW_A_STRIDE + r * 16) =
+          make_uint4(pack_bf16(f.x, f.y), pack_bf16(f.z, f.w), pack_bf16(g.x, g.y), pack_bf16(g.z, g.w));
+    }
+#pragma unroll
+    for (int u = 0; u < kB; ++u) {
+      const int e = tid + u * TC_THREADS, r = e / (DW_N / 8), c = e % (DW_N / 8);
+      if (r >= TC_ROWS) break;
+      const float4 f = b[u][0], g = b[u][1];
+      *reinterpret_cast<uint4*>(sB + c * DW_B_STRIDE + r * 16) =
+          make_uint4(pack_bf16(fmaxf(f.x, 0.f), fmaxf(f.y, 0.f)), pack_bf16(fmaxf(f.z, 0.f), fmaxf(f.w, 0.f)),
+                     pack_bf16(fmaxf(g.x, 0.f), fmaxf(g.y, 0.f)), pack_bf16(fmaxf(g.z, 0.f), fmaxf(g.w, 0.f)));
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t ab = base + buf * DW_BUF, bb = ab + DW_A_BYTES;
+#pragma unroll 1
+      for (int t = 0; t < TC_TAPS; ++t)
+#pragma unroll
+        for (int k = 0; k < TC_N / 16; ++k) {
+          const uint64_t ad = tc_desc(ab + (uint32_t)k * 256, 128, DW_A_STRIDE);
+          const uint64_t bd = tc_desc(bb + (uint32_t)(16 * k + t) * 16, 128, DW_B_STRIDE);
+          const uint32_t accum = (n | k) ? 1u : 0u;
+          asm volatile(
+              "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+              " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + (uint32_t)(t * DW_N)),
+              "l"(ad), "l"(bd), "r"(DW_IDESC), "r"(accum)
+              : "memory");
+        }
+      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar0 + 8 * buf)
+                   : "memory");
+    }
+  }
+  // every MMA has completed: the last tile of each buffer
+  for (int b = 0; b < 2; ++b)
+    if (n > b) ok = mbar_wait(bar0 + 8 * b, (((n - 1 - b) >> 1) & 1)) && ok;
+  ok = __syncthreads_and(ok);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (!ok && tid == 0) atomicOr(P.error, 1u);
+  if (ok && n > 0) {
+    // warps w and w + 4, ..: TMEM lanes 32 (w % 4) ..; 20 pieces of 16 columns over 4 warps
+    const int m = (warp & 3) * 32 + lane;
+    float* dW = P.g + layer * P.gstride + (int64_t)m * TC_K + half * DW_N;
+    for (int piece = warp >> 2; piece < TC_TAPS * (DW_N / 16); piece += TC_THREADS / 128) {
+      uint32_t v[16];
+      tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(piece * 16), v);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      const int t = piece / (DW_N / 16), j = piece % (DW_N / 16) * 16;
+#pragma unroll
+      for (int k = 0; k < 16; k += 4)
+        atomicAdd(reinterpret_cast<float4*>(dW + t * TC_KC + j + k),
+                  make_float4(__uint_as_float(v[k]), __uint_as_float(v[k + 1]), __uint_as_float(v[k + 2]),
+                              __uint_as_float(v[k + 3])));
+    }
+    if (half == 0) {
+      // column sums of dY: threads of equal tid % 16 hold the same 8 channels
+      float* red = reinterpret_cast<float*>(tc_smem);  // [16 warps][128 channels]
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const float v = bsum[k] + __shfl_xor_sync(0xffffffffu, bsum[k], 16);
+        if (lane < 16) red[warp * TC_M + lane * 8 + k] = v;
+      }
+    }
+  }
+  __syncthreads();
+  if (ok && n > 0 && half == 0 && tid < TC_M) {
+    const float* red = reinterpret_cast<const float*>(tc_smem);
+    float v = 0.f;
+    for (int w = 0; w < TC_THREADS / 32; ++w) v += red[w * TC_M + tid];
+    atomicAdd(P.g + layer * P.gstride + (int64_t)TC_M * TC_K + tid, v);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(DW_COLS) : "memory");
+}
+
 struct DwArgs {
   const float* dY;  // [npos][M]
   const float* X;   // [npos][Kc]
@@ -721,7 +905,9 @@ struct rpk_net {
   // activation workspace for up to cap_q coarse positions
   int64_t cap_q = 0;
   float* act = nullptr;   // h_0..h_B (B+1), z0 per block (B): (2B+1) x cap_q x width
-  float* work = nullptr;  // 2 x cap_q x width scratch for gradients
+  // training workspace for up to cap_t coarse positions
+  int64_t cap_t = 0;
+  float* work = nullptr;  // (2B+1) x cap_t x width: slot 0 the lift's, slot l + 1 block layer l's output gradient
   float* headout = nullptr;
   float* dybuf = nullptr;
   double* loss = nullptr;
@@ -750,21 +936,31 @@ rpk_status net_alloc(void** p, size_t bytes) {
 rpk_status ensure_workspace(rpk_net* N, int64_t nq) {
   if (nq <= N->cap_q) return RPK_OK;
   cudaFree(N->act);
-  cudaFree(N->work);
-  cudaFree(N->headout);
-  cudaFree(N->dybuf);
   cudaFree(N->qseq);
-  N->act = N->work = N->headout = N->dybuf = nullptr;
+  N->act = nullptr;
   N->qseq = nullptr;
   N->cap_q = 0;
   const size_t W = N->width;
   rpk_status st = net_alloc((void**)&N->act, sizeof(float) * (2 * N->nblocks + 1) * nq * W);
-  if (st == RPK_OK) st = net_alloc((void**)&N->work, sizeof(float) * 2 * nq * W);
-  if (st == RPK_OK) st = net_alloc((void**)&N->headout, sizeof(float) * nq * R * N->cout);
-  if (st == RPK_OK) st = net_alloc((void**)&N->dybuf, sizeof(float) * nq * R * N->cout);
   if (st == RPK_OK) st = net_alloc((void**)&N->qseq, sizeof(int2) * nq);
   if (st != RPK_OK) return st;
   N->cap_q = nq;
+  return RPK_OK;
+}
+
+rpk_status ensure_training(rpk_net* N, int64_t nq) {
+  rpk_status st = ensure_workspace(N, nq);
+  if (st != RPK_OK || nq <= N->cap_t) return st;
+  cudaFree(N->work);
+  cudaFree(N->headout);
+  cudaFree(N->dybuf);
+  N->work = N->headout = N->dybuf = nullptr;
+  N->cap_t = 0;
+  st = net_alloc((void**)&N->work, sizeof(float) * (2 * N->nblocks + 1) * nq * N->width);
+  if (st == RPK_OK) st = net_alloc((void**)&N->headout, sizeof(float) * nq * R * N->cout);
+  if (st == RPK_OK) st = net_alloc((void**)&N->dybuf, sizeof(float) * nq * R * N->cout);
+  if (st != RPK_OK) return st;
+  N->cap_t = nq;
   return RPK_OK;
 }
 
@@ -868,14 +1064,44 @@ __global__ void k_fill_qseq(const int* __restrict__ starts, int2* __restrict__ q
   for (int q = lo + threadIdx.x; q < hi; q += blockDim.x) qseq[q] = make_int2(lo, hi - lo);
 }
 
-// Backward pass from dy (fine layout == coarse layout), gradients into N->g.
+// Gradients of every block convolution's weights and biases from the output
+// gradients in N->work (slot l + 1: block layer l).
+rpk_status block_grads(rpk_net* N, int64_t nq, int Lq) {
+  const int64_t stride = nq * N->width;
+  const int nl = 2 * N->nblocks, W = N->width;
+  if (nl == 0) return RPK_OK;
+  const auto& first = N->layers[1];
+  if (N->tc && (((uintptr_t)(N->g + first.w_off)) & 15) == 0) {
+    DwTcArgs P{N->work + stride, N->act, N->act + (N->nblocks + 1) * stride, N->g + first.w_off, stride,
+               (int64_t)W * TC_K + W, 0, (Lq + TC_N - 1) / TC_N, Lq, 1, N->tc_error};
+    P.ntiles = (int)(nq / Lq) * P.tiles_per_seq;
+    // one CTA per SM: as many shares of the tiles as the SMs hold (layer, half) pairs
+    P.splits = std::max(1, std::min(P.ntiles, N->nsm / (2 * nl)));
+    k_dw_tc<<<2 * nl * P.splits, TC_THREADS, DW_SMEM, N->stream>>>(P);
+    RPK_CUDA(cudaGetLastError());
+    return RPK_OK;
+  }
+  for (int l = 0; l < nl; ++l) {
+    const float* X = N->act + ((l & 1) ? N->nblocks + 1 + l / 2 : l / 2) * stride;
+    const float* dY = N->work + (l + 1) * stride;
+    const auto& L = N->layers[1 + l];
+    rpk_status st = conv_dw(N, dY, W, X, W, K5, 1, N->g + L.w_off, nq, Lq);
+    if (st != RPK_OK) return st;
+    k_bias_grad<<<W, 256, 0, N->stream>>>(dY, (int)nq, W, N->g + L.b_off);
+  }
+  RPK_CUDA(cudaGetLastError());
+  return RPK_OK;
+}
+
+// Backward pass from dy (fine layout == coarse layout), gradients into N->g:
+// the chain of input gradients first (each layer's output gradient kept in its
+// own slot of N->work), then the block layers' weight gradients together.
 rpk_status backward(rpk_net* N, const float* x, const float* dy, int nseq, int L) {
   const int64_t nq = (int64_t)nseq * (L / R);
   const int Lq = L / R;
   const int64_t stride = nq * N->width;
   RPK_CUDA(cudaMemsetAsync(N->g, 0, sizeof(float) * N->nparams, N->stream));
-  float* dh = N->work;           // gradient wrt h (current block output)
-  float* tmp = N->work + stride;  // gradient wrt z0
+  auto slot = [&](int k) { return N->work + k * stride; };
   const int W = N->width;
   const auto& head = N->layers.back();
   const float* hB = N->act + N->nblocks * stride;
@@ -883,28 +1109,24 @@ rpk_status backward(rpk_net* N, const float* x, const float* dy, int nseq, int L
   k_bias_grad<<<R * N->cout, 256, 0, N->stream>>>(dy, (int)nq, R * N->cout, N->g + head.b_off);
   // d relu(h_B) = W_head^T dy, then mask by h_B > 0
   if (st == RPK_OK)
-    st = conv(N, N->wtb + head.wb_off, W, 1, R * N->cout, -1, dy, 0, dh, nullptr, nullptr, hB, nq, Lq);
+    st = conv(N, N->wtb + head.wb_off, W, 1, R * N->cout, -1, dy, 0, slot(2 * N->nblocks), nullptr, nullptr, hB, nq, Lq);
   for (int b = N->nblocks - 1; b >= 0 && st == RPK_OK; --b) {
     const auto& c0 = N->layers[1 + 2 * b];
     const auto& c1 = N->layers[2 + 2 * b];
     const float* hb = N->act + b * stride;
     const float* z0 = N->act + (N->nblocks + 1 + b) * stride;
-    // z1 = conv(relu(z0)); d z1 = dh
-    st = conv_dw(N, dh, W, z0, W, K5, 1, N->g + c1.w_off, nq, Lq);
-    k_bias_grad<<<W, 256, 0, N->stream>>>(dh, (int)nq, W, N->g + c1.b_off);
+    const float* dh = slot(2 * b + 2);  // z1 = conv(relu(z0)); d z1 = dh
+    float* dz = slot(2 * b + 1);        // z0 = conv(relu(h_b)); d z0
+    st = conv(N, N->wtb + c1.wb_off, W, K5, W, -1, dh, 0, dz, nullptr, nullptr, z0, nq, Lq);
+    // d h_b = dh + (W0^T dz) masked by h_b > 0
     if (st == RPK_OK)
-      st = conv(N, N->wtb + c1.wb_off, W, K5, W, -1, dh, 0, tmp, nullptr, nullptr, z0, nq, Lq);
-    // z0 = conv(relu(h_b)); d z0 = tmp
-    if (st == RPK_OK) st = conv_dw(N, tmp, W, hb, W, K5, 1, N->g + c0.w_off, nq, Lq);
-    k_bias_grad<<<W, 256, 0, N->stream>>>(tmp, (int)nq, W, N->g + c0.b_off);
-    // d h_b = dh + (W0^T tmp) masked by h_b > 0   (written in place of dh)
-    if (st == RPK_OK)
-      st = conv(N, N->wtb + c0.wb_off, W, K5, W, -1, tmp, 0, dh, nullptr, dh, hb, nq, Lq);
+      st = conv(N, N->wtb + c0.wb_off, W, K5, W, -1, dz, 0, slot(2 * b), nullptr, dh, hb, nq, Lq);
   }
+  if (st == RPK_OK) st = block_grads(N, nq, Lq);
   if (st != RPK_OK) return st;
   const auto& lift = N->layers[0];
-  st = conv_dw(N, dh, W, x, R * N->cin, 1, 0, N->g + lift.w_off, nq, Lq);
-  k_bias_grad<<<W, 256, 0, N->stream>>>(dh, (int)nq, W, N->g + lift.b_off);
+  st = conv_dw(N, slot(0), W, x, R * N->cin, 1, 0, N->g + lift.w_off, nq, Lq);
+  k_bias_grad<<<W, 256, 0, N->stream>>>(slot(0), (int)nq, W, N->g + lift.b_off);
   RPK_CUDA(cudaGetLastError());
   return st;
 }
@@ -961,7 +1183,8 @@ rpk_status rpk_net_create(int cin, int cout, int width, int nblocks, uint64_t se
     cudaDeviceGetAttribute(&N->nsm, cudaDevAttrMultiProcessorCount, N->device);
     N->tc = width == TC_M &&
             cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM) ==
-                cudaSuccess;
+                cudaSuccess &&
+            cudaFuncSetAttribute(k_dw_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DW_SMEM) == cudaSuccess;
     cudaGetLastError();
   }
   cudaError_t err = cudaSuccess;
@@ -1073,7 +1296,7 @@ rpk_status rpk_net_loss_grad(rpk_net* N, const float* x, const float* target, co
   if (nseq < 1 || len < R || len % R) return rpk::fail(RPK_ERR_ARG, "len must be a positive multiple of 4");
   RPK_CUDA(cudaSetDevice(N->device));
   const int64_t nq = (int64_t)nseq * (len / R);
-  rpk_status st = ensure_workspace(N, nq);
+  rpk_status st = ensure_training(N, nq);
   if (st != RPK_OK) return st;
   float* y = N->headout;
   st = forward(N, x, nq, len / R, nullptr, y);
