@@ -91,8 +91,7 @@ template <typename Store, typename Real, int kBC>
 static rpk_status wall_launch_t(rpk_lattice* L, const StepConst<Real>& K) {
   const int64_t n = ((kBC & kWallY) ? 2 * (int64_t)L->grid.nx * L->grid.nz : 0) +
                     ((kBC & kWallX) ? 2 * (int64_t)L->grid.ny * L->grid.nz : 0);
-  k_wall_rho<Store, Real, kBC><<<(unsigned)((n + 127) / 128), 128, 0, L->stream>>>(
-      K, static_cast<const Store*>(L->pop[L->cur]), static_cast<const Real*>(L->ghost),
+  k_wall_rho<Store, Real, kBC><<<(unsigned)((n + 31) / 32), 32, 0, L->stream>>>(K, static_cast<const Store*>(L->pop[L->cur]), static_cast<const Real*>(L->ghost),
       static_cast<Real*>(L->wrho));
   return check_launch("k_wall_rho");
 }
@@ -119,20 +118,17 @@ static rpk_status collide_launch(rpk_lattice* L, const StepConst<Real>& K) {
         // two x-adjacent points per thread, packed FP32x2 arithmetic
         const PointLaunch at(L, L->n3 / 2);
         if constexpr (std::is_same<Store, __half>::value)
-          k_collide_pair_w<Store, true><<<at.grid, at.block, 0, L->stream>>>(
-              K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
+          k_collide_pair_w<Store, true><<<at.grid, at.block, 0, L->stream>>>(K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
               static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status,
               static_cast<Real*>(L->thbuf));
         else
-          k_collide_pair<Store, true><<<at.grid, at.block, 0, L->stream>>>(
-              K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
+          k_collide_pair<Store, true><<<at.grid, at.block, 0, L->stream>>>(K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
               static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status,
               static_cast<Real*>(L->thbuf));
         return check_launch("k_collide_pair");
       }
     }
-    k_collide<Store, Real, kPull, kBC, true><<<pt.grid, pt.block, 0, L->stream>>>(
-        K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
+    k_collide<Store, Real, kPull, kBC, true><<<pt.grid, pt.block, 0, L->stream>>>(K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
         static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap),
         static_cast<const Real*>(L->ghost), L->status, static_cast<Real*>(L->thbuf), wcol);
     return check_launch("k_collide");
@@ -143,18 +139,15 @@ static rpk_status collide_launch(rpk_lattice* L, const StepConst<Real>& K) {
       const PointLaunch at(L, L->n3 / 2);
       // FP16 storage holds the pair words, not their FP32 values, across the collision
       if constexpr (std::is_same<Store, __half>::value)
-        k_collide_pair_w<Store, false><<<at.grid, at.block, 0, L->stream>>>(
-            K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
+        k_collide_pair_w<Store, false><<<at.grid, at.block, 0, L->stream>>>(K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
             static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status, nullptr);
       else
-        k_collide_pair<Store, false><<<at.grid, at.block, 0, L->stream>>>(
-            K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
+        k_collide_pair<Store, false><<<at.grid, at.block, 0, L->stream>>>(K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
             static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status, nullptr);
       return check_launch("k_collide_pair");
     }
   }
-  k_collide<Store, Real, kPull, kBC, false><<<pt.grid, pt.block, 0, L->stream>>>(
-      K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
+  k_collide<Store, Real, kPull, kBC, false><<<pt.grid, pt.block, 0, L->stream>>>(K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
       static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap),
       static_cast<const Real*>(L->ghost), L->status, nullptr, wcol);
   return check_launch("k_collide");
@@ -190,7 +183,6 @@ static int line_launches(rpk_lattice* L, const StepConst<Real>& K, const Real* e
 
 template <typename Real, int kBC>
 static rpk_status transport_launch(rpk_lattice* L, const StepConst<Real>& K) {
-  const PointLaunch pt(L, L->n3);
   const Real* ucur = static_cast<const Real*>(L->u[L->steps & 1]);
   const Real* uprev = static_cast<const Real*>(L->u[(L->steps + 1) & 1]);
   const Real* gh = static_cast<const Real*>(L->ghost);
@@ -245,29 +237,33 @@ static rpk_status transport_launch(rpk_lattice* L, const StepConst<Real>& K) {
       return check_launch("rotational transport (line)");
     }
   }
-  // predictor, corrector and the first FTCS sub-step; further sub-steps end in e
-  Real* dst = L->nsub == 1 ? e : ea;
+  // predictor and corrector, then the FTCS sub-steps: e in place from the
+  // second on, theta_R between the transport's scratch planes
   bool quads = false;
   if constexpr (kBC == 0 && sizeof(Real) == 4) quads = L->grid.nx % 4 == 0;
+  // periodic FP32 grid, nx a multiple of 4: four x-adjacent points per thread
+  const dim3 qgrid((unsigned)((L->grid.nx / 4 + kTBX - 1) / kTBX),
+                   (unsigned)((L->grid.ny + kTBY - 1) / kTBY), (unsigned)(2 * L->grid.nz));
   if (quads) {
     if constexpr (kBC == 0 && sizeof(Real) == 4) {
-      // periodic FP32 grid, nx a multiple of 4: four x-adjacent points per thread
-      const dim3 qgrid((unsigned)((L->grid.nx / 4 + kTBX - 1) / kTBX),
-                       (unsigned)((L->grid.ny + kTBY - 1) / kTBY), (unsigned)(2 * L->grid.nz));
       k_mac_pred4<<<qgrid, tb, 0, L->stream>>>(K, es, ucur, uprev, ea, v);
       k_mac_corr4<<<qgrid, tb, 0, L->stream>>>(K, es, ea, v, drho, eb, th);
-      k_ftcs_first4<<<qgrid, tb, 0, L->stream>>>(K, eb, th, kap, dst);
     }
   } else {
     k_mac_pred<Real, kBC><<<tgrid, tb, 0, L->stream>>>(K, es, ucur, uprev, ea, v, gh);
     k_mac_corr<Real, kBC><<<tgrid, tb, 0, L->stream>>>(K, es, ea, v, drho, eb, th, gh);
-    k_ftcs_first<Real, kBC><<<tgrid, tb, 0, L->stream>>>(K, eb, th, kap, dst, gh);
   }
-  Real* src = dst;
-  for (int k = 1; k < L->nsub; ++k) {
-    dst = (k == L->nsub - 1) ? e : (src == ea ? eb : ea);
-    k_ftcs<Real, kBC><<<pt.grid, pt.block, 0, L->stream>>>(K, src, drho, kap, dst, gh);
-    src = dst;
+  const Real* src = eb;
+  for (int k = 0; k < L->nsub; ++k) {
+    Real* th_next = k == L->nsub - 1 ? nullptr : (th == ea ? static_cast<Real*>(L->thbuf) : ea);
+    if (quads) {
+      if constexpr (kBC == 0 && sizeof(Real) == 4)
+        k_ftcs4<<<qgrid, tb, 0, L->stream>>>(K, src, th, kap, e, drho, th_next);
+    } else {
+      k_ftcs<Real, kBC><<<tgrid, tb, 0, L->stream>>>(K, src, th, kap, e, drho, th_next, gh);
+    }
+    src = e;
+    th = th_next;
   }
   RPK_CUDA(timing_end(L, RPK_KC_TRANSPORT, 2 + L->nsub));
   return check_launch("rotational transport");
