@@ -105,6 +105,7 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 ? 5 : 1)
               Real* __restrict__ u_out, Real* __restrict__ kap_out,
               const Real* __restrict__ ghost, unsigned* __restrict__ status,
               Real* __restrict__ tt_out, const Real* __restrict__ wcol) {
+  pdl_wait();
   PointIdx P;
   if (!point_from_block(K, P)) return;
   const int64_t p = (int64_t)P.s * K.n3 + P.cell;
@@ -159,6 +160,7 @@ __global__ void __launch_bounds__(128, sizeof(Store) == 4 ? 3 : 4)
                    const float* __restrict__ e_in, float* __restrict__ e_out, float* __restrict__ drho_out,
                    float* __restrict__ u_out, float* __restrict__ kap_out, unsigned* __restrict__ status,
                    float* __restrict__ tt_out) {
+  pdl_wait();
   using IO = PairIO<Store>;
   using Word = typename IO::Word;
   int s, i, y, z;
@@ -198,6 +200,7 @@ __global__ void __launch_bounds__(128, kPaper ? 4 : 5)
                      const float* __restrict__ e_in, float* __restrict__ e_out, float* __restrict__ drho_out,
                      float* __restrict__ u_out, float* __restrict__ kap_out, unsigned* __restrict__ status,
                      float* __restrict__ tt_out) {
+  pdl_wait();
   static_assert(std::is_same<Store, __half>::value, "the word-holding collision serves FP16 storage");
   using IO = PairIO<Store>;
   int s, i, y, z;

@@ -639,6 +639,7 @@ template <typename Store, typename Real, int kBC>
 __global__ void __launch_bounds__(128)
     k_wall_rho(StepConst<Real> K, const Store* __restrict__ pin, const Real* __restrict__ ghost,
                Real* __restrict__ wcol) {
+  pdl_wait();
   const int64_t ny_cols = (int64_t)K.nx * K.nz, nx_cols = (int64_t)K.ny * K.nz;
   const int64_t ybase = (kBC & kWallY) ? 2 * ny_cols : 0;
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

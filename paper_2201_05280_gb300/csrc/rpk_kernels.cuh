@@ -141,6 +141,7 @@ __global__ void __launch_bounds__(kTBX * kTBY)
     k_mac_pred(StepConst<Real> K, const Real* __restrict__ e, const Real* __restrict__ ucur,
                const Real* __restrict__ uprev, Real* __restrict__ ep, Real* __restrict__ v,
                const Real* __restrict__ ghost) {
+  pdl_wait();
   PointIdx P;
   if (!point_from_block2d(K, P)) return;
   const int64_t npts = 2 * K.n3;
@@ -173,6 +174,7 @@ __global__ void __launch_bounds__(kTBX * kTBY)
     k_mac_corr(StepConst<Real> K, const Real* __restrict__ e, const Real* __restrict__ ep,
                const Real* __restrict__ v, const Real* __restrict__ drho, Real* __restrict__ ec,
                Real* __restrict__ th, const Real* __restrict__ ghost) {
+  pdl_wait();
   PointIdx P;
   if (!point_from_block2d(K, P)) return;
   const int64_t npts = 2 * K.n3;
@@ -207,6 +209,7 @@ __global__ void __launch_bounds__(kTBX * kTBY)
     k_ftcs(StepConst<Real> K, const Real* ec, const Real* __restrict__ th, const Real* __restrict__ kap,
            Real* e_next, const Real* __restrict__ drho, Real* __restrict__ th_next,
            const Real* __restrict__ ghost) {
+  pdl_wait();
   PointIdx P;
   if (!point_from_block2d(K, P)) return;
   const int64_t p = (int64_t)P.s * K.n3 + P.cell;
@@ -267,6 +270,7 @@ __global__ void k_line_transport(StepConst<Real> K, const Real* __restrict__ e, 
                                  const Real* __restrict__ uprev, const Real* __restrict__ drho,
                                  const Real* __restrict__ kap, Real* __restrict__ e_next,
                                  const Real* __restrict__ ghost, int nsub) {
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char line_smem[];
   const int T = blockDim.x, l = threadIdx.x, nx = K.nx;
   Real* s0 = reinterpret_cast<Real*>(line_smem);  // two slots per thread, one spare at each end
@@ -366,6 +370,7 @@ __device__ __forceinline__ void un4(float4 q, float (&v)[4]) {
 static __global__ void __launch_bounds__(kTBX * kTBY)
     k_mac_pred4(StepConst<float> K, const float* __restrict__ e, const float* __restrict__ ucur,
                 const float* __restrict__ uprev, float* __restrict__ ep, float* __restrict__ v) {
+  pdl_wait();
   Quad Q;
   if (!quad_from_block(K, Q)) return;
   const int64_t npts = 2 * K.n3, p = Q.p;
@@ -409,6 +414,7 @@ static __global__ void __launch_bounds__(kTBX * kTBY)
     k_mac_corr4(StepConst<float> K, const float* __restrict__ e, const float* __restrict__ ep,
                 const float* __restrict__ v, const float* __restrict__ drho, float* __restrict__ ec,
                 float* __restrict__ th) {
+  pdl_wait();
   Quad Q;
   if (!quad_from_block(K, Q)) return;
   const int64_t npts = 2 * K.n3, p = Q.p;
@@ -449,6 +455,7 @@ static __global__ void __launch_bounds__(kTBX * kTBY)
 static __global__ void __launch_bounds__(kTBX * kTBY)
     k_ftcs4(StepConst<float> K, const float* ec, const float* __restrict__ th, const float* __restrict__ kap,
             float* e_next, const float* __restrict__ drho, float* __restrict__ th_next) {
+  pdl_wait();
   Quad Q;
   if (!quad_from_block(K, Q)) return;
   const int64_t p = Q.p;
@@ -507,6 +514,7 @@ static __global__ void __launch_bounds__(kTBX * kTBY)
 static __global__ void __launch_bounds__(kTBX * kTBY)
     k_pm_pred4(StepConst<float> K, const float* __restrict__ r, const float* __restrict__ ucur,
                float* __restrict__ rp) {
+  pdl_wait();
   Quad Q;
   if (!quad_from_block(K, Q)) return;
   const int64_t npts = 2 * K.n3, p = Q.p;
@@ -535,6 +543,7 @@ static __global__ void __launch_bounds__(kTBX * kTBY)
 static __global__ void __launch_bounds__(kTBX * kTBY)
     k_pm_corr4(StepConst<float> K, const float* __restrict__ r, const float* __restrict__ rp,
                const float* __restrict__ ucur, float* __restrict__ rc) {
+  pdl_wait();
   Quad Q;
   if (!quad_from_block(K, Q)) return;
   const int64_t npts = 2 * K.n3, p = Q.p;
@@ -564,6 +573,7 @@ static __global__ void __launch_bounds__(kTBX * kTBY)
 static __global__ void __launch_bounds__(kTBX * kTBY)
     k_pm_ftcs4(StepConst<float> K, const float* __restrict__ r, const float* __restrict__ drho,
                const float* __restrict__ kap, const float* __restrict__ tt, float* __restrict__ rn, int last) {
+  pdl_wait();
   Quad Q;
   if (!quad_from_block(K, Q)) return;
   const int64_t p = Q.p;
@@ -627,6 +637,7 @@ template <typename Real, int kBC>
 __global__ void __launch_bounds__(kTBX * kTBY)
     k_pm_pred(StepConst<Real> K, const Real* __restrict__ r, const Real* __restrict__ ucur,
               Real* __restrict__ rp, const Real* __restrict__ ghost) {
+  pdl_wait();
   PointIdx P;
   if (!point_from_block2d(K, P)) return;
   const int64_t p = (int64_t)P.s * K.n3 + P.cell, npts = 2 * K.n3;
@@ -641,6 +652,7 @@ template <typename Real, int kBC>
 __global__ void __launch_bounds__(kTBX * kTBY)
     k_pm_corr(StepConst<Real> K, const Real* __restrict__ r, const Real* __restrict__ rp,
               const Real* __restrict__ ucur, Real* __restrict__ rc, const Real* __restrict__ ghost) {
+  pdl_wait();
   PointIdx P;
   if (!point_from_block2d(K, P)) return;
   const int64_t p = (int64_t)P.s * K.n3 + P.cell, npts = 2 * K.n3;
@@ -656,6 +668,7 @@ __global__ void __launch_bounds__(kTBX * kTBY)
     k_pm_ftcs(StepConst<Real> K, const Real* __restrict__ r, const Real* __restrict__ drho,
               const Real* __restrict__ kap, const Real* __restrict__ tt, Real* __restrict__ rn,
               const Real* __restrict__ ghost, int last) {
+  pdl_wait();
   PointIdx P;
   if (!point_from_block2d(K, P)) return;
   const int64_t p = (int64_t)P.s * K.n3 + P.cell;

@@ -47,6 +47,15 @@ __device__ __forceinline__ F2 fmad(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v,
 __device__ __forceinline__ F2 fmad(float a, F2 b, F2 c) { return fmad(F2(a), b, c); }
 __device__ __forceinline__ F2 fmad(F2 a, float b, F2 c) { return fmad(a, F2(b), c); }
 
+// Programmatic dependent launch: the kernels of a step let the next one's
+// blocks become resident while their own still run, and wait here until every
+// earlier kernel has completed (a no-op for ordinary launches). Nothing that an
+// earlier kernel writes or reads may be touched before it.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Scalar type of a value type: the type of the per-launch constants.
 template <typename V>
 struct ScalarOf {
