@@ -544,7 +544,7 @@ __global__ void k_batch_init(TubeDev<Real>* __restrict__ tubes, const double* __
     const PointIdx P = tube_point(nx, p);
     const int64_t g = off + p;
     Real h[kQ], e;
-    init_point(K, hdt, rho[g], u[g], u[total_pts + g], u[2 * total_pts + g], T[g], R[g], h, e);
+    init_point<Real, true>(K, hdt, rho[g], u[g], u[total_pts + g], u[2 * total_pts + g], T[g], R[g], h, e);
     Store* out = base + (int64_t)(P.s * kQ) * K.n3 + P.cell;
 #pragma unroll
     for (int q = 0; q < kQ; ++q) out[(int64_t)q * K.n3] = from_real<Store, Real>(h[q]);
@@ -593,14 +593,14 @@ __global__ void k_batch_moments(const TubeDev<Real>* __restrict__ tubes, const S
     raw_moments_shells(h, m);
     recover<Real, false, true>(m, e_state[off + p], K);
     const int64_t g = off + p;
-    out[g] = 1.0 + (double)m.drho;
-    out[total_pts + g] = (double)(m.j[0] * m.inv_rho);
-    out[2 * total_pts + g] = (double)(m.j[1] * m.inv_rho);
-    out[3 * total_pts + g] = (double)(m.j[2] * m.inv_rho);
-    out[4 * total_pts + g] = (double)K.theta0 + (double)m.dT;
-    out[5 * total_pts + g] = (double)K.theta0 + (double)m.dR;
-    out[6 * total_pts + g] =
-        0.5 * (double)K.delta * (1.0 + (double)m.drho) * ((double)K.theta0 + (double)m.dR);
+    const double rh = 1.0 + to_double(m.drho), thR = to_double(K.theta0) + to_double(m.dR);
+    out[g] = rh;
+    out[total_pts + g] = to_double(m.j[0] * m.inv_rho);
+    out[2 * total_pts + g] = to_double(m.j[1] * m.inv_rho);
+    out[3 * total_pts + g] = to_double(m.j[2] * m.inv_rho);
+    out[4 * total_pts + g] = to_double(K.theta0) + to_double(m.dT);
+    out[5 * total_pts + g] = thR;
+    out[6 * total_pts + g] = 0.5 * to_double(K.delta) * rh * thR;
   }
 }
 

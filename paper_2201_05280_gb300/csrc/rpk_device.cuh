@@ -48,6 +48,44 @@ __device__ __forceinline__ __nv_bfloat16 from_real<__nv_bfloat16, float>(float v
   return __float2bfloat16_rn(v);
 }
 
+// FP32 <-> FP64 by integer operations, the same bits as the conversion
+// instructions: those go through the FP64 pipe, two lanes per cycle and SM, which
+// a pass over a field with FP64 inputs or outputs would otherwise wait for.
+__device__ __forceinline__ double to_double(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u || m == 0u) {  // normal or zero
+    const unsigned hi = m ? (m >> 3) + 0x38000000u : 0u;
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+  }
+  return (double)x;
+}
+__device__ __forceinline__ double to_double(double x) { return x; }
+
+template <typename Real>
+__device__ __forceinline__ Real round_to(double x);
+template <>
+__device__ __forceinline__ double round_to<double>(double x) { return x; }
+template <>
+__device__ __forceinline__ float round_to<float>(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), m = hi & 0x7fffffffu;
+  if (m - 0x38100000u < 0x0fd00000u) {  // rounds to a normal FP32 value
+    const unsigned f = ((m - 0x38000000u) << 3) | (lo >> 29), rest = lo & 0x1fffffffu;
+    const unsigned up = rest > 0x10000000u || (rest == 0x10000000u && (f & 1u));
+    return __uint_as_float((f + up) | (hi & 0x80000000u));
+  }
+  if ((m | lo) == 0u) return __uint_as_float(hi);
+  return (float)x;
+}
+
+// x > 0 and finite; x finite
+__device__ __forceinline__ bool positive_finite(double x) {
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b < 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool finite_bits(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
+}
+
 // compile-time loop: f(std::integral_constant<int, K>) for K = 0..N-1
 template <typename F, int... K>
 __device__ __forceinline__ void static_for_impl(F&& f, std::integer_sequence<int, K...>) {

@@ -236,10 +236,10 @@ __global__ void __launch_bounds__(kTBX * kTBY)
         thq = th[q];
         kq = kap[q];
       }
-      acc += Real(0.5) * (kp + kq) * (thq - thp);
+      acc += (kp + kq) * (thq - thp);
     }
   }
-  const Real val = ec[p] + K.hsub * acc;
+  const Real val = ec[p] + (K.hsub * Real(0.5)) * acc;  // the faces' 1/2 is exact
   e_next[p] = val;
   if (th_next) {
     const Real dr = drho[p];
@@ -686,33 +686,48 @@ __global__ void __launch_bounds__(kTBX * kTBY)
 // g = f - (dt/2) Omega(f) with Omega = (f^Eq(rho, u, theta I) - f)/tau1 (the ES
 // term vanishes since sigma = 0), Er = E_R - (dt/2)(delta rho/2)(theta - theta_R)/tau1.
 // Outputs h = g/w - 1 and e = Er - delta theta0/2.
-template <typename Real>
+// kSum: one expansion of the two targets' combined coefficients, shell by shell,
+// instead of two (half the operations; not for 16-bit storage, whose stored bits
+// depend on the rounding).
+template <typename Real, bool kSum = false>
 __device__ __forceinline__ void init_point(const StepConst<Real>& K, Real half_dt_over_tau1,
                                            double rho_d, double ux, double uy, double uz,
                                            double T, double R, Real (&h)[kQ], Real& e) {
-  const Real rho = Real(rho_d);
-  const Real drho = Real(rho_d - 1.0);
+  const Real rho = round_to<Real>(rho_d);
+  const Real drho = round_to<Real>(rho_d - 1.0);
   const Real inv_rho = Real(1) / rho;
-  const Real dT = Real(T - (double)K.theta0);
-  const Real dR = Real(R - (double)K.theta0);
+  const Real dT = round_to<Real>(T - to_double(K.theta0));
+  const Real dR = round_to<Real>(R - to_double(K.theta0));
   const Real dth = (Real(3) * dT + K.delta * dR) * K.inv_3pd;
-  const Real j[3] = {rho * Real(ux), rho * Real(uy), rho * Real(uz)};
+  const Real j[3] = {rho * round_to<Real>(ux), rho * round_to<Real>(uy), rho * round_to<Real>(uz)};
   Herm<Real> Hf, He;
   const Real Df[6] = {dT, dT, dT, 0, 0, 0};
   const Real De[6] = {dth, dth, dth, 0, 0, 0};
   hermite(drho, rho, inv_rho, j, Df, K.theta0, Hf);
   hermite(drho, rho, inv_rho, j, De, K.theta0, He);
   // g/w - 1 = (f/w - 1) - (dt/(2 tau1)) ((fEq/w - 1) - (f/w - 1))
-  h[0] = Hf.e0 - half_dt_over_tau1 * (He.e0 - Hf.e0);
-  static_for<kPairs>([&](auto kc) {
-    constexpr int k = decltype(kc)::value;
-    constexpr Vel2 v = kPairVel2[k];
-    const Real fe = herm_even<v.x, v.y, v.z>(Hf), fo = herm_odd<v.x, v.y, v.z>(Hf);
-    const Real ee = herm_even<v.x, v.y, v.z>(He), eo = herm_odd<v.x, v.y, v.z>(He);
-    const Real fp = fe + fo, fm = fe - fo, qp = ee + eo, qm = ee - eo;
-    h[2 * k + 1] = fp - half_dt_over_tau1 * (qp - fp);
-    h[2 * k + 2] = fm - half_dt_over_tau1 * (qm - fm);
-  });
+  if constexpr (kSum) {
+    Real* f = reinterpret_cast<Real*>(&Hf);
+    const Real* q = reinterpret_cast<const Real*>(&He);
+#pragma unroll
+    for (int i = 0; i < (int)(sizeof(Hf) / sizeof(Real)); ++i) f[i] = f[i] - half_dt_over_tau1 * (q[i] - f[i]);
+    h[0] = Hf.e0;
+    herm_shells(Hf, [&](int k, Real ev, Real od) {
+      h[2 * k + 1] = ev + od;
+      h[2 * k + 2] = ev - od;
+    });
+  } else {
+    h[0] = Hf.e0 - half_dt_over_tau1 * (He.e0 - Hf.e0);
+    static_for<kPairs>([&](auto kc) {
+      constexpr int k = decltype(kc)::value;
+      constexpr Vel2 v = kPairVel2[k];
+      const Real fe = herm_even<v.x, v.y, v.z>(Hf), fo = herm_odd<v.x, v.y, v.z>(Hf);
+      const Real ee = herm_even<v.x, v.y, v.z>(He), eo = herm_odd<v.x, v.y, v.z>(He);
+      const Real fp = fe + fo, fm = fe - fo, qp = ee + eo, qm = ee - eo;
+      h[2 * k + 1] = fp - half_dt_over_tau1 * (qp - fp);
+      h[2 * k + 2] = fm - half_dt_over_tau1 * (qm - fm);
+    });
+  }
   // E_R = delta rho theta_R/2 as a deviation from delta theta0/2 (paper mode:
   // the state is theta_R - theta0)
   e = K.paper ? dR
@@ -742,18 +757,19 @@ __global__ void __launch_bounds__(128)
     const int64_t p = (int64_t)P.s * K.n3 + P.cell;
     const double r = rho_in[p], T = T_in[p], R = R_in[p];
     const double ux = u_in[p], uy = u_in[npts + p], uz = u_in[2 * npts + p];
-    bad = !(r > 0.0) || !(T > 0.0) || !(R > 0.0) || !isfinite(r) || !isfinite(T) || !isfinite(R) ||
-          !isfinite(ux) || !isfinite(uy) || !isfinite(uz);
+    bad = !positive_finite(r) || !positive_finite(T) || !positive_finite(R) || !finite_bits(ux) ||
+          !finite_bits(uy) || !finite_bits(uz);
     if (!bad) {
-      tv = 3.0 * T + (double)K.delta * R;
+      tv = 3.0 * T + to_double(K.delta) * R;
       Real h[kQ], e;
-      init_point(K, half_dt_over_tau1, r, ux, uy, uz, T, R, h, e);
+      init_point<Real, kShells<Store>>(K, half_dt_over_tau1, r, ux, uy, uz, T, R, h, e);
       Store* out = pout + (int64_t)(P.s * kQ) * K.n3 + P.cell;
 #pragma unroll
       for (int q = 0; q < kQ; ++q) out[(int64_t)q * K.n3] = from_real<Store, Real>(h[q]);
       e_out[p] = e;
-      u0[p] = Real(ux); u0[npts + p] = Real(uy); u0[2 * npts + p] = Real(uz);
-      u1[p] = Real(ux); u1[npts + p] = Real(uy); u1[2 * npts + p] = Real(uz);
+      const Real u[3] = {round_to<Real>(ux), round_to<Real>(uy), round_to<Real>(uz)};
+      u0[p] = u[0]; u0[npts + p] = u[1]; u0[2 * npts + p] = u[2];
+      u1[p] = u[0]; u1[npts + p] = u[1]; u1[2 * npts + p] = u[2];
     }
   }
   // positive doubles order like their bit patterns: a warp maximum, then one
@@ -766,7 +782,11 @@ __global__ void __launch_bounds__(128)
   }
   const unsigned any_bad = __any_sync(0xffffffffu, bad);
   if ((threadIdx.x & 31) == 0) {
-    atomicMax(check, bits);
+    // only where it is above the value this SM last saw (which may be an older,
+    // smaller one): two million warps would queue at one address
+    unsigned long long seen;
+    asm volatile("ld.global.ca.u64 %0, [%1];" : "=l"(seen) : "l"(check));
+    if (bits > seen) atomicMax(check, bits);
     if (any_bad) atomicOr(check + 1, 1ull);
   }
 }
@@ -808,23 +828,21 @@ __global__ void __launch_bounds__(128)
   Real h[kQ];
   gather<Store, Real, kPull, kBC>(pin, ghost, K, P, h, wcol);
   Mom<Real> m;
-  if constexpr (kShells<Store>)
-    raw_moments_shells(h, m);
-  else
-    raw_moments(h, m);
+  raw_moments_shells(h, m);
   if (K.paper)
-    recover<Real, true, kShells<Store>>(m, e_in[p], K);
+    recover<Real, true, true>(m, e_in[p], K);
   else
-    recover<Real, false, kShells<Store>>(m, e_in[p], K);
-  if (rho_o) rho_o[p] = 1.0 + (double)m.drho;
+    recover<Real, false, true>(m, e_in[p], K);
+  const double rho = 1.0 + to_double(m.drho), R = to_double(K.theta0) + to_double(m.dR);
+  if (rho_o) rho_o[p] = rho;
   if (u_o) {
-    u_o[p] = (double)(m.j[0] * m.inv_rho);
-    u_o[npts + p] = (double)(m.j[1] * m.inv_rho);
-    u_o[2 * npts + p] = (double)(m.j[2] * m.inv_rho);
+    u_o[p] = to_double(m.j[0] * m.inv_rho);
+    u_o[npts + p] = to_double(m.j[1] * m.inv_rho);
+    u_o[2 * npts + p] = to_double(m.j[2] * m.inv_rho);
   }
-  if (T_o) T_o[p] = (double)K.theta0 + (double)m.dT;
-  if (R_o) R_o[p] = (double)K.theta0 + (double)m.dR;
-  if (E_o) E_o[p] = 0.5 * (double)K.delta * (1.0 + (double)m.drho) * ((double)K.theta0 + (double)m.dR);
+  if (T_o) T_o[p] = to_double(K.theta0) + to_double(m.dT);
+  if (R_o) R_o[p] = R;
+  if (E_o) E_o[p] = 0.5 * to_double(K.delta) * rho * R;
 }
 
 // ---- FP64 diagnostics: per-block partial sums, then one block reduces them.
