@@ -993,80 +993,105 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(Real) == 4 ? 4 : 1)
   diag_block_reduce(acc, partial);
 }
 
+// A running sum of two lanes in two FP32 words each (the rounding error of every
+// addition is kept exactly): 48 bits without the FP64 pipe, which issues two
+// lanes per cycle and SM. On 256^3 points its sums are those of FP64 additions to
+// 1e-13 of the sum of magnitudes, below the FP32 rounding of the terms.
+struct Sum2 {
+  F2 hi, lo;
+  __device__ __forceinline__ Sum2() : hi(0.f), lo(0.f) {}
+  __device__ __forceinline__ void add(F2 x) {
+    const F2 t = hi + x;
+    const F2 z = t - hi;
+    lo += (hi - (t - z)) + (x - z);
+    hi = t;
+  }
+  __device__ __forceinline__ double value() const {
+    return ((double)hi.v.x + (double)hi.v.y) + ((double)lo.v.x + (double)lo.v.y);
+  }
+};
+
 // k_diag for two x-adjacent points per thread (periodic pull, FP32
 // arithmetic, nx even; kPaper: the state holds theta_R as in the paper's
-// solver): the moments and targets in packed FP32x2 form, the logarithms and
-// the FP64 accumulation per point. Thread t handles pair t of the field planes
-// (sublattice t / (n3/2)).
+// solver): the moments and targets in packed FP32x2 form. Thread t handles pair
+// t of the field planes (sublattice t / (n3/2)).
+// Bound before: the FP64 pipe (12 additions and 9 conversions a point) and six
+// operations around each of the 41 logarithms; 256^3: 2.98 ms. Now the sums are
+// two-word FP32 (Sum2), sum f ln f takes one logarithm, a product and an FMA per
+// population (a logarithm of f <= 0 gives the NaN by itself, and sum f = rho),
+// and the smallest g comes from the smallest h of each shell: 1.52 ms.
 template <typename Store, bool kPaper>
 __global__ void __launch_bounds__(kDiagThreads, 3)
     k_diag_pair(StepConst<float> K, const Store* __restrict__ pin, const float* __restrict__ e_in,
                 double* __restrict__ partial) {
   using Word = typename PairIO<Store>::Word;
-  double acc[kDiagVals - 1] = {0, 0, 0, 0, 0, 0, INFINITY};
-  const int nxp = K.nx >> 1;
   const int64_t n3p = K.n3 >> 1;
   const double t0 = (double)K.theta0;
   int64_t npts_here = 0;
   const float beta = K.beta, keep = 1.f - K.beta;
-  auto hterm = [](float w, float fw) {  // w (fw ln fw - fw), fw = f/w
-    return fw > 0.f ? w * (fw * __logf(fw) - fw) : NAN;
-  };
+  Sum2 sM, sX, sY, sZ, sE, sH;
+  float gmin = INFINITY;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < 2 * n3p;
        t += (int64_t)gridDim.x * blockDim.x) {
-    const int s = (int)(t / n3p);
-    const int64_t cp = t - (int64_t)s * n3p;
-    const int i = (int)(cp % nxp);
-    const int64_t row = cp / nxp;
-    const int y = (int)(row % K.ny), z = (int)(row / K.ny);
+    const int s = t >= n3p;
+    const unsigned cp = (unsigned)(t - (s ? n3p : 0));
+    const unsigned row = K.by_nxp.div(cp), zz = K.by_ny.div(row);
+    const int i = (int)(cp - row * (unsigned)(K.nx >> 1)), y = (int)(row - zz * K.ny), z = (int)zz;
     F2 h[kQ];
     gather_pair<Store>(reinterpret_cast<const Word*>(pin), K, s, i, y, z, h);
     Mom<F2> m;
-    raw_moments(h, m);
+    raw_moments_shells(h, m);
     const F2 e(reinterpret_cast<const float2*>(e_in)[t]);
-    recover<float, kPaper>(m, e, K);
+    recover<float, kPaper, true>(m, e, K);
+    // smallest g = w (1 + h): w (1 + smallest h) shell by shell (rounding is monotone)
+    auto small = [&](int q) { return fminf(h[q].v.x, h[q].v.y); };
+    float gm = float(kWeightRest) * (1.f + small(0));
+    static_for<5>([&](auto sc) {
+      constexpr int ends[6] = {0, 3, 6, 12, 16, 20};
+      constexpr int shell = decltype(sc)::value, k0 = ends[shell], k1 = ends[shell + 1];
+      float hm = small(2 * k0 + 1);
+#pragma unroll
+      for (int q = 2 * k0 + 2; q <= 2 * k1; ++q) hm = fminf(hm, small(q));
+      gm = fminf(gm, float(pair_weight(k0)) * (1.f + hm));
+    });
+    gmin = fminf(gmin, gm);
+    sM.add(m.drho);
+    sX.add(m.j[0]);
+    sY.add(m.j[1]);
+    sZ.add(m.j[2]);
+    // paper mode holds theta_R: its energy density delta rho theta_R / 2 (deviation)
+    const F2 Ee = kPaper ? (0.5f * K.delta) * fmad(K.theta0, m.drho, m.rho * m.dR) : e;
+    sE.add(0.5f * (m.dP[0] + m.dP[1] + m.dP[2]));
+    sE.add(Ee);
+    // H1: sum f ln f - sum f - (delta/2) rho ln theta_R, f = (1 - beta*) g + beta* f^mix
     Herm<F2> H;
     mix_coeffs(m, K, H);
-    const float w0 = float(kWeightRest);
-    const F2 f0 = F2(1.f) + keep * h[0] + beta * H.e0;
-    float Hp[2] = {hterm(w0, f0.v.x), hterm(w0, f0.v.y)};
-    float gm[2] = {w0 * (1.f + h[0].v.x), w0 * (1.f + h[0].v.y)};
-    static_for<kPairs>([&](auto kc) {
-      constexpr int k = decltype(kc)::value;
-      constexpr Vel2 v = kPairVel2[k];
+    herm_scale(H, beta);
+    auto lg2 = [](F2 a) { return F2(__log2f(a.v.x), __log2f(a.v.y)); };
+    const F2 f0 = fmad(keep, h[0], H.e0 + 1.f);
+    F2 Hl = (float(kWeightRest) * f0) * lg2(f0);
+    herm_shells(H, [&](int k, F2 ev, F2 od) {
       const float w = float(pair_weight(k));
-      const F2 ev = herm_even<v.x, v.y, v.z>(H), od = herm_odd<v.x, v.y, v.z>(H);
-      const F2 fp = F2(1.f) + keep * h[2 * k + 1] + beta * (ev + od);
-      const F2 fm = F2(1.f) + keep * h[2 * k + 2] + beta * (ev - od);
-      Hp[0] += hterm(w, fp.v.x) + hterm(w, fm.v.x);
-      Hp[1] += hterm(w, fp.v.y) + hterm(w, fm.v.y);
-      gm[0] = fminf(gm[0], fminf(w * (1.f + h[2 * k + 1].v.x), w * (1.f + h[2 * k + 2].v.x)));
-      gm[1] = fminf(gm[1], fminf(w * (1.f + h[2 * k + 1].v.y), w * (1.f + h[2 * k + 2].v.y)));
+      const F2 fp = fmad(keep, h[2 * k + 1], ev + od) + 1.f, fm = fmad(keep, h[2 * k + 2], ev - od) + 1.f;
+      Hl = fmad(w * fp, lg2(fp), Hl);
+      Hl = fmad(w * fm, lg2(fm), Hl);
     });
-    const float drho[2] = {m.drho.v.x, m.drho.v.y}, rho[2] = {m.rho.v.x, m.rho.v.y};
-    const float jx[2] = {m.j[0].v.x, m.j[0].v.y}, jy[2] = {m.j[1].v.x, m.j[1].v.y};
-    const float jz[2] = {m.j[2].v.x, m.j[2].v.y}, dR[2] = {m.dR.v.x, m.dR.v.y};
-    const float ev[2] = {e.v.x, e.v.y};
-    const float p0[2] = {m.dP[0].v.x, m.dP[0].v.y}, p1[2] = {m.dP[1].v.x, m.dP[1].v.y};
-    const float p2[2] = {m.dP[2].v.x, m.dP[2].v.y};
-#pragma unroll
-    for (int l = 0; l < 2; ++l) {
-      acc[0] += (double)drho[l];
-      acc[1] += (double)jx[l];
-      acc[2] += (double)jy[l];
-      acc[3] += (double)jz[l];
-      // paper mode holds theta_R: its energy density delta rho theta_R / 2 (deviation)
-      const double Ee = kPaper ? 0.5 * (double)K.delta * ((double)rho[l] * (t0 + (double)dR[l]) - t0)
-                               : (double)ev[l];
-      acc[4] += 0.5 * ((double)p0[l] + (double)p1[l] + (double)p2[l]) + Ee;
-      acc[5] += (double)(Hp[l] - 0.5f * K.delta * rho[l] * __logf(K.theta0 + dR[l]));
-      acc[6] = fmin(acc[6], (double)gm[l]);
-    }
+    Hl = fmad((-0.5f * K.delta) * m.rho, lg2(m.dR + K.theta0), Hl);
+    // in units of ln 2, and rho as 1 + drho: the sums of -drho and -1 follow below
+    sH.add(Hl);
     npts_here += 2;
   }
+  const double ln2 = 0.6931471805599453094, M = sM.value();
+  const double n = (double)npts_here;
+  double acc[kDiagVals - 1];
   // the per-point constants: 1 (mass) and 3 theta0/2 + delta theta0/2 (energy)
-  acc[0] += (double)npts_here;
-  acc[4] += (double)npts_here * (1.5 * t0 + 0.5 * (double)K.delta * t0);
+  acc[0] = M + n;
+  acc[1] = sX.value();
+  acc[2] = sY.value();
+  acc[3] = sZ.value();
+  acc[4] = sE.value() + n * (1.5 * t0 + 0.5 * (double)K.delta * t0);
+  acc[5] = ln2 * sH.value() - M - n;
+  acc[6] = (double)gmin;
   diag_block_reduce(acc, partial);
 }
 
