@@ -173,65 +173,163 @@ __global__ void __launch_bounds__(kThreads) k_conv(ConvArgs P) {
       }
 }
 
+// k_conv for one tap (lift, head and the head's input gradient), bound by its
+// input and output: a warp takes 16 positions, reads their rows straight into
+// fragments (32-byte segments, each element once) and all kMT x 16 output channels
+// from weights that the block stages once for all its positions. The same
+// mma.sync shapes in the same order over k as k_conv, which re-staged 64 x 64
+// tiles element by element (606 K positions: lift 340 -> 141 us, head 324 -> 60
+// us).
+struct Conv1Args {
+  const __nv_bfloat16* A;  // [M][K]
+  const float* X;          // [npos][K]
+  float* out;              // [npos][M]
+  const float* bias;
+  const float* mask;
+  int M, K, relu_in, npos;
+};
+constexpr int kConv1Threads = 256;
+
+template <int kMT>
+__global__ void __launch_bounds__(kConv1Threads) k_conv1(Conv1Args P) {
+  extern __shared__ __align__(16) uint16_t c1_smem[];
+  const int Kp = (P.K + 15) / 16 * 16, ld = Kp + kPadK;
+  const int m0 = blockIdx.y * kMT * 16;
+  for (int e = threadIdx.x; e < kMT * 16 * ld; e += kConv1Threads) {
+    const int m = e / ld, k = e - m * ld;
+    const uint16_t* src = reinterpret_cast<const uint16_t*>(P.A);
+    c1_smem[e] = m0 + m < P.M && k < P.K ? src[(int64_t)(m0 + m) * P.K + k] : (uint16_t)0;
+  }
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int tiles = (P.npos + 15) / 16;
+  for (int tile = blockIdx.x * (kConv1Threads / 32) + warp; tile < tiles; tile += gridDim.x * (kConv1Threads / 32)) {
+    const int n0 = tile * 16;
+    float acc[kMT][2][4] = {};
+#pragma unroll 3
+    for (int k0 = 0; k0 < Kp; k0 += 16) {
+      uint32_t b[2][2];
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int q = n0 + j * 8 + g, k = k0 + 2 * t + 8 * h;
+          float2 x = make_float2(0.f, 0.f);
+          if (q < P.npos && k < P.K) x = *reinterpret_cast<const float2*>(P.X + (int64_t)q * P.K + k);
+          if (P.relu_in) x.x = fmaxf(x.x, 0.f), x.y = fmaxf(x.y, 0.f);
+          b[j][h] = pack_bf16(x.x, x.y);
+        }
+#pragma unroll
+      for (int i = 0; i < kMT; ++i) {
+        const uint16_t* r = c1_smem + (i * 16 + g) * ld + k0 + 2 * t;
+        const uint32_t a[4] = {*reinterpret_cast<const uint32_t*>(r), *reinterpret_cast<const uint32_t*>(r + 8 * ld),
+                               *reinterpret_cast<const uint32_t*>(r + 8),
+                               *reinterpret_cast<const uint32_t*>(r + 8 * ld + 8)};
+#pragma unroll
+        for (int j = 0; j < 2; ++j) mma_bf16(acc[i][j], a, b[j]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kMT; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          const int m = m0 + i * 16 + g + (h >= 2 ? 8 : 0), q = n0 + j * 8 + 2 * t + (h & 1);
+          if (m < P.M && q < P.npos) {
+            const int64_t o = (int64_t)q * P.M + m;
+            float v = acc[i][j][h];
+            if (P.bias) v += P.bias[m];
+            if (P.mask && !(P.mask[o] > 0.f)) v = 0.f;
+            P.out[o] = v;
+          }
+        }
+  }
+}
+
 // ---------------------------------------------------------------------------
-// Tensor-core (tcgen05) path of the residual-block convolutions: Co = Ci = 128,
-// 5 taps. One persistent CTA per SM keeps the layer's BF16 weights in shared
-// memory (A: 128 x 640, K-major) and walks over tiles of 128 output positions
-// of one sequence. Three roles run concurrently:
-//   producers (warps 8-15) load tile i's 132 input rows (positions q0 - 2 ..
-//     q0 + 129, every load in flight at once, 9 per thread) into registers
-//     while the MMAs of tile i - 1 still read the single input buffer B, then
-//     wait for B to be free and store the rows (activation applied, BF16);
-//   one issuing thread (warp 8, lane 0) waits for B and for the accumulator
-//     i % 2 to be free, issues 40 MMAs (M 128, N 128, K 16) into TMEM columns
-//     128 (i % 2) .. + 127 and commits to two mbarriers (B free, accumulator
-//     full);
-//   the epilogue (warps 0-7; TMEM lane = output channel, lane quadrant
-//     warp % 4) writes the tile as four quarters of 32 positions through two
-//     16 KB staging buffers in the output's own layout: the residual rows of
-//     the next quarter are bulk-copied into the other buffer (cp.async.bulk,
-//     completion on an mbarrier) while each thread adds its accumulator
-//     column, bias and mask to its elements of this one, and one thread
-//     bulk-copies the quarter to the output rows. The epilogue's global
-//     traffic is then two bulk copies per quarter instead of 64 loads and 64
-//     stores per thread, whose latency had set the tile period.
+// Tensor-core (tcgen05) path of a residual block, both convolutions (Co = Ci =
+// 128, 5 taps) in one kernel; the same kernel runs the block's input gradient:
+//   forward:   z = conv(relu(x); W1) + b1,    out = (conv(relu(z); W2) + b2) + x
+//   gradient:  z = conv^T(x; W1) (m1 > 0),    out = conv^T(z; W2) (m2 > 0) + x
+// (z is stored when zout is given: training needs it.) One persistent CTA per SM
+// walks over tiles of 124 output positions of one sequence; the tile's 128 rows
+// of z never leave the SM between the two convolutions. Roles:
+//   producers (warps 8-15) load tile i's 132 input rows into registers while
+//     the MMAs of tile i - 1 still read B1, then store them (activation, BF16);
+//   a loader thread (warp 16) keeps a ring of five 16 KB slots filled with half
+//     taps of weights, which lie in memory in the operand's own layout: one bulk
+//     copy each;
+//   an issuing thread (warp 17): 40 MMAs (M 128 positions, N 128 channels, K 16)
+//     per convolution in the order conv1(0), conv1(1), conv2(0), conv1(2),
+//     conv2(1), ..., so that the tensor cores work on conv1(i + 1) while the
+//     epilogue turns conv1(i) into conv2(i)'s operand;
+//   the epilogue (warps 0-7; TMEM lane = position, so that a thread holds 64
+//     consecutive channels of one position): e1(i) moves the first accumulator
+//     through bias, mask and activation into B2 (16-byte BF16 stores), then e2(i - 1)
+//     adds bias, mask and residual to the second one. Each warp owns 32 positions x
+//     64 channels of the tile: its residual rows were copied into its own staging
+//     block (cp.async) a tile earlier, and its output rows leave from there two
+//     whole rows an instruction, so no warp waits for another. Staging rows are 16
+//     bytes longer than their data: threads reading 16 bytes of 32 rows hit
+//     distinct banks.
 // The operand of tap t is the staged tile seen from row t (forward) or 4 - t
-// (input gradient): in the interleaved no-swizzle layout (rows 16 bytes apart
-// inside each 8-column chunk) a row shift is a start-address offset.
+// (gradient): in the interleaved no-swizzle layout (rows 16 bytes apart inside
+// each 8-column chunk) a row shift is a start-address offset. Every element is
+// accumulated in the same order as one convolution per launch did.
+// Bound: two launches per block moved 2.5 KB a position (z written and read, the
+// residual read again) at 3.5-5 TB/s with the epilogue's residual latency in the
+// way; one moves 1 KB, and the weights' 320 KB per tile come from L2. What is left
+// is shared memory: 8 KB per MMA, 320 KB of weights and the epilogue's rows make
+// 1.35 MB a tile, 10.5 k of the tile's 12.5 k cycles at 128 bytes a cycle. 606 K
+// positions: 2 x 178 us a block in two launches, 225 us in one; 32 crops of 1024
+// points (training, 96 tiles): 2 x 29.9 us -> 18.9 us. Tried: residual rows loaded
+// in the epilogue instead of copied ahead, 1715 against 1685 us a forward pass;
+// TMEM lane = channel with 2-byte stores into B2 and whole-block staging
+// barriers, 1863.
 constexpr int TC_M = 128, TC_N = 128, TC_KC = 128, TC_TAPS = 5;
+constexpr int TC_OUT = TC_N - (TC_TAPS - 1);               // 124 output positions per tile
 constexpr int TC_ROWS = TC_N + TC_TAPS - 1;                // 132 staged rows
 constexpr int TC_K = TC_TAPS * TC_KC;                      // 640
-constexpr uint32_t TC_A_LBO = TC_M * 16;                   // bytes between 8-wide k chunks of A
-// bytes between 8-wide k chunks of B: one row more than staged, so that the
-// producers' 16-byte stores of one row's consecutive chunks fall in distinct
+constexpr uint32_t TC_W_LBO = TC_N * 16;                   // bytes between 8-wide k chunks of a tap's weights
+// bytes between 8-wide k chunks of B1 and B2: one row more than staged, so that
+// the producers' 16-byte stores of one row's consecutive chunks fall in distinct
 // shared-memory banks (2128 / 4 = 532 = 20 mod 32)
 constexpr uint32_t TC_B_LBO = (TC_ROWS + 1) * 16;
-constexpr uint32_t TC_A_BYTES = (TC_K / 8) * TC_A_LBO;     // 163840
 constexpr uint32_t TC_B_BYTES = (TC_KC / 8) * TC_B_LBO;    // 34048
-constexpr int TC_QTR = TC_N / 4;                           // positions per staged quarter tile
-constexpr uint32_t TC_SQ_BYTES = TC_QTR * TC_M * 4;        // 16384: FP32 rows of a quarter tile
-constexpr uint32_t TC_S_BYTES = 2 * TC_SQ_BYTES;           // two staging buffers
-constexpr uint32_t TC_S_OFF = TC_A_BYTES + TC_B_BYTES;
-constexpr uint32_t TC_BAR_OFF = TC_S_OFF + TC_S_BYTES;
-constexpr uint32_t TC_SMEM = TC_BAR_OFF + 128;             // 8 mbarriers + TMEM address
+constexpr uint32_t TC_HALF_BYTES = TC_N * TC_KC;           // 16384: half a tap's weights (64 k)
+constexpr int TC_RING = 5;
+constexpr int TC_WCH = 64;                                 // channels of an epilogue warp's block
+constexpr uint32_t TC_S_LD = TC_WCH * 4 + 16;              // bytes between its staged rows
+constexpr uint32_t TC_SW_BYTES = 32 * TC_S_LD;             // staging of a warp
+constexpr uint32_t TC_W_OFF = 0;
+constexpr uint32_t TC_S_OFF = TC_W_OFF + TC_RING * TC_HALF_BYTES;
+constexpr uint32_t TC_B1_OFF = TC_S_OFF + 8 * TC_SW_BYTES;
+constexpr uint32_t TC_B2_OFF = TC_B1_OFF + TC_B_BYTES;
+constexpr uint32_t TC_BAR_OFF = TC_B2_OFF + TC_B_BYTES;
+constexpr uint32_t TC_BIAS_OFF = TC_BAR_OFF + 256;         // 17 mbarriers + TMEM address, then both biases
+constexpr uint32_t TC_SMEM = TC_BIAS_OFF + 2 * TC_N * 4;
 static_assert(TC_SMEM <= 227 * 1024, "tensor-core tiles exceed shared memory");
-static_assert(TC_S_OFF % 128 == 0, "the staging buffer is a bulk-copy operand");
-constexpr int TC_THREADS = 512;
+static_assert(TC_S_OFF % 128 == 0 && TC_B1_OFF % 128 == 0 && TC_BIAS_OFF % 16 == 0, "operand alignment");
 constexpr int TC_EPI = 256;                                // epilogue threads (warps 0-7)
-constexpr int TC_PROD = TC_THREADS - TC_EPI;               // producer threads (warps 8-15)
-constexpr int TC_COLS = 2 * TC_N;                          // two accumulators
+constexpr int TC_PROD = 256;                               // producer threads (warps 8-15)
+constexpr int TC_THREADS = TC_EPI + TC_PROD + 64;          // + loader and issuing warps
+constexpr int TC_COLS = 4 * TC_N;                          // two accumulators per convolution
 constexpr long long TC_WAIT_LIMIT = 1ll << 22;             // mbarrier polls before giving up
 
-struct TcArgs {
-  const __nv_bfloat16* A;  // [128][5][128]
-  const float* X;          // [npos][128]
-  float* out;              // [npos][128]
-  const float* bias;
-  const float* res;
-  const float* mask;
-  const int4* tiles;       // per tile (q0, count, sequence start, sequence length), or null
-  int ntiles, seq_len, tiles_per_seq, sgn, relu_in;
-  unsigned* error;         // set to 1 when an mbarrier wait gives up
+struct BlockArgs {
+  const __nv_bfloat16* w1;  // taps' weights, [5][16 chunks of 8 k][128 channels][8]
+  const __nv_bfloat16* w2;
+  const float* x;           // [npos][128] input, and the residual
+  float* zout;              // [npos][128], or null
+  float* out;               // [npos][128]
+  const float* b1;          // biases, or null
+  const float* b2;
+  const float* m1;          // masks (> 0 keeps), or null
+  const float* m2;
+  const int4* tiles;        // per tile (q0, count, sequence start, sequence length), or null
+  int ntiles, seq_len, tiles_per_seq, sgn, relu;
+  unsigned* error;          // set to 1 when an mbarrier wait gives up
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -268,7 +366,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
 }
 
-__device__ __forceinline__ void tc_tile(const TcArgs& P, int tile, int& q0, int& cnt, int& lo, int& len) {
+__device__ __forceinline__ void tc_tile(const BlockArgs& P, int tile, int& q0, int& cnt, int& lo, int& len) {
   if (P.tiles) {
     const int4 d = P.tiles[tile];
     q0 = d.x, cnt = d.y, lo = d.z, len = d.w;
@@ -276,17 +374,11 @@ __device__ __forceinline__ void tc_tile(const TcArgs& P, int tile, int& q0, int&
     const int sq = tile / P.tiles_per_seq, part = tile - sq * P.tiles_per_seq;
     lo = sq * P.seq_len;
     len = P.seq_len;
-    q0 = lo + part * TC_N;
-    cnt = min(TC_N, len - part * TC_N);
+    q0 = lo + part * TC_OUT;
+    cnt = min(TC_OUT, len - part * TC_OUT);
   }
 }
 
-// Barrier 1 among the 256 epilogue threads (the producers never use it).
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(TC_EPI) : "memory"); }
-
-// The same barrier, returning whether p holds in every epilogue thread: the
-// epilogue warps then leave their loops together and no warp waits at a
-// barrier that another has left.
 // 16 consecutive accumulator columns of this thread's TMEM lane (32x32b shape)
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
   asm volatile(
@@ -297,38 +389,53 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
       : "r"(taddr));
 }
 
-__device__ __forceinline__ bool epi_all(bool p) {
-  int r;
+// 32 consecutive accumulator columns
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile(
-      "{\n .reg .pred pi, po;\n setp.ne.b32 pi, %1, 0;\n bar.red.and.pred po, 1, %2, pi;\n"
-      " selp.b32 %0, 1, 0, po;\n}\n"
-      : "=r"(r)
-      : "r"((int)p), "n"(TC_EPI)
-      : "memory");
-  return r != 0;
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
+        "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+        "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      : "r"(taddr));
 }
 
-// Bulk copy of the residual rows of quarter q of a tile (positions q0 + 32 q ..)
-// into a staging buffer, completing with its byte count on the mbarrier bar.
-__device__ __forceinline__ void qtr_load(const TcArgs& P, uint32_t bar, uint32_t dst, int q0, int cnt, int q) {
-  const int rows = min(TC_QTR, cnt - q * TC_QTR);
-  const uint32_t bytes = (uint32_t)rows * TC_M * 4;
+// Announce the bytes that bulk copies will complete on bar (its one arrival).
+__device__ __forceinline__ void bulk_expect(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+
+// Bulk copy of bytes into shared memory, counted on bar.
+__device__ __forceinline__ void bulk_load(uint32_t bar, uint32_t dst, const void* src, uint32_t bytes) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(P.res + (int64_t)(q0 + q * TC_QTR) * TC_M), "r"(bytes), "r"(bar)
+               "l"(src), "r"(bytes), "r"(bar)
                : "memory");
 }
 
-__global__ void __launch_bounds__(TC_THREADS, 1) k_conv_tc(TcArgs P) {
-  extern __shared__ __align__(1024) unsigned char tc_smem[];
-  unsigned char* sA = tc_smem;
-  unsigned char* sB = tc_smem + TC_A_BYTES;
-  float* sS = reinterpret_cast<float*>(tc_smem + TC_S_OFF);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(tc_smem + TC_BAR_OFF);
-  // bars: 0 B full, 1 B free, 2-3 accumulator full, 4-5 accumulator free, 6-7 residual in S[0], S[1]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tc_smem + TC_BAR_OFF + 64);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+// mbarriers of k_block_tc
+enum {
+  kB1Full = 0,   // producers: x tile staged
+  kB1Free,       // MMAs of conv1 done with it
+  kB2Full,       // epilogue: z tile staged (its TMEM reads done)
+  kAcc1,         // + 0, 1: conv1's accumulator ready
+  kAcc2 = kAcc1 + 2,  // + 0, 1: conv2's accumulator ready, B2 free
+  kWFull = kAcc2 + 2,
+  kWFree = kWFull + TC_RING,
+  kBars = kWFree + TC_RING
+};
+static_assert(kBars * 8 + 8 <= 256, "barrier space");
 
+__global__ void __launch_bounds__(TC_THREADS, 1) k_block_tc(BlockArgs P) {
+  extern __shared__ __align__(1024) unsigned char tc_smem[];
+  uint64_t* bars = reinterpret_cast<uint64_t*>(tc_smem + TC_BAR_OFF);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tc_smem + TC_BAR_OFF + 8 * kBars);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t base = smem_u32(tc_smem), bar0 = smem_u32(bars);
+  auto bar = [&](int k) { return bar0 + 8u * (uint32_t)k; };
+
+  // the next kernel's CTAs may take the SMs this grid leaves free
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)),
@@ -337,70 +444,135 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv_tc(TcArgs P) {
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bars)), "r"(TC_PROD) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bars + 1)), "r"(1) : "memory");
-    for (int a = 0; a < 2; ++a) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bars + 2 + a)), "r"(1) : "memory");
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bars + 4 + a)), "r"(TC_EPI) : "memory");
+    for (int k = 0; k < kBars; ++k) {
+      const int n = k == kB1Full ? TC_PROD : k == kB2Full ? TC_EPI : 1;
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar(k)), "r"(n) : "memory");
     }
-    for (int q = 0; q < 2; ++q)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bars + 6 + q)), "r"(1) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // weights: chunk c (k = 8c .. 8c + 7) of row m at c * TC_A_LBO + m * 16,
-  // copied global -> shared asynchronously (every thread's 20 copies in flight
-  // at once, no register round trip)
-  for (int e = tid; e < TC_M * (TC_K / 8); e += TC_THREADS) {
-    const int m = e % TC_M, c = e / TC_M;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(sA + c * TC_A_LBO + m * 16)),
-                 "l"(P.A + (int64_t)m * TC_K + 8 * c)
-                 : "memory");
+  // parameters (weights and biases) are never written while kernels of one pass
+  // follow each other: they are read before the previous kernel has finished
+  float* sbias = reinterpret_cast<float*>(tc_smem + TC_BIAS_OFF);
+  if (tid < 2 * TC_N) {
+    const float* b = tid < TC_N ? P.b1 : P.b2;
+    sbias[tid] = b ? b[tid & (TC_N - 1)] : 0.f;
   }
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
-  const uint32_t a_base = smem_u32(sA), b_base = smem_u32(sB), s_base = smem_u32(sS);
-  const uint32_t bar0 = smem_u32(bars);
+  // tiles of this CTA: blockIdx.x + i gridDim.x, i < n
+  const int n = (P.ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
   bool ok = true;
 
-  if (tid >= TC_EPI) {
-    // producers, and the issuing thread
+  if (warp == 16) {
+    if (lane == 0) {
+      int r = 0;
+      for (int i = 0; i <= n && ok; ++i)
+        for (int c = 0; c < 2 && ok; ++c) {
+          if (c == 0 ? i == n : i == 0) continue;
+          const unsigned char* w = reinterpret_cast<const unsigned char*>(c == 0 ? P.w1 : P.w2);
+          for (int t = 0; t < 2 * TC_TAPS && ok; ++t, ++r) {
+            const int slot = r % TC_RING;
+            if (r >= TC_RING) ok = mbar_wait(bar(kWFree + slot), ((r / TC_RING) - 1) & 1);
+            if (ok) {
+              bulk_expect(bar(kWFull + slot), TC_HALF_BYTES);
+              bulk_load(bar(kWFull + slot), base + TC_W_OFF + slot * TC_HALF_BYTES, w + t * TC_HALF_BYTES, TC_HALF_BYTES);
+            }
+          }
+        }
+      if (!ok) atomicOr(P.error, 1u);
+      // copies still in flight land before the CTA's shared memory is released
+      for (int k = max(0, r - TC_RING); k < r; ++k) mbar_wait(bar(kWFull + k % TC_RING), (k / TC_RING) & 1);
+    }
+  } else if (warp == 17) {
+    // the whole warp runs the loop, so that descriptors stay in uniform
+    // registers; one elected lane issues
+    uint32_t one;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(one));
+    int r = 0;
+    auto commit = [&](uint32_t b) {
+      asm volatile(
+          "{\n .reg .pred e;\n setp.ne.b32 e, %1, 0;\n"
+          " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(b),
+          "r"(one)
+          : "memory");
+    };
+    auto conv = [&](uint32_t b_base, uint32_t d) {
+#pragma unroll 2
+      for (int t = 0; t < 2 * TC_TAPS; ++t, ++r) {  // half taps
+        const int slot = r % TC_RING;
+        if (!mbar_wait(bar(kWFull + slot), (r / TC_RING) & 1)) return false;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int tap = t >> 1, row0 = P.sgn > 0 ? tap : TC_TAPS - 1 - tap;
+        const uint64_t ad = tc_desc(b_base + (uint32_t)((t & 1) * 8) * TC_B_LBO + (uint32_t)row0 * 16, TC_B_LBO, 128);
+        const uint64_t bd = tc_desc(base + TC_W_OFF + slot * TC_HALF_BYTES, TC_W_LBO, 128);
+#pragma unroll
+        for (int k = 0; k < TC_KC / 32; ++k) {
+          // the address field counts 16 bytes
+          asm volatile(
+              "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 e, %5, 0;\n"
+              " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+              "l"(ad + (uint64_t)(2 * k * (TC_B_LBO / 16))), "l"(bd + (uint64_t)(2 * k * (TC_W_LBO / 16))),
+              "r"(TC_IDESC), "r"((uint32_t)(t | k)), "r"(one)
+              : "memory");
+        }
+        commit(bar(kWFree + slot));
+      }
+      return true;
+    };
+    for (int i = 0; i <= n && ok; ++i) {
+      if (i < n) {
+        // accumulator i % 2 was read by e1(i - 2), before conv2(i - 2) was issued
+        ok = mbar_wait(bar(kB1Full), i & 1) && conv(base + TC_B1_OFF, tmem + (uint32_t)((i & 1) * TC_N));
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        commit(bar(kB1Free));
+        commit(bar(kAcc1 + (i & 1)));
+      }
+      if (i >= 1) {
+        const int j = i - 1;
+        // accumulator j % 2 was read by e2(j - 2), before e1(j) staged B2
+        ok = mbar_wait(bar(kB2Full), j & 1) && conv(base + TC_B2_OFF, tmem + (uint32_t)((2 + (j & 1)) * TC_N));
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        commit(bar(kAcc2 + (j & 1)));
+      }
+    }
+    if (!ok && lane == 0) atomicOr(P.error, 1u);
+  } else if (tid >= TC_EPI) {
+    // producers: 2112 (row, 8-channel chunk) elements, at most 9 per thread;
+    // consecutive threads take consecutive 32-byte chunks of a row
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int ptid = tid - TC_EPI;
-    // 2112 (row, 8-channel chunk) elements, at most 9 per thread; consecutive
-    // threads take consecutive 32-byte chunks of a row (coalesced 512-byte rows)
     constexpr int kElems = TC_ROWS * (TC_KC / 8);
     constexpr int kBatch = (kElems + TC_PROD - 1) / TC_PROD;
-    static_assert(kBatch * TC_PROD >= kElems, "one batch of loads covers the tile");
-    for (int i = 0, tile = blockIdx.x; tile < P.ntiles && ok; ++i, tile += gridDim.x) {
+    for (int i = 0; i < n && ok; ++i) {
       int q0, cnt, lo, len;
-      tc_tile(P, tile, q0, cnt, lo, len);
-      // every load of tile i is issued while the MMAs of tile i - 1 still read B
+      tc_tile(P, (int)blockIdx.x + i * (int)gridDim.x, q0, cnt, lo, len);
       float4 f[kBatch][2];
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) {
         const int e = ptid + u * TC_PROD;
         const int r = e / (TC_KC / 8), c = e % (TC_KC / 8);
-        const int q = q0 - 2 + r;
+        const int q = q0 - (TC_TAPS - 1) + r;
         f[u][0] = f[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (e < kElems && q >= lo && q < lo + len) {
-          const float4* src = reinterpret_cast<const float4*>(P.X + (int64_t)q * TC_KC + 8 * c);
+          const float4* src = reinterpret_cast<const float4*>(P.x + (int64_t)q * TC_KC + 8 * c);
           f[u][0] = src[0];
           f[u][1] = src[1];
         }
       }
-      // B free: the MMAs of tile i - 1 have completed
-      if (i >= 1) ok = __all_sync(0xffffffffu, mbar_wait(bar0 + 8, (i - 1) & 1));
+      if (i >= 1) ok = __all_sync(0xffffffffu, mbar_wait(bar(kB1Free), (i - 1) & 1));
       if (!ok) break;
+      unsigned char* sB = tc_smem + TC_B1_OFF;
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) {
         const int e = ptid + u * TC_PROD;
         if (e >= kElems) break;
         const int r = e / (TC_KC / 8), c = e % (TC_KC / 8);
         float4 f0 = f[u][0], f1 = f[u][1];
-        if (P.relu_in) {
+        if (P.relu) {
           f0.x = fmaxf(f0.x, 0.f), f0.y = fmaxf(f0.y, 0.f), f0.z = fmaxf(f0.z, 0.f), f0.w = fmaxf(f0.w, 0.f);
           f1.x = fmaxf(f1.x, 0.f), f1.y = fmaxf(f1.y, 0.f), f1.z = fmaxf(f1.z, 0.f), f1.w = fmaxf(f1.w, 0.f);
         }
@@ -409,135 +581,150 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv_tc(TcArgs P) {
                        pack_bf16(f1.z, f1.w));
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      mbar_arrive(bar0);  // B full (TC_PROD arrivals)
-      if (ptid == 0) {
-        // the issuing thread: B staged by all producers, accumulator i % 2 free
-        const int acc = i & 1;
-        bool go = mbar_wait(bar0, i & 1);
-        if (go && i >= 2) go = mbar_wait(bar0 + 8 * (4 + acc), ((i >> 1) - 1) & 1);
-        if (go) {
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t d = tmem + (uint32_t)(acc * TC_N);
-#pragma unroll 1
-          for (int t = 0; t < TC_TAPS; ++t) {
-            const int row0 = P.sgn > 0 ? t : TC_TAPS - 1 - t;
-#pragma unroll
-            for (int s = 0; s < TC_KC / 16; ++s) {
-              const uint64_t ad =
-                  tc_desc(a_base + (uint32_t)(t * (TC_KC / 8) + 2 * s) * TC_A_LBO, TC_A_LBO, 128);
-              const uint64_t bd = tc_desc(b_base + (uint32_t)(2 * s) * TC_B_LBO + (uint32_t)row0 * 16, TC_B_LBO, 128);
-              const uint32_t accum = (t | s) ? 1u : 0u;
-              asm volatile(
-                  "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                  " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-                  "l"(ad), "l"(bd), "r"(TC_IDESC), "r"(accum)
-                  : "memory");
-            }
-          }
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           bar0 + 8)
-                       : "memory");
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                           bar0 + 8 * (2 + acc))
-                       : "memory");
-        } else {
-          atomicOr(P.error, 1u);
-        }
-      }
-      __syncwarp();
+      mbar_arrive(bar(kB1Full));
     }
+    if (!ok && lane == 0) atomicOr(P.error, 1u);
   } else {
-    // epilogue: TMEM lane = output channel m; a tile is written as four
-    // quarters of 32 positions through two 16 KB staging buffers (quarter q in
-    // S[q % 2]); warps 0-3 take positions 0-15 of a quarter, warps 4-7 16-31.
-    // With a residual, the rows of quarter q + 1 are bulk-loaded into the other
-    // buffer while quarter q is computed; every quarter leaves as one bulk store.
-    const int quad = warp & 3, sub = warp >> 2;
-    const int m = quad * 32 + lane;
-    const float bm = P.bias ? P.bias[m] : 0.f;
-    const uint32_t rbar = bar0 + 8 * 6;  // 6: residual in S[0], 7: residual in S[1]
-    int rphase[2] = {0, 0};  // residual copies waited for, per buffer (every thread)
-    int rissued[2] = {0, 0};  // residual copies issued, per buffer (thread 0)
-    for (int i = 0, tile = blockIdx.x; tile < P.ntiles; ++i, tile += gridDim.x) {
-      const int acc = i & 1;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int quad = warp & 3, c0 = (warp >> 2) * TC_WCH;  // positions 32 quad .., channels c0 ..
+    const int row = quad * 32 + lane;
+    const uint32_t lanes = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0;
+    const uint32_t s_base = base + TC_S_OFF + warp * TC_SW_BYTES;
+    float* srow = reinterpret_cast<float*>(tc_smem + TC_S_OFF + warp * TC_SW_BYTES + lane * TC_S_LD);
+    // lane's 16-byte piece of a row pair: rows 2 k + (lane / 16), piece lane % 16
+    const int prow = lane >> 4, piece = lane & 15;
+    // residual rows of tile i, asynchronously
+    auto load_residual = [&](int i) {
       int q0, cnt, lo, len;
-      tc_tile(P, tile, q0, cnt, lo, len);
-      const int nq = (cnt + TC_QTR - 1) / TC_QTR;  // quarters holding positions
-      if (tid == 0) {
-        // both buffers are free once every earlier bulk store has read them out
-        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-        if (P.res)
-          for (int q = 0; q < 2 && q < nq; ++q) {
-            qtr_load(P, rbar + 8 * q, s_base + q * TC_SQ_BYTES, q0, cnt, q);
-            ++rissued[q];
-          }
+      tc_tile(P, (int)blockIdx.x + i * (int)gridDim.x, q0, cnt, lo, len);
+      const float* src = P.x + (int64_t)(q0 + quad * 32 + prow) * TC_M + c0 + 4 * piece;
+      const uint32_t dst = s_base + prow * TC_S_LD + 16 * piece;
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        if (quad * 32 + 2 * k + prow < cnt)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 2 * k * TC_S_LD),
+                       "l"(src + 2 * k * TC_M)
+                       : "memory");
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // bit c: channel c0 + c of position q is masked out (q inside its sequence)
+    auto masked = [&](const float* mask, int64_t q) {
+      uint64_t drop = 0;
+      const float4* src = reinterpret_cast<const float4*>(mask + q * TC_M + c0);
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        float4 f[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) f[k] = src[8 * g + k];
+        uint32_t bits = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          bits |= ((f[k].x > 0.f ? 0u : 1u) | (f[k].y > 0.f ? 0u : 2u) | (f[k].z > 0.f ? 0u : 4u) |
+                   (f[k].w > 0.f ? 0u : 8u))
+                  << (4 * k);
+        drop |= (uint64_t)bits << (32 * g);
       }
-      ok = epi_all(mbar_wait(bar0 + 8 * (2 + acc), (i >> 1) & 1));
-      if (!ok) break;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      for (int q = 0; q < nq && ok; ++q) {
-        const int buf = q & 1;
-        const int rows = min(TC_QTR, cnt - q * TC_QTR);
-        const int64_t qq = (int64_t)(q0 + q * TC_QTR);
-        float* S = sS + buf * (TC_QTR * TC_M);
-        if (P.res) {
-          ok = epi_all(mbar_wait(rbar + 8 * buf, rphase[buf] & 1));
-          if (!ok) break;
-          ++rphase[buf];
-          if (tid == 0 && q >= 1 && q + 1 < nq) {
-            // the store of quarter q - 1 has read S[1 - buf] before the next rows land there
-            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            qtr_load(P, rbar + 8 * (1 - buf), s_base + (1 - buf) * TC_SQ_BYTES, q0, cnt, q + 1);
-            ++rissued[1 - buf];
-          }
-        } else {
-          // the store of quarter q - 2 has read S[buf] (the latest one may still be reading the other)
-          if (tid == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-          epi_sync();
-        }
-        uint32_t v[16];
-        tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * TC_N + q * TC_QTR + sub * 16), v);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        uint32_t drop = 0;  // bit k: masked out
-        if (P.mask) {
+      return drop;
+    };
+    if (n > 0) load_residual(0);
+    for (int i = 0; i <= n && ok; ++i) {
+      if (i < n) {
+        // e1(i): row q0 - 2 + row of z
+        int q0, cnt, lo, len;
+        tc_tile(P, (int)blockIdx.x + i * (int)gridDim.x, q0, cnt, lo, len);
+        const int q = q0 - 2 + row;
+        const bool in = q >= lo && q < lo + len;  // else zero padding of the second convolution
+        const uint64_t drop = P.m1 ? masked(P.m1, min(max(q, lo), lo + len - 1)) : 0;
+        ok = mbar_wait(bar(kAcc1 + (i & 1)), (i >> 1) & 1);
+        // conv2(i - 1) has read B2
+        if (ok && i >= 1) ok = mbar_wait(bar(kAcc2 + ((i - 1) & 1)), ((i - 1) >> 1) & 1);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        unsigned char* zb = tc_smem + TC_B2_OFF + (c0 / 8) * TC_B_LBO + row * 16;
+        float4* zo = P.zout && row >= 2 && row < 2 + cnt ? reinterpret_cast<float4*>(P.zout + (int64_t)q * TC_M + c0)
+                                                         : nullptr;
 #pragma unroll
-          for (int k = 0; k < 16; ++k) {
-            const int r = sub * 16 + k;
-            if (r < rows && !(P.mask[(qq + r) * TC_M + m] > 0.f)) drop |= 1u << k;
-          }
-        }
+        for (int g = 0; g < 2; ++g) {
+          uint32_t v[32];
+          tmem_ld32(lanes + (uint32_t)((i & 1) * TC_N + g * 32), v);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          const uint32_t d32 = (uint32_t)(drop >> (32 * g));
+          const float4* b4 = reinterpret_cast<const float4*>(sbias + c0 + g * 32);
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-          const int r = sub * 16 + k;
-          if (r < rows) {
-            float* sp = S + r * TC_M + m;
-            float val = ((drop >> k) & 1u) ? 0.f : __uint_as_float(v[k]) + bm;
-            if (P.res) val += *sp;
-            *sp = val;
+          for (int k = 0; k < 8; ++k) {
+            const float4 b = b4[k];
+            float f[4] = {__uint_as_float(v[4 * k]) + b.x, __uint_as_float(v[4 * k + 1]) + b.y,
+                          __uint_as_float(v[4 * k + 2]) + b.z, __uint_as_float(v[4 * k + 3]) + b.w};
+#pragma unroll
+            for (int l = 0; l < 4; ++l)
+              if (!in || ((d32 >> (4 * k + l)) & 1u)) f[l] = 0.f;
+            if (zo) zo[8 * g + k] = make_float4(f[0], f[1], f[2], f[3]);
+            if (P.relu) {
+#pragma unroll
+              for (int l = 0; l < 4; ++l) f[l] = fmaxf(f[l], 0.f);
+            }
+            v[2 * k] = pack_bf16(f[0], f[1]);
+            v[2 * k + 1] = pack_bf16(f[2], f[3]);
           }
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            *reinterpret_cast<uint4*>(zb + (4 * g + c) * TC_B_LBO) =
+                make_uint4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        epi_sync();
-        if (tid == 0) {
-          asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(P.out + qq * TC_M),
-                       "r"(s_base + buf * TC_SQ_BYTES), "r"((uint32_t)rows * TC_M * 4)
-                       : "memory");
-          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        mbar_arrive(bar(kB2Full));
+      } else if (n > 0) {
+        ok = __all_sync(0xffffffffu, mbar_wait(bar(kAcc2 + ((n - 1) & 1)), ((n - 1) >> 1) & 1));
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       }
-      if (!ok) break;
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      mbar_arrive(bar0 + 8 * (4 + acc));  // accumulator free (TC_EPI arrivals)
+      if (i >= 1) {
+        // e2(i - 1)
+        const int j = i - 1;
+        int q0, cnt, lo, len;
+        tc_tile(P, (int)blockIdx.x + j * (int)gridDim.x, q0, cnt, lo, len);
+        const uint64_t drop = P.m2 ? masked(P.m2, min(q0 + row, lo + len - 1)) : 0;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncwarp();  // every lane's pieces have landed
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          uint32_t v[32];
+          tmem_ld32(lanes + (uint32_t)((2 + (j & 1)) * TC_N + g * 32), v);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          const uint32_t d32 = (uint32_t)(drop >> (32 * g));
+          const float4* b4 = reinterpret_cast<const float4*>(sbias + TC_N + c0 + g * 32);
+          float4* s4 = reinterpret_cast<float4*>(srow + g * 32);
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const float4 b = b4[k];
+            float4 r = s4[k];
+            float f[4] = {__uint_as_float(v[4 * k]) + b.x, __uint_as_float(v[4 * k + 1]) + b.y,
+                          __uint_as_float(v[4 * k + 2]) + b.z, __uint_as_float(v[4 * k + 3]) + b.w};
+#pragma unroll
+            for (int l = 0; l < 4; ++l)
+              if ((d32 >> (4 * k + l)) & 1u) f[l] = 0.f;
+            r.x = f[0] + r.x, r.y = f[1] + r.y, r.z = f[2] + r.z, r.w = f[3] + r.w;
+            s4[k] = r;
+          }
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        const float4* from = reinterpret_cast<const float4*>(tc_smem + TC_S_OFF + warp * TC_SW_BYTES +
+                                                             prow * TC_S_LD + 16 * piece);
+        float* to = P.out + (int64_t)(q0 + quad * 32 + prow) * TC_M + c0 + 4 * piece;
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          if (quad * 32 + 2 * k + prow < cnt)
+            *reinterpret_cast<float4*>(to + 2 * k * TC_M) = from[2 * k * (TC_S_LD / 16)];
+        __syncwarp();  // read out before the next residual lands there
+        if (i < n) load_residual(i);
+      }
     }
-    if (!ok && tid == 0) {
-      atomicOr(P.error, 1u);
-      // after a wait that gave up, let residual copies still in flight land
-      // (bounded waits) before the CTA's shared memory is released
-      for (int b = 0; b < 2; ++b)
-        for (; rphase[b] < rissued[b]; ++rphase[b]) mbar_wait(rbar + 8 * b, rphase[b] & 1);
-    }
-    // the output is written and S read out before the CTA ends
-    if (tid == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    if (!ok && lane == 0) atomicOr(P.error, 1u);
+    // residual copies still in flight after a wait that gave up
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -550,7 +737,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv_tc(TcArgs P) {
 // (tcgen05; Co = Ci = 128, 5 taps, ReLU inputs):
 //   dW[o][t][i] += sum_q dY[q][o] relu(X[q + t - 2][i]),  db[o] += sum_q dY[q][o].
 // The reduction runs over positions, so both operands are MN-major: a tile of
-// 128 positions is staged as in k_conv_tc (8-channel chunks, rows 16 bytes
+// 128 positions is staged as in k_block_tc (8-channel chunks, rows 16 bytes
 // apart), which read with channels as M or N and rows as K is the no-swizzle
 // MN-major layout (SBO = chunk stride, LBO = 128 bytes between groups of 8
 // rows), and the tap shift is again a start-address offset of 16 bytes a row.
@@ -564,6 +751,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_conv_tc(TcArgs P) {
 // tiles re-staged by every block: 12 launches of 99 us (mma.sync) and 12 of
 // 22.5 us (bias) for 32 crops of 1024 points became one of 41 us.
 constexpr int DW_N = 64;                                    // input channels per CTA
+constexpr int DW_THREADS = 512;
 constexpr uint32_t DW_A_STRIDE = (TC_N + 1) * 16;           // dY: bytes between 8-channel chunks
 constexpr uint32_t DW_B_STRIDE = (TC_ROWS + 1) * 16;        // X
 constexpr uint32_t DW_A_BYTES = (TC_M / 8) * DW_A_STRIDE;   // 33024
@@ -585,7 +773,7 @@ struct DwTcArgs {
   unsigned* error;
 };
 
-__global__ void __launch_bounds__(TC_THREADS, 1) k_dw_tc(DwTcArgs P) {
+__global__ void __launch_bounds__(DW_THREADS, 1) k_dw_tc(DwTcArgs P) {
   extern __shared__ __align__(1024) unsigned char tc_smem[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(tc_smem + DW_BAR_OFF);  // MMAs of buffer 0, 1 done
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tc_smem + DW_BAR_OFF + 32);
@@ -609,8 +797,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_dw_tc(DwTcArgs P) {
   const uint32_t tmem = *tmem_slot, bar0 = smem_u32(bars), base = smem_u32(tc_smem);
   const float* dY = P.dY + layer * P.stride;
   const float* X = ((layer & 1) ? P.z : P.h) + (layer >> 1) * P.stride + half * DW_N;
-  constexpr int kA = TC_N * (TC_M / 8) / TC_THREADS;                              // 4 dY elements per thread
-  constexpr int kB = (TC_ROWS * (DW_N / 8) + TC_THREADS - 1) / TC_THREADS;        // 3 X elements
+  constexpr int kA = TC_N * (TC_M / 8) / DW_THREADS;                              // 4 dY elements per thread
+  constexpr int kB = (TC_ROWS * (DW_N / 8) + DW_THREADS - 1) / DW_THREADS;        // 3 X elements
   float bsum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   bool ok = true;
   int n = 0;  // tiles issued
@@ -620,7 +808,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_dw_tc(DwTcArgs P) {
     float4 a[kA][2], b[kB][2];
 #pragma unroll
     for (int u = 0; u < kA; ++u) {
-      const int e = tid + u * TC_THREADS, r = e / (TC_M / 8), c = e % (TC_M / 8);
+      const int e = tid + u * DW_THREADS, r = e / (TC_M / 8), c = e % (TC_M / 8);
       a[u][0] = a[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (r < cnt) {
         const float4* src = reinterpret_cast<const float4*>(dY + (int64_t)(q0 + r) * TC_M + 8 * c);
@@ -630,7 +818,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_dw_tc(DwTcArgs P) {
     }
 #pragma unroll
     for (int u = 0; u < kB; ++u) {
-      const int e = tid + u * TC_THREADS, r = e / (DW_N / 8), c = e % (DW_N / 8);
+      const int e = tid + u * DW_THREADS, r = e / (DW_N / 8), c = e % (DW_N / 8);
       const int q = q0 - 2 + r;
       b[u][0] = b[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (r < TC_ROWS && q >= lo && q < lo + P.seq_len) {
@@ -647,7 +835,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_dw_tc(DwTcArgs P) {
     unsigned char* sB = sA + DW_A_BYTES;
 #pragma unroll
     for (int u = 0; u < kA; ++u) {
-      const int e = tid + u * TC_THREADS, r = e / (TC_M / 8), c = e % (TC_M / 8);
+      const int e = tid + u * DW_THREADS, r = e / (TC_M / 8), c = e % (TC_M / 8);
       const float4 f = a[u][0], g = a[u][1];
       bsum[0] += f.x, bsum[1] += f.y, bsum[2] += f.z, bsum[3] += f.w;
       bsum[4] += g.x, bsum[5] += g.y, bsum[6] += g.z, bsum[7] += g.w;
@@ -656,7 +844,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_dw_tc(DwTcArgs P) {
     }
 #pragma unroll
     for (int u = 0; u < kB; ++u) {
-      const int e = tid + u * TC_THREADS, r = e / (DW_N / 8), c = e % (DW_N / 8);
+      const int e = tid + u * DW_THREADS, r = e / (DW_N / 8), c = e % (DW_N / 8);
       if (r >= TC_ROWS) break;
       const float4 f = b[u][0], g = b[u][1];
       *reinterpret_cast<uint4*>(sB + c * DW_B_STRIDE + r * 16) =
@@ -695,7 +883,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_dw_tc(DwTcArgs P) {
     // warps w and w + 4, ..: TMEM lanes 32 (w % 4) ..; 20 pieces of 16 columns over 4 warps
     const int m = (warp & 3) * 32 + lane;
     float* dW = P.g + layer * P.gstride + (int64_t)m * TC_K + half * DW_N;
-    for (int piece = warp >> 2; piece < TC_TAPS * (DW_N / 16); piece += TC_THREADS / 128) {
+    for (int piece = warp >> 2; piece < TC_TAPS * (DW_N / 16); piece += DW_THREADS / 128) {
       uint32_t v[16];
       tmem_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(piece * 16), v);
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -720,7 +908,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_dw_tc(DwTcArgs P) {
   if (ok && n > 0 && half == 0 && tid < TC_M) {
     const float* red = reinterpret_cast<const float*>(tc_smem);
     float v = 0.f;
-    for (int w = 0; w < TC_THREADS / 32; ++w) v += red[w * TC_M + tid];
+    for (int w = 0; w < DW_THREADS / 32; ++w) v += red[w * TC_M + tid];
     atomicAdd(P.g + layer * P.gstride + (int64_t)TC_M * TC_K + tid, v);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -798,19 +986,26 @@ __global__ void __launch_bounds__(kThreads) k_conv_dw(DwArgs P) {
       }
 }
 
-// db[m] += sum_q dY[q][m]
-__global__ void k_bias_grad(const float* __restrict__ dY, int npos, int M, float* __restrict__ db) {
-  const int m = blockIdx.x;
-  float s = 0.f;
-  for (int q = threadIdx.x; q < npos; q += blockDim.x) s += dY[(int64_t)q * M + m];
+// db[m] += sum_q dY[q][m]: a block takes kBiasRows positions, its threads the
+// channels (rows read whole), and adds its partial sums.
+constexpr int kBiasRows = 128;
+__global__ void __launch_bounds__(256) k_bias_grad(const float* __restrict__ dY, int npos, int M, float* __restrict__ db) {
   __shared__ float red[256];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+  const int q0 = blockIdx.x * kBiasRows, q1 = min(npos, q0 + kBiasRows);
+  const int per = M < 256 ? 256 / M : 1;  // rows read at a time
+  for (int m0 = 0; m0 < M; m0 += 256) {
+    const int row = M < 256 ? threadIdx.x / M : 0, m = M < 256 ? threadIdx.x - row * M : m0 + threadIdx.x;
+    float s = 0.f;
+    if (row < per && m < M)
+      for (int q = q0 + row; q < q1; q += per) s += dY[(int64_t)q * M + m];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    if (row == 0 && m < M) {
+      for (int r = 1; r < per; ++r) s += red[r * M + m];
+      atomicAdd(db + m, s);
+    }
     __syncthreads();
   }
-  if (threadIdx.x == 0) db[m] += red[0];
 }
 
 // Sum of the mask weights, into acc[0] (acc zeroed before).
@@ -869,19 +1064,29 @@ __global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float
   }
 }
 
-// BF16 copy of one layer's weights W[o][t][i] and of its per-tap transpose
-// WT[i][t][o] (the operand of the input-gradient pass).
-__global__ void k_weights_bf16(const float* __restrict__ W, int Co, int taps, int Ci,
-                               __nv_bfloat16* __restrict__ Wb, __nv_bfloat16* __restrict__ WTb) {
-  const int64_t n = (int64_t)Co * taps * Ci;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int o = (int)(e / ((int64_t)taps * Ci));
-    const int t = (int)((e / Ci) % taps);
-    const int i = (int)(e % Ci);
-    const __nv_bfloat16 b = __float2bfloat16_rn(W[e]);
-    Wb[e] = b;
-    if (WTb) WTb[((int64_t)i * taps + t) * Co + o] = b;
+// BF16 copies of every layer's weights W[o][t][i] (blockIdx.y: layer) and of the
+// per-tap transposes WT[i][t][o] (the operands of the input-gradient pass). The
+// residual blocks' layers of the tensor-core path are laid out as that operand's
+// shared-memory image, tap by tap: [t][k / 8][m][k % 8] with (m, k) = (o, i) and (i, o).
+struct LayerDev {
+  int Co, taps, Ci, image;
+  int64_t w_off, wb_off;
+};
+
+__global__ void k_weights_bf16(const float* __restrict__ w, const LayerDev* __restrict__ layers,
+                               __nv_bfloat16* __restrict__ wb, __nv_bfloat16* __restrict__ wtb) {
+  const LayerDev L = layers[blockIdx.y];
+  const int n = L.Co * L.taps * L.Ci;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    const int i = e % L.Ci, ot = e / L.Ci, t = ot % L.taps, o = ot / L.taps;
+    const __nv_bfloat16 b = __float2bfloat16_rn(w[L.w_off + e]);
+    if (L.image) {
+      wb[L.wb_off + (((t * (L.Ci / 8) + i / 8) * L.Co + o) * 8 + i % 8)] = b;
+      wtb[L.wb_off + (((t * (L.Co / 8) + o / 8) * L.Ci + i) * 8 + o % 8)] = b;
+    } else {
+      wb[L.wb_off + e] = b;
+      wtb[L.wb_off + ((int64_t)i * L.taps + t) * L.Co + o] = b;
+    }
   }
 }
 
@@ -901,6 +1106,7 @@ struct rpk_net {
   int64_t nparams = 0, nwb = 0;
   float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
   __nv_bfloat16 *wb = nullptr, *wtb = nullptr;
+  LayerDev* layers_dev = nullptr;
   int64_t step = 0;
   // activation workspace for up to cap_q coarse positions
   int64_t cap_q = 0;
@@ -916,7 +1122,7 @@ struct rpk_net {
   int cap_seq = 0;
   int4* tiles = nullptr;       // ragged tensor-core tiles (q0, count, start, length)
   int ntiles = 0, cap_tiles = 0;
-  unsigned* tc_error = nullptr;  // set by k_conv_tc when a wait gives up
+  unsigned* tc_error = nullptr;  // set by the tcgen05 kernels when a wait gives up
   int nsm = 0;
   bool tc = false;             // the tensor-core path serves the block convolutions
 };
@@ -975,12 +1181,7 @@ rpk_status tc_status(rpk_net* N) {
 }
 
 rpk_status refresh_bf16(rpk_net* N) {
-  for (const auto& L : N->layers) {
-    const int64_t n = (int64_t)L.Co * L.taps * L.Ci;
-    const int blocks = (int)std::min<int64_t>(1024, (n + 255) / 256);
-    k_weights_bf16<<<blocks, 256, 0, N->stream>>>(N->w + L.w_off, L.Co, L.taps, L.Ci,
-                                                   N->wb + L.wb_off, N->wtb + L.wb_off);
-  }
+  k_weights_bf16<<<dim3(64, (unsigned)N->layers.size()), 256, 0, N->stream>>>(N->w, N->layers_dev, N->wb, N->wtb);
   RPK_CUDA(cudaGetLastError());
   return RPK_OK;
 }
@@ -988,20 +1189,18 @@ rpk_status refresh_bf16(rpk_net* N) {
 rpk_status conv(rpk_net* N, const __nv_bfloat16* A, int M, int taps, int Kc, int sgn,
                 const float* X, int relu_in, float* out, const float* bias, const float* res,
                 const float* mask, int64_t nq, int seq_len, const int2* qseq = nullptr) {
-  // 16-byte operands: the weights and inputs for cp.async, the output and
-  // residual rows for the epilogue's bulk copies
-  const bool aligned = (((uintptr_t)A | (uintptr_t)X | (uintptr_t)out | (uintptr_t)res) & 15) == 0;
-  if (N->tc && M == TC_M && Kc == TC_KC && taps == TC_TAPS && aligned && nq > 0) {
-    TcArgs T{A, X, out, bias, res, mask, nullptr, 0, seq_len, 0, sgn, relu_in, N->tc_error};
-    if (qseq) {
-      T.tiles = N->tiles;
-      T.ntiles = N->ntiles;
-    } else {
-      T.tiles_per_seq = (seq_len + TC_N - 1) / TC_N;
-      T.ntiles = (int)(nq / seq_len) * T.tiles_per_seq;
-    }
-    const int grid = std::max(1, std::min(T.ntiles, N->nsm));
-    k_conv_tc<<<grid, TC_THREADS, TC_SMEM, N->stream>>>(T);
+  // one tap, 8-byte input pairs, weights that fit the default shared memory
+  const int mt = M <= 16 ? 1 : 8;
+  const size_t smem = (size_t)mt * 16 * ((Kc + 15) / 16 * 16 + kPadK) * 2;
+  if (taps == 1 && !res && Kc % 2 == 0 && ((uintptr_t)X & 7) == 0 && smem <= 48 * 1024) {
+    Conv1Args P{A, X, out, bias, mask, M, Kc, relu_in, (int)nq};
+    const int64_t want = (nq + 16 * (kConv1Threads / 32) - 1) / (16 * (kConv1Threads / 32));
+    const dim3 grid((unsigned)std::min<int64_t>(want, 4 * (int64_t)std::max(N->nsm, 1)),
+                    (unsigned)((M + mt * 16 - 1) / (mt * 16)));
+    if (mt == 1)
+      k_conv1<1><<<grid, kConv1Threads, smem, N->stream>>>(P);
+    else
+      k_conv1<8><<<grid, kConv1Threads, smem, N->stream>>>(P);
     RPK_CUDA(cudaGetLastError());
     return RPK_OK;
   }
@@ -1012,14 +1211,40 @@ rpk_status conv(rpk_net* N, const __nv_bfloat16* A, int M, int taps, int Kc, int
   return RPK_OK;
 }
 
+// A residual block (or its input gradient) on the tensor cores. Launched so
+// that its CTAs may start where the previous kernel leaves SMs free.
+rpk_status block_tc(rpk_net* N, BlockArgs T, int64_t nq, int seq_len, const int2* qseq) {
+  T.error = N->tc_error;
+  if (qseq) {
+    T.tiles = N->tiles;
+    T.ntiles = N->ntiles;
+  } else {
+    T.seq_len = seq_len;
+    T.tiles_per_seq = (seq_len + TC_OUT - 1) / TC_OUT;
+    T.ntiles = (int)(nq / seq_len) * T.tiles_per_seq;
+  }
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)std::max(1, std::min(T.ntiles, N->nsm)));
+  c.blockDim = dim3(TC_THREADS);
+  c.dynamicSmemBytes = TC_SMEM;
+  c.stream = N->stream;
+  cudaLaunchAttribute a{};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &a;
+  c.numAttrs = 1;
+  RPK_CUDA(cudaLaunchKernelEx(&c, k_block_tc, T));
+  return RPK_OK;
+}
+
 rpk_status conv_dw(rpk_net* N, const float* dY, int M, const float* X, int Kc, int taps,
                    int relu_in, float* dW, int64_t nq, int seq_len) {
   // positions per block: enough blocks for about four per SM over the
-  // (output x input) tiles, between 128 and 2048 positions, a multiple of BK
+  // (output x input) tiles, between BK and 2048 positions, a multiple of BK
   const int64_t tiles = (int64_t)((taps * Kc + BN - 1) / BN) * ((M + BM - 1) / BM);
   const int64_t want = std::max<int64_t>(1, 4 * (int64_t)std::max(N->nsm, 1) / std::max<int64_t>(tiles, 1));
   int64_t qc = (nq + want - 1) / want;
-  qc = std::min<int64_t>(2048, std::max<int64_t>(128, (qc + BK - 1) / BK * BK));
+  qc = std::min<int64_t>(2048, std::max<int64_t>(BK, (qc + BK - 1) / BK * BK));
   const int qchunk = (int)qc;
   DwArgs P{dY, X, dW, M, Kc, taps, relu_in, (int)nq, seq_len, qchunk};
   const dim3 grid((unsigned)((taps * Kc + BN - 1) / BN), (unsigned)((M + BM - 1) / BM),
@@ -1029,9 +1254,14 @@ rpk_status conv_dw(rpk_net* N, const float* dY, int M, const float* X, int Kc, i
   return RPK_OK;
 }
 
+void bias_grad(rpk_net* N, const float* dY, int64_t nq, int M, float* db) {
+  k_bias_grad<<<(unsigned)((nq + kBiasRows - 1) / kBiasRows), 256, 0, N->stream>>>(dY, (int)nq, M, db);
+}
+
 // Forward pass over nq coarse positions (sequences of Lq positions each, or the
-// sequences described by qseq); keeps the activations.
-rpk_status forward(rpk_net* N, const float* x, int64_t nq, int Lq, const int2* qseq, float* y) {
+// sequences described by qseq); keeps the blocks' inputs and, for training, the
+// activations between their convolutions.
+rpk_status forward(rpk_net* N, const float* x, int64_t nq, int Lq, const int2* qseq, float* y, bool train) {
   rpk_status st = ensure_workspace(N, nq);
   if (st != RPK_OK) return st;
   const int64_t stride = nq * N->width;
@@ -1045,6 +1275,12 @@ rpk_status forward(rpk_net* N, const float* x, int64_t nq, int Lq, const int2* q
     float* hb = N->act + b * stride;
     float* z0 = N->act + (N->nblocks + 1 + b) * stride;
     float* hn = N->act + (b + 1) * stride;
+    if (N->tc) {
+      st = block_tc(N, BlockArgs{N->wb + c0.wb_off, N->wb + c1.wb_off, hb, train ? z0 : nullptr, hn, N->w + c0.b_off,
+                                 N->w + c1.b_off, nullptr, nullptr, nullptr, 0, 0, 0, +1, 1, nullptr},
+                    nq, Lq, qseq);
+      continue;
+    }
     st = conv(N, N->wb + c0.wb_off, N->width, K5, N->width, +1, hb, 1, z0, N->w + c0.b_off,
               nullptr, nullptr, nq, Lq, qseq);
     if (st == RPK_OK)
@@ -1077,7 +1313,7 @@ rpk_status block_grads(rpk_net* N, int64_t nq, int Lq) {
     P.ntiles = (int)(nq / Lq) * P.tiles_per_seq;
     // one CTA per SM: as many shares of the tiles as the SMs hold (layer, half) pairs
     P.splits = std::max(1, std::min(P.ntiles, N->nsm / (2 * nl)));
-    k_dw_tc<<<2 * nl * P.splits, TC_THREADS, DW_SMEM, N->stream>>>(P);
+    k_dw_tc<<<2 * nl * P.splits, DW_THREADS, DW_SMEM, N->stream>>>(P);
     RPK_CUDA(cudaGetLastError());
     return RPK_OK;
   }
@@ -1087,7 +1323,7 @@ rpk_status block_grads(rpk_net* N, int64_t nq, int Lq) {
     const auto& L = N->layers[1 + l];
     rpk_status st = conv_dw(N, dY, W, X, W, K5, 1, N->g + L.w_off, nq, Lq);
     if (st != RPK_OK) return st;
-    k_bias_grad<<<W, 256, 0, N->stream>>>(dY, (int)nq, W, N->g + L.b_off);
+    bias_grad(N, dY, nq, W, N->g + L.b_off);
   }
   RPK_CUDA(cudaGetLastError());
   return RPK_OK;
@@ -1106,7 +1342,7 @@ rpk_status backward(rpk_net* N, const float* x, const float* dy, int nseq, int L
   const auto& head = N->layers.back();
   const float* hB = N->act + N->nblocks * stride;
   rpk_status st = conv_dw(N, dy, R * N->cout, hB, W, 1, 1, N->g + head.w_off, nq, Lq);
-  k_bias_grad<<<R * N->cout, 256, 0, N->stream>>>(dy, (int)nq, R * N->cout, N->g + head.b_off);
+  bias_grad(N, dy, nq, R * N->cout, N->g + head.b_off);
   // d relu(h_B) = W_head^T dy, then mask by h_B > 0
   if (st == RPK_OK)
     st = conv(N, N->wtb + head.wb_off, W, 1, R * N->cout, -1, dy, 0, slot(2 * N->nblocks), nullptr, nullptr, hB, nq, Lq);
@@ -1117,6 +1353,12 @@ rpk_status backward(rpk_net* N, const float* x, const float* dy, int nseq, int L
     const float* z0 = N->act + (N->nblocks + 1 + b) * stride;
     const float* dh = slot(2 * b + 2);  // z1 = conv(relu(z0)); d z1 = dh
     float* dz = slot(2 * b + 1);        // z0 = conv(relu(h_b)); d z0
+    if (N->tc) {
+      st = block_tc(N, BlockArgs{N->wtb + c1.wb_off, N->wtb + c0.wb_off, dh, dz, slot(2 * b), nullptr, nullptr, z0, hb,
+                                 nullptr, 0, 0, 0, -1, 0, nullptr},
+                    nq, Lq, nullptr);
+      continue;
+    }
     st = conv(N, N->wtb + c1.wb_off, W, K5, W, -1, dh, 0, dz, nullptr, nullptr, z0, nq, Lq);
     // d h_b = dh + (W0^T dz) masked by h_b > 0
     if (st == RPK_OK)
@@ -1126,7 +1368,7 @@ rpk_status backward(rpk_net* N, const float* x, const float* dy, int nseq, int L
   if (st != RPK_OK) return st;
   const auto& lift = N->layers[0];
   st = conv_dw(N, slot(0), W, x, R * N->cin, 1, 0, N->g + lift.w_off, nq, Lq);
-  k_bias_grad<<<W, 256, 0, N->stream>>>(slot(0), (int)nq, W, N->g + lift.b_off);
+  bias_grad(N, slot(0), nq, W, N->g + lift.b_off);
   RPK_CUDA(cudaGetLastError());
   return st;
 }
@@ -1179,16 +1421,21 @@ rpk_status rpk_net_create(int cin, int cout, int width, int nblocks, uint64_t se
   if (st == RPK_OK) st = net_alloc((void**)&N->wtb, sizeof(__nv_bfloat16) * N->nwb);
   if (st == RPK_OK) st = net_alloc((void**)&N->loss, 2 * sizeof(double));
   if (st == RPK_OK) st = net_alloc((void**)&N->tc_error, sizeof(unsigned));
+  if (st == RPK_OK) st = net_alloc((void**)&N->layers_dev, sizeof(LayerDev) * N->layers.size());
   if (st == RPK_OK) {
     cudaDeviceGetAttribute(&N->nsm, cudaDevAttrMultiProcessorCount, N->device);
     N->tc = width == TC_M &&
-            cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM) ==
+            cudaFuncSetAttribute(k_block_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM) ==
                 cudaSuccess &&
             cudaFuncSetAttribute(k_dw_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DW_SMEM) == cudaSuccess;
     cudaGetLastError();
   }
+  std::vector<LayerDev> ld;
+  for (const auto& L : N->layers) ld.push_back({L.Co, L.taps, L.Ci, N->tc && L.taps == TC_TAPS, L.w_off, L.wb_off});
   cudaError_t err = cudaSuccess;
   if (st == RPK_OK)
+    err = cudaMemcpyAsync(N->layers_dev, ld.data(), sizeof(LayerDev) * ld.size(), cudaMemcpyHostToDevice, N->stream);
+  if (st == RPK_OK && err == cudaSuccess)
     err = cudaMemcpyAsync(N->w, w.data(), sizeof(float) * N->nparams, cudaMemcpyHostToDevice, N->stream);
   if (st == RPK_OK && err == cudaSuccess) err = cudaMemsetAsync(N->m, 0, sizeof(float) * N->nparams, N->stream);
   if (st == RPK_OK && err == cudaSuccess) err = cudaMemsetAsync(N->v, 0, sizeof(float) * N->nparams, N->stream);
@@ -1208,7 +1455,8 @@ void rpk_net_destroy(rpk_net* N) {
   if (!N) return;
   cudaStreamSynchronize(N->stream);
   void* p[] = {N->w,    N->g,       N->m,     N->v,    N->wb,     N->wtb,  N->act,
-               N->work, N->headout, N->dybuf, N->loss, N->qseq, N->starts, N->tiles, N->tc_error};
+               N->work, N->headout, N->dybuf, N->loss, N->qseq, N->starts, N->tiles, N->tc_error,
+               N->layers_dev};
   for (void* q : p)
     if (q) cudaFree(q);
   delete N;
@@ -1237,7 +1485,7 @@ rpk_status rpk_net_forward(rpk_net* N, const float* x, int nseq, int len, float*
   if (!N || !x || !y) return rpk::fail(RPK_ERR_ARG, "NULL argument");
   if (nseq < 1 || len < R || len % R) return rpk::fail(RPK_ERR_ARG, "len must be a positive multiple of 4");
   RPK_CUDA(cudaSetDevice(N->device));
-  return forward(N, x, (int64_t)nseq * (len / R), len / R, nullptr, y);
+  return forward(N, x, (int64_t)nseq * (len / R), len / R, nullptr, y, false);
 }
 
 rpk_status rpk_net_forward_ragged(rpk_net* N, const float* x, int nseq, const int* lens, float* y) {
@@ -1265,11 +1513,11 @@ rpk_status rpk_net_forward_ragged(rpk_net* N, const float* x, int nseq, const in
   }
   RPK_CUDA(cudaMemcpyAsync(N->starts, starts.data(), sizeof(int) * (nseq + 1),
                            cudaMemcpyHostToDevice, N->stream));
-  // tensor-core tiles: 128 positions of one sequence each
+  // tensor-core tiles: TC_OUT positions of one sequence each
   std::vector<int4> tiles;
   for (int s = 0; s < nseq; ++s)
-    for (int q = starts[s]; q < starts[s + 1]; q += TC_N)
-      tiles.push_back(make_int4(q, std::min(TC_N, starts[s + 1] - q), starts[s], starts[s + 1] - starts[s]));
+    for (int q = starts[s]; q < starts[s + 1]; q += TC_OUT)
+      tiles.push_back(make_int4(q, std::min(TC_OUT, starts[s + 1] - q), starts[s], starts[s + 1] - starts[s]));
   if ((int)tiles.size() > N->cap_tiles) {
     cudaFree(N->tiles);
     N->tiles = nullptr;
@@ -1283,7 +1531,7 @@ rpk_status rpk_net_forward_ragged(rpk_net* N, const float* x, int nseq, const in
                            N->stream));
   k_fill_qseq<<<nseq, 256, 0, N->stream>>>(N->starts, N->qseq);
   RPK_CUDA(cudaGetLastError());
-  st = forward(N, x, nq, 0, N->qseq, y);
+  st = forward(N, x, nq, 0, N->qseq, y, false);
   // the host tables are read before they go away
   if (st == RPK_OK) RPK_CUDA(cudaStreamSynchronize(N->stream));
   if (st == RPK_OK) st = tc_status(N);
@@ -1299,7 +1547,7 @@ rpk_status rpk_net_loss_grad(rpk_net* N, const float* x, const float* target, co
   rpk_status st = ensure_training(N, nq);
   if (st != RPK_OK) return st;
   float* y = N->headout;
-  st = forward(N, x, nq, len / R, nullptr, y);
+  st = forward(N, x, nq, len / R, nullptr, y, true);
   if (st != RPK_OK) return st;
   RPK_CUDA(cudaMemsetAsync(N->loss, 0, 2 * sizeof(double), N->stream));
   const int64_t npts = (int64_t)nseq * len;
