@@ -195,10 +195,13 @@ __global__ void __launch_bounds__(kConv1Threads) k_conv1(Conv1Args P) {
   extern __shared__ __align__(16) uint16_t c1_smem[];
   const int Kp = (P.K + 15) / 16 * 16, ld = Kp + kPadK;
   const int m0 = blockIdx.y * kMT * 16;
-  for (int e = threadIdx.x; e < kMT * 16 * ld; e += kConv1Threads) {
-    const int m = e / ld, k = e - m * ld;
-    const uint16_t* src = reinterpret_cast<const uint16_t*>(P.A);
-    c1_smem[e] = m0 + m < P.M && k < P.K ? src[(int64_t)(m0 + m) * P.K + k] : (uint16_t)0;
+  // a warp takes whole rows of weights, a word of two at a time (K is even, so words are
+  // aligned)
+#pragma unroll 4
+  for (int m = threadIdx.x >> 5; m < kMT * 16; m += kConv1Threads / 32) {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(P.A + (int64_t)(m0 + m) * P.K);
+    for (int k = threadIdx.x & 31; k < ld / 2; k += 32)
+      reinterpret_cast<uint32_t*>(c1_smem)[m * (ld / 2) + k] = m0 + m < P.M && 2 * k < P.K ? src[k] : 0u;
   }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -988,7 +991,7 @@ __global__ void __launch_bounds__(kThreads) k_conv_dw(DwArgs P) {
 
 // db[m] += sum_q dY[q][m]: a block takes kBiasRows positions, its threads the
 // channels (rows read whole), and adds its partial sums.
-constexpr int kBiasRows = 128;
+constexpr int kBiasRows = 32;
 __global__ void __launch_bounds__(256) k_bias_grad(const float* __restrict__ dY, int npos, int M, float* __restrict__ db) {
   __shared__ float red[256];
   const int q0 = blockIdx.x * kBiasRows, q1 = min(npos, q0 + kBiasRows);
@@ -997,6 +1000,7 @@ __global__ void __launch_bounds__(256) k_bias_grad(const float* __restrict__ dY,
     const int row = M < 256 ? threadIdx.x / M : 0, m = M < 256 ? threadIdx.x - row * M : m0 + threadIdx.x;
     float s = 0.f;
     if (row < per && m < M)
+#pragma unroll 8
       for (int q = q0 + row; q < q1; q += per) s += dY[(int64_t)q * M + m];
     red[threadIdx.x] = s;
     __syncthreads();
