@@ -66,12 +66,12 @@ __device__ __forceinline__ V collide_emit(const StepConst<Real>& K, const V (&h)
   return collide_relax<Real, kPaper>(K, m, e, [&](int q) { return h[q]; }, emit);
 }
 
-// One point: the populations go to out[q * n3].
+// One point: population q goes to cell of the plane out + q * n3.
 template <typename Store, typename Real, bool kPaper = false>
 __device__ __forceinline__ Real collide_point(const StepConst<Real>& K, const Real (&h)[kQ], Real e,
-                                              Store* __restrict__ out, Mom<Real>& m) {
+                                              Store* __restrict__ out, unsigned cell, Mom<Real>& m) {
   const int64_t n3 = K.n3;
-  auto put = [&](int q, Real v) { out[(int64_t)q * n3] = from_real<Store, Real>(v); };
+  auto put = [&](int q, Real v) { (out + (int64_t)q * n3)[cell] = from_real<Store, Real>(v); };
   if constexpr (kShells<Store>)
     return collide_shells<Real, kPaper>(K, h, e, put, m);
   else
@@ -113,7 +113,8 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 ? 5 : 1)
   gather<Store, Real, kPull, kBC>(pin, ghost, K, P, h, wcol);
   Mom<Real> m;
   const Real es = collide_point<Store, Real, kPaper>(K, h, e_in[p],
-                                             pout + (int64_t)(P.s * kQ) * K.n3 + P.cell, m);
+                                             pout + (int64_t)(P.s * kQ) * K.n3,
+                                             (unsigned)P.cell, m);
   e_out[p] = es;
   drho_out[p] = m.drho;
   const int64_t npts = 2 * K.n3;
@@ -171,10 +172,11 @@ __global__ void __launch_bounds__(128, sizeof(Store) == 4 ? 3 : 4)
   F2 h[kQ];
   gather_pair<Store>(reinterpret_cast<const Word*>(pin), K, s, i, y, z, h);
   Mom<F2> m;
-  Word* out = reinterpret_cast<Word*>(pout) + (int64_t)(s * kQ) * n3p + cellp;
+  Word* out = reinterpret_cast<Word*>(pout) + (int64_t)(s * kQ) * n3p;
+  const unsigned cell = (unsigned)cellp;
   const F2 es = collide_emit<float, kPaper>(
       K, h, F2(reinterpret_cast<const float2*>(e_in)[pp]),
-      [&](int q, F2 v) { out[(int64_t)q * n3p] = IO::from_f2(v); }, m);
+      [&](int q, F2 v) { (out + (int64_t)q * n3p)[cell] = IO::from_f2(v); }, m);
   reinterpret_cast<float2*>(e_out)[pp] = es.v;
   reinterpret_cast<float2*>(drho_out)[pp] = m.drho.v;
   float2* u2 = reinterpret_cast<float2*>(u_out);
@@ -217,11 +219,12 @@ __global__ void __launch_bounds__(128, kPaper ? 4 : 5)
     for (int q = 0; q < kQ; ++q) h[q] = IO::to_f2(hw[q]);
     raw_moments(h, m);
   }
-  unsigned* out = reinterpret_cast<unsigned*>(pout) + (int64_t)(s * kQ) * n3p + cellp;
+  unsigned* out = reinterpret_cast<unsigned*>(pout) + (int64_t)(s * kQ) * n3p;
+  const unsigned cell = (unsigned)cellp;
   const F2 es = collide_relax<float, kPaper>(
       K, m, F2(reinterpret_cast<const float2*>(e_in)[pp]),
       [&](int q) { return word_to_f2_here<Store>(hw[q]); },
-      [&](int q, F2 v) { out[(int64_t)q * n3p] = IO::from_f2(v); });
+      [&](int q, F2 v) { (out + (int64_t)q * n3p)[cell] = IO::from_f2(v); });
   reinterpret_cast<float2*>(e_out)[pp] = es.v;
   reinterpret_cast<float2*>(drho_out)[pp] = m.drho.v;
   float2* u2 = reinterpret_cast<float2*>(u_out);

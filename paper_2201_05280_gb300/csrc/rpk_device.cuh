@@ -529,9 +529,9 @@ __device__ __forceinline__ void gather(const Store* __restrict__ pin,
                                        const Real* __restrict__ wcol = nullptr) {
   const int64_t n3 = K.n3;
   if constexpr (!kPull) {
-    const Store* base = pin + (int64_t)(P.s * kQ) * n3 + P.cell;
+    const unsigned cell = (unsigned)P.cell;
 #pragma unroll
-    for (int q = 0; q < kQ; ++q) h[q] = to_real<Store, Real>(base[(int64_t)q * n3]);
+    for (int q = 0; q < kQ; ++q) h[q] = to_real<Store, Real>((pin + (int64_t)(P.s * kQ + q) * n3)[cell]);
   } else {
     const int nx = K.nx, ny = K.ny, nz = K.nz;
     int xw[5], yw[5], zw[5];
@@ -539,8 +539,10 @@ __device__ __forceinline__ void gather(const Store* __restrict__ pin,
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
       xw[k] = wrap_near(P.x + k - 2, nx);
-      yw[k] = wrap_near(P.y + k - 2, ny);
-      zw[k] = wrap_near(P.z + k - 2, nz);
+      // cell offsets of the row and the plane: 32 bits (a sublattice holds fewer
+      // than 2^31 cells), added to a base that is the same for the whole block
+      yw[k] = wrap_near(P.y + k - 2, ny) * nx;
+      zw[k] = wrap_near(P.z + k - 2, nz) * (ny * nx);
       xin[k] = (P.x + k - 2 >= 0) && (P.x + k - 2 < nx);
       yin[k] = (P.y + k - 2 >= 0) && (P.y + k - 2 < ny);
     }
@@ -553,7 +555,7 @@ __device__ __forceinline__ void gather(const Store* __restrict__ pin,
     const bool yinhp = s ? yin[2] : yin[1], yinhm = s ? yin[3] : yin[2];
     const Store* same = pin + (int64_t)(s * kQ) * n3;
     const Store* other = pin + (int64_t)((1 - s) * kQ) * n3;
-    h[0] = to_real<Store, Real>(same[P.cell]);
+    h[0] = to_real<Store, Real>(same[(unsigned)P.cell]);
     static_for<kQ - 1>([&](auto qc) {
       constexpr int q = decltype(qc)::value + 1;
       constexpr Vel2 v = vel2(q);
@@ -576,7 +578,7 @@ __device__ __forceinline__ void gather(const Store* __restrict__ pin,
         insy = yin[2 - v.y / 2];
         base = same;
       }
-      const int64_t cell = ((int64_t)zs * ny + ys) * nx + xs;
+      const unsigned cell = (unsigned)(zs + ys + xs);
       if constexpr (kBC == 1) {
         if (!insx) {
           h[q] = ghost[(v.x > 0 ? 0 : kGhostStride) + q];
@@ -601,7 +603,7 @@ __device__ __forceinline__ void gather(const Store* __restrict__ pin,
           return;
         }
       }
-      h[q] = to_real<Store, Real>(base[(int64_t)q * n3 + cell]);
+      h[q] = to_real<Store, Real>((base + (int64_t)q * n3)[cell]);
     });
   }
 }

@@ -61,13 +61,16 @@ __device__ __forceinline__ void gather_pair(const typename PairIO<Store>::Word* 
                                             const StepConst<float>& K, int s, int i, int y, int z,
                                             F2 (&h)[kQ]) {
   using IO = PairIO<Store>;
-  const int nx = K.nx, ny = K.ny, nz = K.nz, nxp = nx >> 1;
+  const int ny = K.ny, nz = K.nz, nxp = K.nx >> 1;
   const int64_t n3p = K.n3 >> 1;
+  // word offsets of the rows y + k - 2 and planes z + k - 2 from the plane's start
+  // and the array's: 32 bits (a sublattice holds fewer than 2^31 cells), added to
+  // a base that is the same for the whole block
   int yw[5], zw[5];
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
-    yw[k] = wrap_near(y + k - 2, ny);
-    zw[k] = wrap_near(z + k - 2, nz);
+    yw[k] = wrap_near(y + k - 2, ny) * nxp;
+    zw[k] = wrap_near(z + k - 2, nz) * (ny * nxp);
   }
   // pair columns i - 1, i, i + 1
   const int ip[3] = {i == 0 ? nxp - 1 : i - 1, i, i == nxp - 1 ? 0 : i + 1};
@@ -77,7 +80,7 @@ __device__ __forceinline__ void gather_pair(const typename PairIO<Store>::Word* 
   const int zhp = s ? zw[2] : zw[1], zhm = s ? zw[3] : zw[2];
   const typename IO::Word* same = w + (int64_t)(s * kQ) * n3p;
   const typename IO::Word* other = w + (int64_t)((1 - s) * kQ) * n3p;
-  h[0] = IO::to_f2(same[(((int64_t)z * ny + y) * nx >> 1) + i]);
+  h[0] = IO::to_f2(same[(unsigned)(zw[2] + yw[2] + i)]);
   static_for<kQ - 1>([&](auto qc) {
     constexpr int q = decltype(qc)::value + 1;
     constexpr Vel2 v = vel2(q);
@@ -93,24 +96,26 @@ __device__ __forceinline__ void gather_pair(const typename PairIO<Store>::Word* 
       zs = zw[2 - v.z / 2];
       base = same;
     }
-    const typename IO::Word* row = base + (int64_t)q * n3p + (((int64_t)zs * ny + ys) * nx >> 1);
+    const typename IO::Word* plane = base + (int64_t)q * n3p;
+    const int r0 = zs + ys;
+    auto row = [&](int col) { return plane[(unsigned)(r0 + col)]; };
     if constexpr (half) {
       // x shift 1 (c > 0, s = 0) or -1 (c < 0, s = 1) straddles; otherwise none
       const bool odd = (v.x > 0) == (s == 0);
       if (odd) {
         const int lo = s == 0 ? ip[0] : ip[1];
-        h[q] = IO::straddle(row[lo], row[lo + 1 == nxp ? 0 : lo + 1]);
+        h[q] = IO::straddle(row(lo), row(lo + 1 == nxp ? 0 : lo + 1));
       } else {
-        h[q] = IO::to_f2(row[ip[1]]);
+        h[q] = IO::to_f2(row(ip[1]));
       }
     } else if constexpr (v.x == 0) {
-      h[q] = IO::to_f2(row[ip[1]]);
+      h[q] = IO::to_f2(row(ip[1]));
     } else if constexpr (v.x == 4 || v.x == -4) {
       // c_x = +-2: the source pair is one column left (+2) or right (-2)
-      h[q] = IO::to_f2(row[ip[v.x > 0 ? 0 : 2]]);
+      h[q] = IO::to_f2(row(ip[v.x > 0 ? 0 : 2]));
     } else {
       // c_x = +-1: straddles columns (i - 1, i) or (i, i + 1)
-      h[q] = v.x > 0 ? IO::straddle(row[ip[0]], row[ip[1]]) : IO::straddle(row[ip[1]], row[ip[2]]);
+      h[q] = v.x > 0 ? IO::straddle(row(ip[0]), row(ip[1])) : IO::straddle(row(ip[1]), row(ip[2]));
     }
   });
 }
@@ -126,13 +131,16 @@ template <typename Store>
 __device__ __forceinline__ void gather_pair_words(const unsigned* __restrict__ w, const StepConst<float>& K,
                                                   int s, int i, int y, int z, unsigned (&hw)[kQ]) {
   static_assert(sizeof(Store) == 2, "pair words of 16-bit storage");
-  const int nx = K.nx, ny = K.ny, nz = K.nz, nxp = nx >> 1;
+  const int ny = K.ny, nz = K.nz, nxp = K.nx >> 1;
   const int64_t n3p = K.n3 >> 1;
+  // word offsets of the rows y + k - 2 and planes z + k - 2 from the plane's start
+  // and the array's: 32 bits (a sublattice holds fewer than 2^31 cells), added to
+  // a base that is the same for the whole block
   int yw[5], zw[5];
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
-    yw[k] = wrap_near(y + k - 2, ny);
-    zw[k] = wrap_near(z + k - 2, nz);
+    yw[k] = wrap_near(y + k - 2, ny) * nxp;
+    zw[k] = wrap_near(z + k - 2, nz) * (ny * nxp);
   }
   const int ip[3] = {i == 0 ? nxp - 1 : i - 1, i, i == nxp - 1 ? 0 : i + 1};
   const int yhp = s ? yw[2] : yw[1], yhm = s ? yw[3] : yw[2];
@@ -140,7 +148,7 @@ __device__ __forceinline__ void gather_pair_words(const unsigned* __restrict__ w
   const unsigned* same = w + (int64_t)(s * kQ) * n3p;
   const unsigned* other = w + (int64_t)((1 - s) * kQ) * n3p;
   auto join = [](unsigned lo, unsigned hi) { return __byte_perm(lo, hi, 0x5432); };
-  hw[0] = same[(((int64_t)z * ny + y) * nx >> 1) + i];
+  hw[0] = same[(unsigned)(zw[2] + yw[2] + i)];
   static_for<kQ - 1>([&](auto qc) {
     constexpr int q = decltype(qc)::value + 1;
     constexpr Vel2 v = vel2(q);
@@ -156,21 +164,23 @@ __device__ __forceinline__ void gather_pair_words(const unsigned* __restrict__ w
       zs = zw[2 - v.z / 2];
       base = same;
     }
-    const unsigned* row = base + (int64_t)q * n3p + (((int64_t)zs * ny + ys) * nx >> 1);
+    const unsigned* plane = base + (int64_t)q * n3p;
+    const int r0 = zs + ys;
+    auto row = [&](int col) { return plane[(unsigned)(r0 + col)]; };
     if constexpr (half) {
       const bool odd = (v.x > 0) == (s == 0);
       if (odd) {
         const int lo = s == 0 ? ip[0] : ip[1];
-        hw[q] = join(row[lo], row[lo + 1 == nxp ? 0 : lo + 1]);
+        hw[q] = join(row(lo), row(lo + 1 == nxp ? 0 : lo + 1));
       } else {
-        hw[q] = row[ip[1]];
+        hw[q] = row(ip[1]);
       }
     } else if constexpr (v.x == 0) {
-      hw[q] = row[ip[1]];
+      hw[q] = row(ip[1]);
     } else if constexpr (v.x == 4 || v.x == -4) {
-      hw[q] = row[ip[v.x > 0 ? 0 : 2]];
+      hw[q] = row(ip[v.x > 0 ? 0 : 2]);
     } else {
-      hw[q] = v.x > 0 ? join(row[ip[0]], row[ip[1]]) : join(row[ip[1]], row[ip[2]]);
+      hw[q] = v.x > 0 ? join(row(ip[0]), row(ip[1])) : join(row(ip[1]), row(ip[2]));
     }
   });
 }
