@@ -23,7 +23,15 @@
 
 namespace rpk {
 
-constexpr int kBatchArrays = 7;  // e, e*/theta, u slot 0, u slot 1, rho - 1, kappa, predictor
+// Shared arrays per tube point: e (e*, corrected e), u slot 0, u slot 1, rho - 1,
+// kappa, predictor, and for FTCS theta_R of the corrector; the backward-Euler solve
+// needs four values per block of kBE points instead. Shared memory that is not
+// asked for stays L1 cache, which bounds the loads in flight: with seven arrays
+// tubes of 4000 cells (224 KB) ran at 13.3 G point steps a second, with six at 15.8
+// (backward Euler); FTCS is bound by its sub-steps.
+// Tube lengths and CTAs per SM are accepted as for seven arrays either way.
+constexpr int kBatchArrays = 6;
+constexpr int kBatchRuleArrays = 7;
 constexpr size_t kBatchSmemLimit = 227 * 1024;
 
 template <typename Real>
@@ -96,8 +104,8 @@ __device__ __forceinline__ void gather_line(const Store* __restrict__ pin, const
 // products of non-negative numbers, with no cancellation however large K is
 // (FP32, K = 400: error 9e-9 rms of phi where the reduction of the assembled
 // matrix has 1.9e-7).
-// In: e (sE), D (sD), kappa (sK). l -> sL, u -> sU, r -> sR, g -> sE (e is read by
-// its own thread only). Out: e in sE.
+// In: e (sE), D (sD), kappa (sK). l -> sL, r -> sR, u -> sE (e is read by its own
+// thread only), g of each block's first and last point -> sG. Out: e in sE.
 constexpr int kBE = 9;
 
 // A row of the elimination: x = r + l x_prev + u x_next, l + u + g = 1.
@@ -124,13 +132,14 @@ __device__ __forceinline__ void be_fold(BeRow<Real>& a, const BeRow<Real>& n) {
 
 template <typename Real>
 __device__ __forceinline__ void be_blocks(const StepConst<Real>& K, int nx, int nthreads, Real* sE, const Real* sD,
-                                          const Real* sK, Real* sL, Real* sU, Real* sR, Real kGl, Real kGh, Real thGl,
+                                          const Real* sK, Real* sL, Real* sR, Real* sG, Real kGl, Real kGh, Real thGl,
                                           Real thGh) {
   const int nb = (nx + kBE - 1) / kBE;
   const Real half = Real(0.5), t0d = K.delta * K.theta0;
   for (int b = threadIdx.x; b < 2 * nb; b += nthreads) {
     const int line = b >= nb, x0 = (b - line * nb) * kBE, n = min(kBE, nx - x0), o = line * nx + x0;
     BeRow<Real> w[kBE];
+    Real g_last = Real(0);
     Real kp = sK[o];
     Real kf = K.dt * (half * (kp + (x0 == 0 ? kGl : sK[o - 1])));  // face below
 #pragma unroll
@@ -155,6 +164,7 @@ __device__ __forceinline__ void be_blocks(const StepConst<Real>& K, int nx, int 
         // before a block's first point lies x_prev itself
         const BeRow<Real> before = i == 0 ? BeRow<Real>{Real(1), Real(0), Real(0), Real(0)} : w[i > 0 ? i - 1 : 0];
         w[i] = be_eliminate(before, l, u, s, r);
+        g_last = w[i].g;
         kp = kn;
         kf = kq;
       }
@@ -166,33 +176,41 @@ __device__ __forceinline__ void be_blocks(const StepConst<Real>& K, int nx, int 
     for (int i = 0; i < kBE; ++i)
       if (i < n) {
         sL[o + i] = w[i].l;
-        sU[o + i] = w[i].u;
-        sE[o + i] = w[i].g;
+        sE[o + i] = w[i].u;
         sR[o + i] = w[i].r;
       }
+    sG[2 * b] = w[0].g;
+    sG[2 * b + 1] = g_last;
   }
 }
 
 // Separators of a line by one warp; their solution replaces sR at the separators.
 template <typename Real>
-__device__ __forceinline__ void be_separators(int nx, int line, Real* sL, Real* sU, Real* sG, Real* sR) {
+__device__ __forceinline__ void be_separators(int nx, int line, Real* sL, Real* sU, Real* sR, Real* sG) {
   const unsigned all = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int nb = (nx + kBE - 1) / kBE, per = (nb + 31) / 32;
   const int j0 = lane * per, cnt = max(0, min(per, nb - j0));
   auto sep = [&](int j) { return line * nx + min((j + 1) * kBE, nx) - 1; };
-  auto get = [&](int p) { return BeRow<Real>{sL[p], sU[p], sG[p], sR[p]}; };
-  auto put = [&](int p, const BeRow<Real>& w) { sL[p] = w.l, sU[p] = w.u, sG[p] = w.g, sR[p] = w.r; };
+  Real* gl = sG + 2 * line * nb;  // g of block j's first (2 j) and last (2 j + 1) point
+  auto get = [&](int j) {
+    const int p = sep(j);
+    return BeRow<Real>{sL[p], sU[p], gl[2 * j + 1], sR[p]};
+  };
+  auto put = [&](int j, const BeRow<Real>& w) {
+    const int p = sep(j);
+    sL[p] = w.l, sU[p] = w.u, gl[2 * j + 1] = w.g, sR[p] = w.r;
+  };
   const BeRow<Real> none{Real(0), Real(1), Real(0), Real(0)};  // x_next is the separator itself
   // forward sweep over the lane's separators, rows kept at the separators' slots
   BeRow<Real> w{Real(0), Real(0), Real(1), Real(0)};
   for (int k = 0; k < cnt; ++k) {
-    const int j = j0 + k, p = sep(j);
-    BeRow<Real> a = get(p);
+    const int j = j0 + k;
+    BeRow<Real> a = get(j);
     // the next block's first point by the separators (its own last point when
     // the block has one point; nothing beyond the last block, where u = 0)
     const int q = line * nx + (j + 1) * kBE;
-    const BeRow<Real> n = j + 1 < nb && (j + 1) * kBE < nx - 1 ? get(q) : none;
+    const BeRow<Real> n = j + 1 < nb && (j + 1) * kBE < nx - 1 ? BeRow<Real>{sL[q], sU[q], gl[2 * j + 2], sR[q]} : none;
     // a = r + l x_prev + u (n.r + n.l x + n.u x_next): 1 - u n.l = l + g + u (n.u + n.g)
     const Real inv = Real(1) / (a.l + fmad(a.u, n.u + n.g, a.g));
     a.g = fmad(a.u, n.g, a.g) * inv;
@@ -200,18 +218,17 @@ __device__ __forceinline__ void be_separators(int nx, int line, Real* sL, Real* 
     a.u = a.u * n.u * inv;
     a.l = a.l * inv;
     w = k == 0 ? a : be_eliminate(w, a.l, a.u, a.g, a.r);
-    put(p, w);
+    put(j, w);
   }
   // the lane's first separator by the previous lane's last one and its own
   // last one; w stays the last row
   BeRow<Real> f = none;
   if (cnt > 1) {
-    f = get(sep(j0 + cnt - 2));
+    f = get(j0 + cnt - 2);
     for (int k = cnt - 3; k >= 0; --k) {
-      const int p = sep(j0 + k);
-      BeRow<Real> a = get(p);
+      BeRow<Real> a = get(j0 + k);
       be_fold(a, f);
-      put(p, a);
+      put(j0 + k, a);
       f = a;
     }
   }
@@ -243,18 +260,22 @@ __device__ __forceinline__ void be_separators(int nx, int line, Real* sL, Real* 
 // e of every point from its block's and the previous block's separators.
 template <typename Real>
 __device__ __forceinline__ void be_points(const StepConst<Real>& K, int nx, int nthreads, Real* sE, const Real* sD,
-                                          const Real* sL, const Real* sU, const Real* sR) {
+                                          const Real* sL, const Real* sR) {
   for (int p = threadIdx.x; p < 2 * nx; p += nthreads) {
     const int s = p >= nx, x = p - s * nx, j = x / kBE;
     const int q = s * nx + min((j + 1) * kBE, nx) - 1;
     Real phi = sR[q];
     if (p != q) {
-      phi = fmad(sU[p], phi, sR[p]);
+      phi = fmad(sE[p], phi, sR[p]);  // u
       if (j > 0) phi = fmad(sL[p], sR[s * nx + j * kBE - 1], phi);
     }
     const Real dr = sD[p];
     sE[p] = Real(0.5) * K.delta * ((Real(1) + dr) * phi + K.theta0 * dr);
   }
+}
+
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
 // FTCS sub-steps of a tube's two sublattice lines, several per block barrier.
@@ -274,9 +295,9 @@ template <typename Real>
 struct FtcsLine {
   const Real* a;     // theta_R - theta0 = a e + c
   const Real* c;
+  const Real* th0;   // theta_R - theta0 of the corrector, for the first sub-step
   const Real* face;  // K of the face below each point
   const Real* last;  // and of the face above the last point, per line
-  const Real* th0;   // theta_R - theta0 of the corrector, for the first sub-step
   int nx;
   Real h;             // dt / nsub
   Real th_lo, th_hi;  // reservoir values
@@ -299,12 +320,15 @@ __device__ __forceinline__ void ftcs_pass(const FtcsLine<Real>& L, const Real* e
       e[i] = in ? ein[off + x] : Real(0);
       a[i] = in ? L.a[off + x] : Real(0);
       c[i] = in ? L.c[off + x] : (x < 0 ? L.th_lo : L.th_hi);
+      th[i] = fmad(a[i], e[i], c[i]);
       f[i] = in ? L.face[off + x] : (x == nx ? L.last[s] : Real(0));
     }
     f[kP] = __shfl_down_sync(0xffffffffu, f[0], 1);
+    if (first) {
 #pragma unroll
-    for (int i = 0; i < kP; ++i)
-      th[i] = first && x0 + i >= 0 && x0 + i < nx ? L.th0[off + x0 + i] : fmad(a[i], e[i], c[i]);
+      for (int i = 0; i < kP; ++i)
+        if (x0 + i >= 0 && x0 + i < nx) th[i] = L.th0[off + x0 + i];
+    }
     for (int k = 0; k < m; ++k) {
       const Real lo = __shfl_up_sync(0xffffffffu, th[kP - 1], 1);
       const Real hi = __shfl_down_sync(0xffffffffu, th[0], 1);
@@ -348,15 +372,16 @@ __global__ void __launch_bounds__(kThreads)
     k_batch(TubeDev<Real>* __restrict__ tubes, const int* __restrict__ order, int ntubes,
             int* __restrict__ counter, Store* __restrict__ pop0, Store* __restrict__ pop1,
             Real* __restrict__ e_state, Real* __restrict__ ux_state, float* __restrict__ snaps,
-            int save_every, int max_np, unsigned* __restrict__ status) {
+            int save_every, int max_np, int prefetch, unsigned* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  Real* sE = reinterpret_cast<Real*>(smem_raw);  // auxiliary E_R (state), then corrector
-  Real* sS = sE + max_np;                        // e* after exchange, then theta_R
-  Real* sU0 = sS + max_np;                       // u_x ring slot 0
+  Real* sE = reinterpret_cast<Real*>(smem_raw);  // auxiliary E_R (state), e* after the exchange, then corrector
+  Real* sU0 = sE + max_np;                       // u_x ring slot 0
   Real* sU1 = sU0 + max_np;                      // u_x ring slot 1
   Real* sD = sU1 + max_np;                       // rho - 1
   Real* sK = sD + max_np;                        // kappa_R
   Real* sP = sK + max_np;                        // predictor
+  [[maybe_unused]] Real* sG = sP + max_np;       // backward Euler: row excesses at block ends
+  [[maybe_unused]] Real* sT = sG;                // FTCS: theta_R - theta0 of the corrector
   __shared__ int s_slot;
   __shared__ Real s_last[2];  // K of each line's last face
   const int tid = threadIdx.x;
@@ -396,6 +421,16 @@ __global__ void __launch_bounds__(kThreads)
       // 1. pull + collide + exchange of every point of the tube
       for (int p = tid; p < np; p += kThreads) {
         const int s = p >= nx, x = p - s * nx;
+        // the populations of this warp's next points come from device memory while
+        // these are worked on: lane l asks for planes l and l + 32 (L2 only, one
+        // request per plane and warp). 3000 cells: 13.9 -> 15.6 G point steps a
+        // second; where the running tubes fit L2 it costs (1000 cells: 16.1 -> 15.5)
+        const int pn = p - (tid & 31) + kThreads;
+        if (prefetch && pn < np) {
+          const int sn = pn >= nx, xn = pn - sn * nx;
+          prefetch_l2(pin + (sn * kQ + (tid & 31)) * nx + xn);
+          if ((tid & 31) < kQ - 32) prefetch_l2(pin + (sn * kQ + 32 + (tid & 31)) * nx + xn);
+        }
         Real h[kQ];
         if (streamed) {
 #pragma unroll
@@ -407,7 +442,7 @@ __global__ void __launch_bounds__(kThreads)
         Store* out = pout + s * kQ * nx + x;
         const Real es = collide_shells<Real, false>(
             K, h, sE[p], [&](int q, Real v) { out[q * nx] = from_real<Store, Real>(v); }, m);
-        sS[p] = es;
+        sE[p] = es;
         sD[p] = m.drho;
         uc[p] = m.j[0] * m.inv_rho;
         sK[p] = K.kapc * m.rho * (K.theta0 + m.dth);
@@ -429,16 +464,16 @@ __global__ void __launch_bounds__(kThreads)
           eq = gh[kGhE];
           vq = gh[kGhU];
         } else {
-          eq = sS[p + 1];
+          eq = sE[p + 1];
           vq = Real(1.5) * uc[p + 1] - Real(0.5) * up[p + 1];
         }
-        const Real e0 = sS[p];
+        const Real e0 = sE[p];
         Real div = Real(0);
         div += K.E0 * (vq - vp) + (eq * vq - e0 * vp);
         sP[p] = e0 - K.dt * div;
       }
       __syncthreads();
-      // 3. corrector (backward difference), then theta_R of the result
+      // 3. corrector (backward difference), then theta_R of the result for FTCS
       for (int p = tid; p < np; p += kThreads) {
         const int s = p >= nx, x = p - s * nx;
         const Real vp = Real(1.5) * uc[p] - Real(0.5) * up[p];
@@ -453,28 +488,29 @@ __global__ void __launch_bounds__(kThreads)
         const Real epp = sP[p];
         Real div = Real(0);
         div += K.E0 * (vp - vq) + (epp * vp - eq * vq);
-        const Real val = Real(0.5) * (sS[p] + epp - K.dt * div);
-        const Real dr = sD[p];
+        const Real val = Real(0.5) * (sE[p] + epp - K.dt * div);
         sE[p] = val;
-        if constexpr (!kImplicit) sS[p] = (Real(2) * val - t0d * dr) / (K.delta * (Real(1) + dr));
+        if constexpr (!kImplicit) {
+          const Real dr = sD[p];
+          sT[p] = (Real(2) * val - t0d * dr) / (K.delta * (Real(1) + dr));
+        }
       }
       __syncthreads();
       if constexpr (kImplicit) {
-        // 4'. backward-Euler variant: l -> sP, u -> sS, g -> sE, r -> the u(t-1) slot (dead
-        //     until the next step's u)
+        // 4'. backward-Euler variant: l -> sP, u -> sE, r -> the u(t-1) slot (dead
+        //     until the next step's u), g at the blocks' ends -> sG
         Real* r = (t & 1) ? sU0 : sU1;
-        be_blocks(K, nx, kThreads, sE, sD, sK, sP, sS, r, gl[kGhKap], gh[kGhKap], thGl, thGh);
+        be_blocks(K, nx, kThreads, sE, sD, sK, sP, r, sG, gl[kGhKap], gh[kGhKap], thGl, thGh);
         __syncthreads();
-        if (tid < 64) be_separators(nx, tid >> 5, sP, sS, sE, r);
+        if (tid < 64) be_separators(nx, tid >> 5, sP, sE, r, sG);
         __syncthreads();
-        be_points(K, nx, kThreads, sE, sD, sP, sS, r);
+        be_points(K, nx, kThreads, sE, sD, sP, r);
         __syncthreads();
       } else {
         // 4. FTCS sub-steps, e += h sum_faces K_face (theta_nb - theta) with
         //    theta_R = a e + c, a = 2/(delta(1 + D)), c = -delta theta0 D/(delta(1 + D))
         //    (affine in e at fixed rho; the first sub-step takes the corrector's
-        //    theta_R): a -> sP, c -> sD, K of every point's low face -> the u(t-1)
-        //    slot (dead until the next step's u), e between sE and sK.
+        //    theta_R): a -> sP, c -> sD, K of every point's low face -> the u(t-1) slot (dead until the next step's u), e between sE and sK.
         Real* face = (t & 1) ? sU0 : sU1;
         for (int p = tid; p < np; p += kThreads) {
           const int s = p >= nx, x = p - s * nx;
@@ -486,7 +522,7 @@ __global__ void __launch_bounds__(kThreads)
           if (x == nx - 1) s_last[s] = Real(0.5) * (kp + gh[kGhKap]);
         }
         __syncthreads();
-        const FtcsLine<Real> FL{sP, sD, face, s_last, sS, nx, K.hsub, thGl, thGh};
+        const FtcsLine<Real> FL{sP, sD, sT, face, s_last, nx, K.hsub, thGl, thGh};
         Real* ein = sE;
         Real* eout = sK;
         const int width = ftcs_width<Real>(nx, kThreads / 32);
@@ -711,8 +747,11 @@ struct BatchOps {
 bool supported_threads(int t) { return t == 128 || t == 256 || t == 384 || t == 512; }
 
 size_t batch_smem(const rpk_batch* B) {
-  return (size_t)kBatchArrays * 2 * B->max_nx * B->real_elem;
+  const size_t n = B->max_nx, blocks = (n + kBE - 1) / kBE;
+  return (kBatchArrays * 2 * n + (B->implicit ? 4 * blocks : 2 * n)) * B->real_elem;
 }
+
+size_t batch_smem_rule(const rpk_batch* B) { return (size_t)kBatchRuleArrays * 2 * B->max_nx * B->real_elem; }
 
 template <typename F>
 rpk_status with_batch_types(int precision, F&& f) {
@@ -806,8 +845,12 @@ rpk_status launch_batch(rpk_batch* B, cudaStream_t stream, int threads, int ctas
   const int max_np = 2 * B->max_nx;
   void* kfn = BatchOps<Store, Real>::kernel(threads, B->implicit);
   int ntubes = B->ntubes, save_every = B->save_every;
+  // both population buffers of the tubes that run at a time, against L2
+  int l2 = 0;
+  RPK_CUDA(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, B->device));
+  int prefetch = (double)B->total_pts / ntubes * grid * 2 * kQ * sizeof(Store) > (double)l2;
   void* args[] = {&tubes, &B->order_dev, &ntubes, &B->counter, &p0,         &p1,
-                  &es,    &us,           &B->snaps, &save_every, (void*)&max_np, &B->status};
+                  &es,    &us,           &B->snaps, &save_every, (void*)&max_np, &prefetch, &B->status};
   RPK_CUDA(cudaLaunchKernel(kfn, dim3(grid), dim3(threads), args, smem, stream));
   RPK_CUDA(cudaGetLastError());
   return RPK_OK;
@@ -844,7 +887,7 @@ rpk_status init_from_stage(rpk_batch* B, const float* state) {
 }
 
 bool config_fits(const rpk_batch* B, int threads, int ctas) {
-  return supported_threads(threads) && ctas >= 1 && batch_smem(B) * ctas <= kBatchSmemLimit &&
+  return supported_threads(threads) && ctas >= 1 && batch_smem_rule(B) * ctas <= kBatchSmemLimit &&
          threads * ctas <= 2048;
 }
 
@@ -854,7 +897,7 @@ extern "C" {
 
 int rpk_batch_max_nx(int precision) {
   const size_t real = precision == RPK_F64 ? 8 : 4;
-  return (int)((kBatchSmemLimit - 1024) / (kBatchArrays * 2 * real));
+  return (int)((kBatchSmemLimit - 1024) / (kBatchRuleArrays * 2 * real));
 }
 
 rpk_status rpk_batch_create(int precision, int ntubes, const rpk_tube* tubes, int save_every,
