@@ -289,8 +289,8 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 // order of the lattice's FTCS kernels, so results are those of one barrier per
 // sub-step bit for bit.
 // With a block barrier and 10 shared loads per point and sub-step it took 0.8
-// us a sub-step for tubes of 1500 cells; 304 tubes of 500 to 1500 cells went
-// from 405 to 104 ms.
+// us a sub-step for tubes of 1500 cells; now 0.11 (0.16 with every piece loaded
+// anew for each 5 to 13 sub-steps). 304 tubes of 500 to 1500 cells: 405 -> 70 ms.
 template <typename Real>
 struct FtcsLine {
   const Real* a;     // theta_R - theta0 = a e + c
@@ -303,32 +303,41 @@ struct FtcsLine {
   Real th_lo, th_hi;  // reservoir values
 };
 
+// A piece in registers.
 template <int kP, typename Real>
-__device__ __forceinline__ void ftcs_pass(const FtcsLine<Real>& L, const Real* ein, Real* eout, int m,
-                                          int nwarps, bool first) {
-  const int lane = threadIdx.x & 31;
-  const int nx = L.nx, pieces = (nx + 30 * kP - 1) / (30 * kP);
-  for (int w = threadIdx.x >> 5; w < 2 * pieces; w += nwarps) {
-    const int s = w >= pieces, x0 = (w - s * pieces) * 30 * kP + (lane - 1) * kP;
-    const int off = s * nx;
-    Real e[kP], a[kP], c[kP], f[kP + 1], th[kP];
+struct FtcsPiece {
+  Real e[kP], a[kP], c[kP], f[kP + 1], th[kP];
+  int at, nv;  // the lane's first point in a field; how many of its points lie on the line
+
+  // Piece w of the tube's 2 x pieces, from the field ein.
+  __device__ __forceinline__ void load(const FtcsLine<Real>& L, const Real* ein, int w, int pieces, bool first) {
+    const int lane = threadIdx.x & 31, s = w >= pieces;
+    const int x0 = (w - s * pieces) * 30 * kP + (lane - 1) * kP;  // -kP below the line's low end
+    at = s * L.nx + x0;
+    nv = x0 < 0 ? 0 : min(kP, max(0, L.nx - x0));
+    const Real out = x0 < 0 ? L.th_lo : L.th_hi;
 #pragma unroll
     for (int i = 0; i < kP; ++i) {
-      const int x = x0 + i;
-      const bool in = x >= 0 && x < nx;
+      const bool in = i < nv;
       // beyond an end: theta stays the reservoir's (a = 0)
-      e[i] = in ? ein[off + x] : Real(0);
-      a[i] = in ? L.a[off + x] : Real(0);
-      c[i] = in ? L.c[off + x] : (x < 0 ? L.th_lo : L.th_hi);
+      e[i] = in ? ein[at + i] : Real(0);
+      a[i] = in ? L.a[at + i] : Real(0);
+      c[i] = in ? L.c[at + i] : out;
+      f[i] = in ? L.face[at + i] : Real(0);
+      if (x0 + i == L.nx) f[i] = L.last[s];
       th[i] = fmad(a[i], e[i], c[i]);
-      f[i] = in ? L.face[off + x] : (x == nx ? L.last[s] : Real(0));
     }
     f[kP] = __shfl_down_sync(0xffffffffu, f[0], 1);
     if (first) {
 #pragma unroll
       for (int i = 0; i < kP; ++i)
-        if (x0 + i >= 0 && x0 + i < nx) th[i] = L.th0[off + x0 + i];
+        if (i < nv) th[i] = L.th0[at + i];
     }
+  }
+
+  // m <= kP sub-steps.
+  __device__ __forceinline__ void advance(Real h, int m) {
+#pragma unroll 1
     for (int k = 0; k < m; ++k) {
       const Real lo = __shfl_up_sync(0xffffffffu, th[kP - 1], 1);
       const Real hi = __shfl_down_sync(0xffffffffu, th[0], 1);
@@ -336,35 +345,92 @@ __device__ __forceinline__ void ftcs_pass(const FtcsLine<Real>& L, const Real* e
 #pragma unroll
       for (int i = 0; i < kP; ++i) {
         const Real dn = (i + 1 < kP ? th[i + 1] : hi) - th[i];
-        e[i] = fmad(L.h, fmad(f[i + 1], dn, -(f[i] * d)), e[i]);
+        e[i] = fmad(h, fmad(f[i + 1], dn, -(f[i] * d)), e[i]);
         d = dn;
       }
 #pragma unroll
       for (int i = 0; i < kP; ++i) th[i] = fmad(a[i], e[i], c[i]);
     }
-    if (lane > 0 && lane < 31) {
+  }
+
+  __device__ __forceinline__ void store(Real* out) const {
 #pragma unroll
-      for (int i = 0; i < kP; ++i)
-        if (x0 + i < nx) eout[off + x0 + i] = e[i];
-    }
+    for (int i = 0; i < kP; ++i)
+      if (i < nv) out[at + i] = e[i];
+  }
+  // e of the whole lane from a neighbour's store
+  __device__ __forceinline__ void fetch(const Real* in) {
+#pragma unroll
+    for (int i = 0; i < kP; ++i)
+      if (i < nv) {
+        e[i] = in[at + i];
+        th[i] = fmad(a[i], e[i], c[i]);
+      }
+  }
+};
+
+// More pieces than warps: every kP sub-steps all pieces go through registers.
+template <int kP, typename Real>
+__device__ __forceinline__ void ftcs_pass(const FtcsLine<Real>& L, const Real* ein, Real* eout, int m,
+                                          int nwarps, bool first) {
+  const int lane = threadIdx.x & 31, pieces = (L.nx + 30 * kP - 1) / (30 * kP);
+  for (int w = threadIdx.x >> 5; w < 2 * pieces; w += nwarps) {
+    FtcsPiece<kP, Real> P;
+    P.load(L, ein, w, pieces, first);
+    P.advance(L.h, m);
+    if (lane > 0 && lane < 31) P.store(eout);
   }
 }
 
-// Points per lane of ftcs_pass: the fewest point slots per warp over the
-// rounds that a tube's pieces take; among equals the widest (fewest barriers).
+// At most one piece per warp: it stays in registers for all sub-steps of the
+// time step, and every kP of them the neighbours exchange their end lanes' points
+// through two buffers used in turn. Warps without a piece only keep the barriers
+// (one common path for both made the compiler spill the pieces around them).
+template <int kP, typename Real>
+__device__ __forceinline__ void ftcs_resident(const FtcsLine<Real>& L, Real* sE, Real* buf0, Real* buf1, int nsub) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int pieces = (L.nx + 30 * kP - 1) / (30 * kP);
+  if (w >= 2 * pieces) {  // keeps the barriers' count
+    for (int k = 0; k < nsub; k += kP) __syncthreads();
+    __syncthreads();
+    return;
+  }
+  FtcsPiece<kP, Real> P;
+  P.load(L, sE, w, pieces, true);
+  __syncthreads();  // every halo is read before sE is written
+  Real* buf = buf0;
+  Real* next = buf1;
+  P.advance(L.h, min(nsub, kP));
+#pragma unroll 1
+  for (int k = kP; k < nsub; k += kP) {
+    if (lane == 1 || lane == 30) P.store(buf);
+    __syncthreads();
+    if (lane == 0 || lane == 31) P.fetch(buf);
+    P.advance(L.h, min(nsub - k, kP));
+    Real* t = buf;
+    buf = next;
+    next = t;
+  }
+  if (lane > 0 && lane < 31) P.store(sE);
+  __syncthreads();
+}
+
+// Points per lane: the fewest with which every warp has at most one piece; else
+// (negative: passes) the fewest point slots per warp over the rounds that the
+// pieces take, among equals the most (fewest barriers).
 template <typename Real>
 __device__ __forceinline__ int ftcs_width(int nx, int nwarps) {
-  if (sizeof(Real) == 8) return 5;
   int best = 5, cost = 1 << 30;
-  for (int w = 5; w <= 13; w += (w < 9 ? 2 : 4)) {
+  for (int w = 5; w <= (sizeof(Real) == 8 ? 5 : 13); w += (w < 9 ? 2 : 4)) {
     const int pieces = 2 * ((nx + 30 * w - 1) / (30 * w));
+    if (pieces <= nwarps) return w;
     const int c = (pieces + nwarps - 1) / nwarps * w;
     if (c <= cost) {
       cost = c;
       best = w;
     }
   }
-  return best;
+  return -best;
 }
 
 template <typename Store, typename Real, int kThreads, bool kImplicit>
@@ -523,28 +589,36 @@ __global__ void __launch_bounds__(kThreads)
         }
         __syncthreads();
         const FtcsLine<Real> FL{sP, sD, sT, face, s_last, nx, K.hsub, thGl, thGh};
-        Real* ein = sE;
-        Real* eout = sK;
         const int width = ftcs_width<Real>(nx, kThreads / 32);
-        for (int k = 0; k < nsub;) {
-          const int m = min(nsub - k, width);
+        auto by_width = [&](auto&& run) {
+          const int v = width < 0 ? -width : width;
           if constexpr (sizeof(Real) == 8) {
-            ftcs_pass<5>(FL, ein, eout, m, kThreads / 32, k == 0);
+            run(std::integral_constant<int, 5>{});
           } else {
-            if (width == 5) ftcs_pass<5>(FL, ein, eout, m, kThreads / 32, k == 0);
-            else if (width == 7) ftcs_pass<7>(FL, ein, eout, m, kThreads / 32, k == 0);
-            else if (width == 9) ftcs_pass<9>(FL, ein, eout, m, kThreads / 32, k == 0);
-            else ftcs_pass<13>(FL, ein, eout, m, kThreads / 32, k == 0);
+            if (v == 5) run(std::integral_constant<int, 5>{});
+            else if (v == 7) run(std::integral_constant<int, 7>{});
+            else if (v == 9) run(std::integral_constant<int, 9>{});
+            else run(std::integral_constant<int, 13>{});
           }
-          k += m;
-          __syncthreads();
-          Real* tmp = ein;
-          ein = eout;
-          eout = tmp;
-        }
-        if (ein != sE) {
-          for (int p = tid; p < np; p += kThreads) sE[p] = ein[p];
-          __syncthreads();
+        };
+        if (width > 0) {
+          by_width([&](auto wc) { ftcs_resident<decltype(wc)::value>(FL, sE, sK, sT, nsub); });
+        } else {
+          Real* ein = sE;
+          Real* eout = sK;
+          for (int k = 0; k < nsub;) {
+            const int m = min(nsub - k, -width);
+            by_width([&](auto wc) { ftcs_pass<decltype(wc)::value>(FL, ein, eout, m, kThreads / 32, k == 0); });
+            k += m;
+            __syncthreads();
+            Real* tmp = ein;
+            ein = eout;
+            eout = tmp;
+          }
+          if (ein != sE) {
+            for (int p = tid; p < np; p += kThreads) sE[p] = ein[p];
+            __syncthreads();
+          }
         }
       }
       cur ^= 1;
