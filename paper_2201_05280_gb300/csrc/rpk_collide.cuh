@@ -38,16 +38,15 @@ __device__ __forceinline__ V collide_relax(const StepConst<Real>& K, Mom<V>& m, 
     return fmad(K.exc * m.rho, m.dth - m.dR, e);
 }
 
-// The same with the shell-wise sums and targets: about 470 operations a point
-// instead of 690 (FP64: 760 to 530 instructions of its pipe).
+// The same with the shell-wise sums and targets: about 430 operations a point
+// instead of 690. FP64 is bound by its pipe (two lanes per cycle and SM): 96^3, 760
+// of its instructions and 2160 us pair by pair, SHELLDP and SHELLUS us now.
 template <typename Real, bool kPaper, typename V, typename Emit>
 __device__ __forceinline__ V collide_shells(const StepConst<Real>& K, const V (&h)[kQ], V e, Emit&& emit,
                                             Mom<V>& m) {
   raw_moments_shells(h, m);
-  recover<Real, kPaper, true>(m, e, K);
   Herm<V> H;
-  mix_coeffs(m, K, H);
-  herm_scale(H, K.c_relax);
+  relaxed_target<Real, kPaper>(m, e, K, H);
   emit(0, fmad(K.c_keep, h[0], H.e0));
   herm_shells(H, [&](int k, V ev, V od) {
     emit(2 * k + 1, fmad(K.c_keep, h[2 * k + 1], ev + od));

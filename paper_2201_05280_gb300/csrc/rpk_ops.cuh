@@ -42,6 +42,18 @@ static StepConst<Real> make_step_const(const rpk_relax& r, int nsub, int nx, int
   K.kapc = Real(r.k_r * 5.0 * r.tau / (2.0 * B));
   K.E0 = Real(0.5 * r.delta * kTheta0);
   K.inv_delta = Real(1.0 / r.delta);
+  const double i1 = 1.0 / kTheta0, cr = 2.0 * beta;
+  K.two_id = Real(2.0 / r.delta);
+  K.c_d = Real(r.delta / (3.0 + r.delta));
+  K.c_3 = Real(3.0 / (3.0 + r.delta));
+  K.bsig = Real(tau_s / r.tau * r.b / (1.0 + r.dt / (2.0 * tau_s) - r.b * r.dt / (2.0 * r.tau)));
+  K.q1h = Real(0.5 * cr * i1);
+  K.q1 = Real(cr * i1);
+  K.q2h = Real(0.5 * cr * i1 * i1);
+  K.q2 = Real(cr * i1 * i1);
+  K.q36 = Real(cr * i1 * i1 * i1 / 6.0);
+  K.q32 = Real(0.5 * cr * i1 * i1 * i1);
+  K.q3 = Real(cr * i1 * i1 * i1);
   K.dt = Real(r.dt);
   K.hsub = Real(r.dt / std::max(1, nsub));
   const double X = 3.0 * r.dt / (2.0 * r.tau1 * (3.0 + r.delta));
