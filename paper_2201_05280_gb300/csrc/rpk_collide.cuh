@@ -40,7 +40,8 @@ __device__ __forceinline__ V collide_relax(const StepConst<Real>& K, Mom<V>& m, 
 
 // The same with the shell-wise sums and targets: about 430 operations a point
 // instead of 690. FP64 is bound by its pipe (two lanes per cycle and SM): 96^3, 760
-// of its instructions and 2160 us pair by pair, SHELLDP and SHELLUS us now.
+// of its instructions a point and 2160 us pair by pair, 422 and 1415 us now (0.9 of
+// the pipe's rate).
 template <typename Real, bool kPaper, typename V, typename Emit>
 __device__ __forceinline__ V collide_shells(const StepConst<Real>& K, const V (&h)[kQ], V e, Emit&& emit,
                                             Mom<V>& m) {
