@@ -100,11 +100,11 @@ __device__ __forceinline__ void flag_moments(const Mom<Real>& m, Real theta0,
 // per SM keep enough loads in flight.
 template <typename Store, typename Real, bool kPull, int kBC, bool kPaper>
 __global__ void __launch_bounds__(128, sizeof(Real) == 4 ? 5 : 1)
-    k_collide(StepConst<Real> K, const Store* __restrict__ pin, Store* __restrict__ pout,
-              const Real* __restrict__ e_in, Real* __restrict__ e_out, Real* __restrict__ drho_out,
+    k_collide(StepConst<Real> K, const Store* pin, Store* __restrict__ pout,
+              const Real* e_in, Real* __restrict__ e_out, Real* __restrict__ drho_out,
               Real* __restrict__ u_out, Real* __restrict__ kap_out,
               const Real* __restrict__ ghost, unsigned* __restrict__ status,
-              Real* __restrict__ tt_out, const Real* __restrict__ wcol) {
+              Real* __restrict__ tt_out, const Real* wcol) {
   pdl_wait();
   PointIdx P;
   if (!point_from_block(K, P)) return;
@@ -157,8 +157,8 @@ __device__ __forceinline__ void flag_moments2(const Mom<F2>& m, float theta0, un
 // time-t theta_T(f) - theta0 goes to tt_out), as in k_collide.
 template <typename Store, bool kPaper = false>
 __global__ void __launch_bounds__(128, sizeof(Store) == 4 ? 3 : 4)
-    k_collide_pair(StepConst<float> K, const Store* __restrict__ pin, Store* __restrict__ pout,
-                   const float* __restrict__ e_in, float* __restrict__ e_out, float* __restrict__ drho_out,
+    k_collide_pair(StepConst<float> K, const Store* pin, Store* __restrict__ pout,
+                   const float* e_in, float* __restrict__ e_out, float* __restrict__ drho_out,
                    float* __restrict__ u_out, float* __restrict__ kap_out, unsigned* __restrict__ status,
                    float* __restrict__ tt_out) {
   pdl_wait();
@@ -198,8 +198,8 @@ __global__ void __launch_bounds__(128, sizeof(Store) == 4 ? 3 : 4)
 // integer operations).
 template <typename Store, bool kPaper = false>
 __global__ void __launch_bounds__(128, kPaper ? 4 : 5)
-    k_collide_pair_w(StepConst<float> K, const Store* __restrict__ pin, Store* __restrict__ pout,
-                     const float* __restrict__ e_in, float* __restrict__ e_out, float* __restrict__ drho_out,
+    k_collide_pair_w(StepConst<float> K, const Store* pin, Store* __restrict__ pout,
+                     const float* e_in, float* __restrict__ e_out, float* __restrict__ drho_out,
                      float* __restrict__ u_out, float* __restrict__ kap_out, unsigned* __restrict__ status,
                      float* __restrict__ tt_out) {
   pdl_wait();

@@ -778,7 +778,7 @@ __device__ __forceinline__ Real wall_column(const StepConst<Real>& K, const Stor
 // (x, z)), then x walls (slots 2 nx nz + [0, 2 ny nz), columns (y, z)).
 template <typename Store, typename Real, int kBC>
 __global__ void __launch_bounds__(128)
-    k_wall_rho(StepConst<Real> K, const Store* __restrict__ pin, const Real* __restrict__ ghost,
+    k_wall_rho(StepConst<Real> K, const Store* pin, const Real* __restrict__ ghost,
                Real* __restrict__ wcol) {
   pdl_wait();
   const int64_t ny_cols = (int64_t)K.nx * K.nz, nx_cols = (int64_t)K.ny * K.nz;

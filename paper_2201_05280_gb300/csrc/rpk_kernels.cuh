@@ -138,8 +138,8 @@ __device__ __forceinline__ Real vadv(const Real* __restrict__ ucur, const Real* 
 // Reservoir values stand beyond the x ends.
 template <typename Real, int kBC>
 __global__ void __launch_bounds__(kTBX * kTBY)
-    k_mac_pred(StepConst<Real> K, const Real* __restrict__ e, const Real* __restrict__ ucur,
-               const Real* __restrict__ uprev, Real* __restrict__ ep, Real* __restrict__ v,
+    k_mac_pred(StepConst<Real> K, const Real* e, const Real* ucur,
+               const Real* uprev, Real* __restrict__ ep, Real* __restrict__ v,
                const Real* __restrict__ ghost) {
   pdl_wait();
   PointIdx P;
@@ -171,8 +171,8 @@ __global__ void __launch_bounds__(kTBX * kTBY)
 
 template <typename Real, int kBC>
 __global__ void __launch_bounds__(kTBX * kTBY)
-    k_mac_corr(StepConst<Real> K, const Real* __restrict__ e, const Real* __restrict__ ep,
-               const Real* __restrict__ v, const Real* __restrict__ drho, Real* __restrict__ ec,
+    k_mac_corr(StepConst<Real> K, const Real* e, const Real* ep,
+               const Real* v, const Real* drho, Real* __restrict__ ec,
                Real* __restrict__ th, const Real* __restrict__ ghost) {
   pdl_wait();
   PointIdx P;
@@ -206,8 +206,8 @@ __global__ void __launch_bounds__(kTBX * kTBY)
 
 template <typename Real, int kBC>
 __global__ void __launch_bounds__(kTBX * kTBY)
-    k_ftcs(StepConst<Real> K, const Real* ec, const Real* __restrict__ th, const Real* __restrict__ kap,
-           Real* e_next, const Real* __restrict__ drho, Real* __restrict__ th_next,
+    k_ftcs(StepConst<Real> K, const Real* ec, const Real* th, const Real* kap,
+           Real* e_next, const Real* drho, Real* __restrict__ th_next,
            const Real* __restrict__ ghost) {
   pdl_wait();
   PointIdx P;
@@ -266,9 +266,9 @@ __global__ void __launch_bounds__(kTBX * kTBY)
 constexpr int kLineSub = 16;
 
 template <typename Real, int kBC, bool kFirst>
-__global__ void k_line_transport(StepConst<Real> K, const Real* __restrict__ e, const Real* __restrict__ ucur,
-                                 const Real* __restrict__ uprev, const Real* __restrict__ drho,
-                                 const Real* __restrict__ kap, Real* __restrict__ e_next,
+__global__ void k_line_transport(StepConst<Real> K, const Real* e, const Real* ucur,
+                                 const Real* uprev, const Real* drho,
+                                 const Real* kap, Real* __restrict__ e_next,
                                  const Real* __restrict__ ghost, int nsub) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char line_smem[];
@@ -368,8 +368,8 @@ __device__ __forceinline__ void un4(float4 q, float (&v)[4]) {
 }
 
 static __global__ void __launch_bounds__(kTBX * kTBY)
-    k_mac_pred4(StepConst<float> K, const float* __restrict__ e, const float* __restrict__ ucur,
-                const float* __restrict__ uprev, float* __restrict__ ep, float* __restrict__ v) {
+    k_mac_pred4(StepConst<float> K, const float* e, const float* ucur,
+                const float* uprev, float* __restrict__ ep, float* __restrict__ v) {
   pdl_wait();
   Quad Q;
   if (!quad_from_block(K, Q)) return;
@@ -411,8 +411,8 @@ static __global__ void __launch_bounds__(kTBX * kTBY)
 }
 
 static __global__ void __launch_bounds__(kTBX * kTBY)
-    k_mac_corr4(StepConst<float> K, const float* __restrict__ e, const float* __restrict__ ep,
-                const float* __restrict__ v, const float* __restrict__ drho, float* __restrict__ ec,
+    k_mac_corr4(StepConst<float> K, const float* e, const float* ep,
+                const float* v, const float* drho, float* __restrict__ ec,
                 float* __restrict__ th) {
   pdl_wait();
   Quad Q;
@@ -453,8 +453,8 @@ static __global__ void __launch_bounds__(kTBX * kTBY)
 }
 
 static __global__ void __launch_bounds__(kTBX * kTBY)
-    k_ftcs4(StepConst<float> K, const float* ec, const float* __restrict__ th, const float* __restrict__ kap,
-            float* e_next, const float* __restrict__ drho, float* __restrict__ th_next) {
+    k_ftcs4(StepConst<float> K, const float* ec, const float* th, const float* kap,
+            float* e_next, const float* drho, float* __restrict__ th_next) {
   pdl_wait();
   Quad Q;
   if (!quad_from_block(K, Q)) return;
@@ -512,7 +512,7 @@ static __global__ void __launch_bounds__(kTBX * kTBY)
 // FP32 grid, nx a multiple of 4): k_pm_pred, k_pm_corr and k_pm_ftcs point by
 // point, in the same order of operations.
 static __global__ void __launch_bounds__(kTBX * kTBY)
-    k_pm_pred4(StepConst<float> K, const float* __restrict__ r, const float* __restrict__ ucur,
+    k_pm_pred4(StepConst<float> K, const float* r, const float* ucur,
                float* __restrict__ rp) {
   pdl_wait();
   Quad Q;
@@ -541,8 +541,8 @@ static __global__ void __launch_bounds__(kTBX * kTBY)
 }
 
 static __global__ void __launch_bounds__(kTBX * kTBY)
-    k_pm_corr4(StepConst<float> K, const float* __restrict__ r, const float* __restrict__ rp,
-               const float* __restrict__ ucur, float* __restrict__ rc) {
+    k_pm_corr4(StepConst<float> K, const float* r, const float* rp,
+               const float* ucur, float* __restrict__ rc) {
   pdl_wait();
   Quad Q;
   if (!quad_from_block(K, Q)) return;
@@ -571,8 +571,8 @@ static __global__ void __launch_bounds__(kTBX * kTBY)
 }
 
 static __global__ void __launch_bounds__(kTBX * kTBY)
-    k_pm_ftcs4(StepConst<float> K, const float* __restrict__ r, const float* __restrict__ drho,
-               const float* __restrict__ kap, const float* __restrict__ tt, float* __restrict__ rn, int last) {
+    k_pm_ftcs4(StepConst<float> K, const float* r, const float* drho,
+               const float* kap, const float* tt, float* __restrict__ rn, int last) {
   pdl_wait();
   Quad Q;
   if (!quad_from_block(K, Q)) return;
@@ -635,7 +635,7 @@ __device__ __forceinline__ Real pm_nb(const StepConst<Real>& K, const PointIdx& 
 
 template <typename Real, int kBC>
 __global__ void __launch_bounds__(kTBX * kTBY)
-    k_pm_pred(StepConst<Real> K, const Real* __restrict__ r, const Real* __restrict__ ucur,
+    k_pm_pred(StepConst<Real> K, const Real* r, const Real* ucur,
               Real* __restrict__ rp, const Real* __restrict__ ghost) {
   pdl_wait();
   PointIdx P;
@@ -650,8 +650,8 @@ __global__ void __launch_bounds__(kTBX * kTBY)
 
 template <typename Real, int kBC>
 __global__ void __launch_bounds__(kTBX * kTBY)
-    k_pm_corr(StepConst<Real> K, const Real* __restrict__ r, const Real* __restrict__ rp,
-              const Real* __restrict__ ucur, Real* __restrict__ rc, const Real* __restrict__ ghost) {
+    k_pm_corr(StepConst<Real> K, const Real* r, const Real* rp,
+              const Real* ucur, Real* __restrict__ rc, const Real* __restrict__ ghost) {
   pdl_wait();
   PointIdx P;
   if (!point_from_block2d(K, P)) return;
@@ -665,8 +665,8 @@ __global__ void __launch_bounds__(kTBX * kTBY)
 
 template <typename Real, int kBC>
 __global__ void __launch_bounds__(kTBX * kTBY)
-    k_pm_ftcs(StepConst<Real> K, const Real* __restrict__ r, const Real* __restrict__ drho,
-              const Real* __restrict__ kap, const Real* __restrict__ tt, Real* __restrict__ rn,
+    k_pm_ftcs(StepConst<Real> K, const Real* r, const Real* drho,
+              const Real* kap, const Real* tt, Real* __restrict__ rn,
               const Real* __restrict__ ghost, int last) {
   pdl_wait();
   PointIdx P;

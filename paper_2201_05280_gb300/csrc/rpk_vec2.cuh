@@ -48,12 +48,16 @@ __device__ __forceinline__ F2 fmad(float a, F2 b, F2 c) { return fmad(F2(a), b, 
 __device__ __forceinline__ F2 fmad(F2 a, float b, F2 c) { return fmad(a, F2(b), c); }
 
 // Programmatic dependent launch: the kernels of a step let the next one's
-// blocks become resident while their own still run, and wait here until every
-// earlier kernel has completed (a no-op for ordinary launches). Nothing that an
-// earlier kernel writes or reads may be touched before it.
+// blocks become resident while their own still run, and wait here until the
+// kernel before has completed (a no-op for ordinary launches). Nothing that an
+// earlier kernel writes or reads may be touched before it, and what an earlier
+// kernel writes is not read through const __restrict__ parameters: those become
+// non-coherent loads, which may find lines that a kernel of two launches ago left in
+// L1 while this one's blocks were already resident. The next kernel is let in after
+// the wait, so that no more than two of a chain are resident.
 __device__ __forceinline__ void pdl_wait() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Scalar type of a value type: the type of the per-launch constants.
