@@ -10,6 +10,18 @@
 
 #include "../../include/rpk.h"
 
+// Launches of the rotational transport of a small lattice (rpk_brick.cuh): sub-steps
+// and points of a tile of each, for the sub-steps and boundaries it was made for;
+// none where a launch per pass is faster.
+struct BrickPlan {
+  struct Part {
+    int nsub;
+    int own[3];
+  };
+  int nsub = 0, open = -1;
+  std::vector<Part> parts;
+};
+
 struct rpk_lattice {
   rpk_grid grid;
   int device = 0;
@@ -49,6 +61,7 @@ struct rpk_lattice {
   double* stage = nullptr;          // 7 x npts doubles for host I/O, lazy
   int64_t steps = 0;
   size_t bytes_held = 0;
+  BrickPlan brick;
   // kernel timing: event pairs recorded around each kernel class
   bool timing = false;
   std::vector<cudaEvent_t> events;

@@ -7,7 +7,7 @@
 #include <type_traits>
 
 #include "rpk_internal.h"
-#include "rpk_kernels.cuh"
+#include "rpk_brick.cuh"
 
 namespace rpk {
 
@@ -213,6 +213,143 @@ static int line_launches(rpk_lattice* L, const StepConst<Real>& K, const Real* e
   return parts;
 }
 
+// Block of k_brick_transport: its region and how the threads share it.
+struct BrickBlock {
+  int ext[3], halo[3];
+  int planes, groups;  // planes a thread, threads a column
+  int threads;
+  size_t smem;
+};
+
+// Fill in the block of tiles of own points with halo h; false if it does not fit.
+static inline bool brick_block(const rpk_lattice* L, int open, const int (&own)[3], int h, BrickBlock& b) {
+  const int n[3] = {L->grid.nx, L->grid.ny, L->grid.nz};
+  for (int a = 0; a < 3; ++a) {
+    const bool op = (a == 0 && (open & (1 | kWallX))) || (a == 1 && (open & kWallY));
+    b.halo[a] = !op && (int64_t)own[a] + 2 * h > n[a] ? 0 : h;
+    b.ext[a] = op ? std::min(own[a] + 2 * h, n[a] + 2) : b.halo[a] ? own[a] + 2 * h : n[a];
+  }
+  const int64_t area = (int64_t)b.ext[0] * b.ext[1], Z = b.ext[2];
+  if (area > kBrickThreads || Z > kBrickMaxP * (kBrickThreads / area)) return false;
+  b.planes = (int)((Z + kBrickThreads / area - 1) / (kBrickThreads / area));
+  b.groups = (int)((Z + b.planes - 1) / b.planes);
+  b.threads = (int)((area * b.groups + 31) / 32 * 32);
+  b.smem = sizeof(float) * kBrickArrays * kBrickThreads * b.planes;
+  return true;
+}
+
+static inline auto brick_kernel(bool first, int planes) {
+  static constexpr decltype(&k_brick_transport<true, 1>) kernels[2][kBrickMaxP] = {
+      {k_brick_transport<false, 1>, k_brick_transport<false, 2>, k_brick_transport<false, 3>,
+       k_brick_transport<false, 4>, k_brick_transport<false, 5>, k_brick_transport<false, 6>},
+      {k_brick_transport<true, 1>, k_brick_transport<true, 2>, k_brick_transport<true, 3>,
+       k_brick_transport<true, 4>, k_brick_transport<true, 5>, k_brick_transport<true, 6>}};
+  return kernels[first][planes - 1];
+}
+
+// The cheapest split of a small lattice's transport into launches and tiles, or
+// none if a launch per pass costs less. Times in cycles, fitted to measurements: a
+// launch costs 3000 plus the greater of latency (1500, 600 a sub-step and 2500 for
+// each round of resident blocks) and work (for each warp and plane on the busiest SM
+// 50 and 22 a sub-step; 60 more for the MacCormack passes); a launch per pass costs 4900 plus one for 60 points of a sublattice, four
+// points a thread, or 5000 plus one for 36. Steps of both, us, passes / tiles: 16^3
+// 10.4 / 7.2, 40^3 16.3 / 14.4, 48^3 20.1 / 22.0 (passes taken), 64^3 45.5 / 53.7
+// (passes); between walls with five sub-steps 64 x 32 x 4 24.2 / 13.2, 150 x 90 x 8
+// 43.9 / 37.7, 160 x 96 x 16 80.6 / 81.3 (passes).
+static inline rpk_status make_brick_plan(rpk_lattice* L, int open) {
+  BrickPlan& B = L->brick;
+  if (B.nsub == L->nsub && B.open == open) return RPK_OK;
+  B.nsub = L->nsub;
+  B.open = open;
+  B.parts.clear();
+  if (L->n3 > (int64_t)kBrickMaxP * kBrickThreads * L->sms) return RPK_OK;
+  const int n[3] = {L->grid.nx, L->grid.ny, L->grid.nz};
+  static constexpr int kCuts[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32, 48, 64, 96, 128};
+  // best tile of a launch of m sub-steps
+  auto best = [&](int m, bool first, BrickPlan::Part& part) {
+    double cost = 1e30;
+    for (int cz : kCuts)
+      for (int cy : kCuts)
+        for (int cx : kCuts) {
+          if (cx > n[0] || cy > n[1] || cz > n[2] || cx * cy * cz > 2 * L->sms) break;
+          const int own[3] = {(n[0] + cx - 1) / cx, (n[1] + cy - 1) / cy, (n[2] + cz - 1) / cz};
+          BrickBlock b;
+          if (!brick_block(L, open, own, m + (first ? 1 : 0), b)) continue;
+          const int blocks = (2 * cx * cy * cz + L->sms - 1) / L->sms;  // of the busiest SM
+          const int rounds = (blocks * b.threads + kBrickThreads - 1) / kBrickThreads;
+          const double latency = 1500 + 600 * m + 2500 * rounds;
+          const double work = (double)blocks * (b.threads / 32) * b.planes * (50 + (first ? 60 : 0) + 22 * m);
+          const double c = 3000 + std::max(latency, work);
+          if (c < cost) {
+            cost = c;
+            part = {m, {own[0], own[1], own[2]}};
+          }
+        }
+    return cost;
+  };
+  double cost = (2 + L->nsub) * (open == 0 && L->grid.nx % 4 == 0 ? 4900 + L->n3 / 60.0 : 5000 + L->n3 / 36.0);
+  for (int m = std::min(L->nsub, kBrickSub); m >= 1; --m) {
+    const int parts = (L->nsub + m - 1) / m;
+    if (m > 1 && (L->nsub + m - 2) / (m - 1) == parts) continue;  // as many launches of fewer sub-steps
+    BrickPlan::Part first, full, rest;
+    // parts of m or m - 1 sub-steps, the first with the deeper halo a short one
+    const int shorter = parts * m - L->nsub, m0 = m - (shorter ? 1 : 0);
+    double c = best(m0, true, first);
+    const int nfull = L->nsub - m0 - (shorter ? shorter - 1 : 0) * (m - 1);
+    if (parts > 1 && nfull > 0) c += nfull / m * best(m, false, full);
+    if (shorter > 1) c += (shorter - 1) * best(m - 1, false, rest);
+    if (c < cost) {
+      cost = c;
+      B.parts.assign(1, first);
+      for (int i = 0; i < nfull / m; ++i) B.parts.push_back(full);
+      for (int i = 1; i < shorter; ++i) B.parts.push_back(rest);
+    }
+  }
+  if (B.parts.empty()) return RPK_OK;
+  for (int planes = 1; planes <= kBrickMaxP; ++planes)
+    for (bool first : {true, false})
+      RPK_CUDA(cudaFuncSetAttribute(brick_kernel(first, planes), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBrickSmem));
+  return RPK_OK;
+}
+
+// Transport of a small lattice in FP32 by its plan (conservative form).
+static inline rpk_status brick_launch(rpk_lattice* L, const StepConst<float>& K, int open) {
+  const float* src = static_cast<const float*>(L->e_star);
+  RPK_CUDA(timing_begin(L));
+  const size_t parts = L->brick.parts.size();
+  for (size_t i = 0; i < parts; ++i) {
+    const BrickPlan::Part& part = L->brick.parts[i];
+    BrickArgs B{};
+    B.nsub = part.nsub;
+    B.open = open;
+    BrickBlock b;
+    if (!brick_block(L, open, part.own, part.nsub + (i == 0 ? 1 : 0), b)) return fail(RPK_ERR_STATE, "transport tile does not fit");
+    const int n[3] = {L->grid.nx, L->grid.ny, L->grid.nz};
+    unsigned cuts[3];
+    for (int a = 0; a < 3; ++a) {
+      B.own[a] = part.own[a];
+      B.ext[a] = b.ext[a];
+      B.halo[a] = b.halo[a];
+      cuts[a] = (n[a] + part.own[a] - 1) / part.own[a];
+    }
+    B.tx = cuts[0];
+    B.ty = cuts[1];
+    B.groups = b.groups;
+    B.by_tx = FastDiv(cuts[0]);
+    B.by_ty = FastDiv(cuts[1]);
+    B.by_X = FastDiv(b.ext[0]);
+    B.by_area = FastDiv(b.ext[0] * b.ext[1]);
+    float* dst = static_cast<float*>(i + 1 == parts ? L->e : src == L->e_a ? L->e_b : L->e_a);
+    launch_step(L, brick_kernel(i == 0, b.planes), dim3(cuts[0] * cuts[1] * cuts[2], 2), dim3(b.threads), b.smem, K, B, src,
+                static_cast<const float*>(L->u[L->steps & 1]), static_cast<const float*>(L->u[(L->steps + 1) & 1]),
+                static_cast<const float*>(L->drho), static_cast<const float*>(L->kap), dst,
+                static_cast<const float*>(L->ghost));
+    src = dst;
+  }
+  RPK_CUDA(timing_end(L, RPK_KC_TRANSPORT, (int)parts));
+  return check_launch("rotational transport (brick)");
+}
+
 template <typename Real, int kBC>
 static rpk_status transport_launch(rpk_lattice* L, const StepConst<Real>& K) {
   const Real* ucur = static_cast<const Real*>(L->u[L->steps & 1]);
@@ -306,6 +443,16 @@ rpk_status Ops<Store, Real>::step(rpk_lattice* L, int64_t n) {
   const StepConst<Real> K = make_const<Real>(L);
   const bool res = L->grid.bc_x == RPK_BC_RESERVOIR;
   const int wm = wall_mask(L);
+  // FP32 storage only: 16-bit states depend on the rounding of every step, and FP64's
+  // pipe has no room for a recomputed halo
+  bool brick = false;
+  if constexpr (std::is_same<Store, float>::value) {
+    if (!L->rot_mode && (wm || L->grid.ny > 1 || L->grid.nz > 1)) {
+      const rpk_status st = make_brick_plan(L, res ? 1 : wm);
+      if (st != RPK_OK) return st;
+      brick = !L->brick.parts.empty();
+    }
+  }
   for (int64_t t = 0; t < n; ++t) {
     rpk_status st;
     RPK_CUDA(timing_begin(L));
@@ -326,7 +473,9 @@ rpk_status Ops<Store, Real>::step(rpk_lattice* L, int64_t n) {
       st = res ? collide_launch<Store, Real, true, 1>(L, K) : collide_launch<Store, Real, true, 0>(L, K);
     if (st != RPK_OK) return st;
     RPK_CUDA(timing_end(L, RPK_KC_COLLIDE, wall_pull ? 2 : 1));
-    if (wm == kWallY)
+    if (brick) {
+      if constexpr (std::is_same<Store, float>::value) st = brick_launch(L, K, res ? 1 : wm);
+    } else if (wm == kWallY)
       st = transport_launch<Real, kWallY>(L, K);
     else if (wm == kWallX)
       st = transport_launch<Real, kWallX>(L, K);
