@@ -176,10 +176,12 @@ __global__ void __launch_bounds__(kThreads) k_conv(ConvArgs P) {
 // k_conv for one tap (lift, head and the head's input gradient), bound by its
 // input and output: a warp takes 16 positions, reads their rows straight into
 // fragments (32-byte segments, each element once) and all kMT x 16 output channels
-// from weights that the block stages once for all its positions. The same
-// mma.sync shapes in the same order over k as k_conv, which re-staged 64 x 64
-// tiles element by element (606 K positions: lift 340 -> 141 us, head 324 -> 60
-// us).
+// from weights that the block stages once for all its positions, in k_conv's order
+// over k. Positions are the rows of the mma and each pair of 8-column tiles holds 16
+// channels interleaved by twos, so that a thread has four consecutive channels of a
+// position: one 16-byte store (with its bias) instead of four. 606 K positions: lift
+// 340 us in 64 x 64 tiles staged element by element, 141 with channels as rows, 79
+// now; head 324, 60 and 59.
 struct Conv1Args {
   const __nv_bfloat16* A;  // [M][K]
   const float* X;          // [npos][K]
@@ -187,22 +189,26 @@ struct Conv1Args {
   const float* bias;
   const float* mask;
   int M, K, relu_in, npos;
+  int quads;               // rows of out (and mask) are whole 16-byte pieces
 };
 constexpr int kConv1Threads = 256;
 
 template <int kMT>
 __global__ void __launch_bounds__(kConv1Threads) k_conv1(Conv1Args P) {
   extern __shared__ __align__(16) uint16_t c1_smem[];
+  __shared__ __align__(16) float c1_bias[kMT * 16];
   const int Kp = (P.K + 15) / 16 * 16, ld = Kp + kPadK;
   const int m0 = blockIdx.y * kMT * 16;
   // a warp takes whole rows of weights, a word of two at a time (K is even, so words are
-  // aligned)
+  // aligned); row 8 j + g of a tile pair holds channel 4 (g / 2) + 2 j + g % 2
 #pragma unroll 4
-  for (int m = threadIdx.x >> 5; m < kMT * 16; m += kConv1Threads / 32) {
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(P.A + (int64_t)(m0 + m) * P.K);
+  for (int r = threadIdx.x >> 5; r < kMT * 16; r += kConv1Threads / 32) {
+    const int m = m0 + (r & ~15) + 4 * ((r & 7) >> 1) + 2 * ((r >> 3) & 1) + (r & 1);
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(P.A + (int64_t)m * P.K);
     for (int k = threadIdx.x & 31; k < ld / 2; k += 32)
-      reinterpret_cast<uint32_t*>(c1_smem)[m * (ld / 2) + k] = m0 + m < P.M && 2 * k < P.K ? src[k] : 0u;
+      reinterpret_cast<uint32_t*>(c1_smem)[r * (ld / 2) + k] = m < P.M && 2 * k < P.K ? src[k] : 0u;
   }
+  if (threadIdx.x < kMT * 16) c1_bias[threadIdx.x] = P.bias && m0 + threadIdx.x < P.M ? P.bias[m0 + threadIdx.x] : 0.f;
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int tiles = (P.npos + 15) / 16;
@@ -211,7 +217,7 @@ __global__ void __launch_bounds__(kConv1Threads) k_conv1(Conv1Args P) {
     float acc[kMT][2][4] = {};
 #pragma unroll 3
     for (int k0 = 0; k0 < Kp; k0 += 16) {
-      uint32_t b[2][2];
+      uint32_t a[4];
 #pragma unroll
       for (int j = 0; j < 2; ++j)
 #pragma unroll
@@ -220,33 +226,47 @@ __global__ void __launch_bounds__(kConv1Threads) k_conv1(Conv1Args P) {
           float2 x = make_float2(0.f, 0.f);
           if (q < P.npos && k < P.K) x = *reinterpret_cast<const float2*>(P.X + (int64_t)q * P.K + k);
           if (P.relu_in) x.x = fmaxf(x.x, 0.f), x.y = fmaxf(x.y, 0.f);
-          b[j][h] = pack_bf16(x.x, x.y);
+          a[j + 2 * h] = pack_bf16(x.x, x.y);
         }
 #pragma unroll
-      for (int i = 0; i < kMT; ++i) {
-        const uint16_t* r = c1_smem + (i * 16 + g) * ld + k0 + 2 * t;
-        const uint32_t a[4] = {*reinterpret_cast<const uint32_t*>(r), *reinterpret_cast<const uint32_t*>(r + 8 * ld),
-                               *reinterpret_cast<const uint32_t*>(r + 8),
-                               *reinterpret_cast<const uint32_t*>(r + 8 * ld + 8)};
+      for (int i = 0; i < kMT; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) mma_bf16(acc[i][j], a, b[j]);
-      }
+        for (int j = 0; j < 2; ++j) {
+          const uint16_t* r = c1_smem + (i * 16 + 8 * j + g) * ld + k0 + 2 * t;
+          const uint32_t b[2] = {*reinterpret_cast<const uint32_t*>(r), *reinterpret_cast<const uint32_t*>(r + 8)};
+          mma_bf16(acc[i][j], a, b);
+        }
     }
 #pragma unroll
-    for (int i = 0; i < kMT; ++i)
+    for (int i = 0; i < kMT; ++i) {
+      const int c = i * 16 + 4 * t;  // first of this thread's four channels
+      const float4 b = *reinterpret_cast<const float4*>(c1_bias + c);
 #pragma unroll
-      for (int j = 0; j < 2; ++j)
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          const int m = m0 + i * 16 + g + (h >= 2 ? 8 : 0), q = n0 + j * 8 + 2 * t + (h & 1);
-          if (m < P.M && q < P.npos) {
-            const int64_t o = (int64_t)q * P.M + m;
-            float v = acc[i][j][h];
-            if (P.bias) v += P.bias[m];
-            if (P.mask && !(P.mask[o] > 0.f)) v = 0.f;
-            P.out[o] = v;
+      for (int h = 0; h < 2; ++h) {
+        const int q = n0 + 8 * h + g;
+        if (q >= P.npos || m0 + c >= P.M) continue;
+        const int64_t o = (int64_t)q * P.M + m0 + c;
+        float v[4] = {acc[i][0][2 * h] + b.x, acc[i][0][2 * h + 1] + b.y, acc[i][1][2 * h] + b.z,
+                      acc[i][1][2 * h + 1] + b.w};
+        if (P.quads) {
+          if (P.mask) {
+            const float4 m = *reinterpret_cast<const float4*>(P.mask + o);
+            if (!(m.x > 0.f)) v[0] = 0.f;
+            if (!(m.y > 0.f)) v[1] = 0.f;
+            if (!(m.z > 0.f)) v[2] = 0.f;
+            if (!(m.w > 0.f)) v[3] = 0.f;
           }
+          *reinterpret_cast<float4*>(P.out + o) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+#pragma unroll
+          for (int l = 0; l < 4; ++l)
+            if (m0 + c + l < P.M) {
+              if (P.mask && !(P.mask[o + l] > 0.f)) v[l] = 0.f;
+              P.out[o + l] = v[l];
+            }
         }
+      }
+    }
   }
 }
 
@@ -1196,8 +1216,9 @@ rpk_status conv(rpk_net* N, const __nv_bfloat16* A, int M, int taps, int Kc, int
   // one tap, 8-byte input pairs, weights that fit the default shared memory
   const int mt = M <= 16 ? 1 : 8;
   const size_t smem = (size_t)mt * 16 * ((Kc + 15) / 16 * 16 + kPadK) * 2;
-  if (taps == 1 && !res && Kc % 2 == 0 && ((uintptr_t)X & 7) == 0 && smem <= 48 * 1024) {
-    Conv1Args P{A, X, out, bias, mask, M, Kc, relu_in, (int)nq};
+  if (taps == 1 && !res && Kc % 2 == 0 && ((uintptr_t)X & 7) == 0 && smem + mt * 64 <= 48 * 1024) {
+    const int quads = M % 4 == 0 && ((uintptr_t)out & 15) == 0 && ((uintptr_t)mask & 15) == 0;
+    Conv1Args P{A, X, out, bias, mask, M, Kc, relu_in, (int)nq, quads};
     const int64_t want = (nq + 16 * (kConv1Threads / 32) - 1) / (16 * (kConv1Threads / 32));
     const dim3 grid((unsigned)std::min<int64_t>(want, 4 * (int64_t)std::max(N->nsm, 1)),
                     (unsigned)((M + mt * 16 - 1) / (mt * 16)));
