@@ -1142,7 +1142,7 @@ struct rpk_net {
   float* dybuf = nullptr;
   double* loss = nullptr;
   int2* qseq = nullptr;        // ragged sequence table, cap_q entries
-  int* starts = nullptr;       // ragged sequence starts, cap_seq + 1 entries
+  int2* starts = nullptr;      // ragged sequences' first position and tile, cap_seq + 1 entries
   int cap_seq = 0;
   int4* tiles = nullptr;       // ragged tensor-core tiles (q0, count, start, length)
   int ntiles = 0, cap_tiles = 0;
@@ -1318,11 +1318,17 @@ rpk_status forward(rpk_net* N, const float* x, int64_t nq, int Lq, const int2* q
               1, y, N->w + head.b_off, nullptr, nullptr, nq, Lq, qseq);
 }
 
-// qseq[q] = (first position, length) of the sequence holding coarse position q;
-// one block per sequence, starts[s] .. starts[s + 1] (coarse positions).
-__global__ void k_fill_qseq(const int* __restrict__ starts, int2* __restrict__ qseq) {
-  const int lo = starts[blockIdx.x], hi = starts[blockIdx.x + 1];
+// qseq[q] = (first position, length) of the sequence holding coarse position q, and
+// the sequence's tensor-core tiles (TC_OUT positions each, the first at index .y); one
+// block per sequence, starts[s].x .. starts[s + 1].x (coarse positions).
+__global__ void k_fill_sequences(const int2* __restrict__ starts, int2* __restrict__ qseq, int4* __restrict__ tiles) {
+  const int2 a = starts[blockIdx.x], b = starts[blockIdx.x + 1];
+  const int lo = a.x, hi = b.x;
   for (int q = lo + threadIdx.x; q < hi; q += blockDim.x) qseq[q] = make_int2(lo, hi - lo);
+  for (int k = threadIdx.x; k < b.y - a.y; k += blockDim.x) {
+    const int q = lo + k * TC_OUT;
+    tiles[a.y + k] = make_int4(q, min(TC_OUT, hi - q), lo, hi - lo);
+  }
 }
 
 // Gradients of every block convolution's weights and biases from the output
@@ -1516,51 +1522,44 @@ rpk_status rpk_net_forward(rpk_net* N, const float* x, int nseq, int len, float*
 rpk_status rpk_net_forward_ragged(rpk_net* N, const float* x, int nseq, const int* lens, float* y) {
   if (!N || !x || !y || !lens) return rpk::fail(RPK_ERR_ARG, "NULL argument");
   if (nseq < 1) return rpk::fail(RPK_ERR_ARG, "nseq must be >= 1");
-  std::vector<int> starts(nseq + 1, 0);
+  std::vector<int2> starts(nseq + 1, make_int2(0, 0));  // first position, first tile
   for (int s = 0; s < nseq; ++s) {
     if (lens[s] < R || lens[s] % R)
       return rpk::fail(RPK_ERR_ARG, "every length must be a positive multiple of 4");
-    if ((int64_t)starts[s] + lens[s] / R > INT32_MAX / 2)
+    const int len = lens[s] / R;
+    if ((int64_t)starts[s].x + len > INT32_MAX / 2)
       return rpk::fail(RPK_ERR_ARG, "too many positions");
-    starts[s + 1] = starts[s] + lens[s] / R;
+    starts[s + 1] = make_int2(starts[s].x + len, starts[s].y + (len + TC_OUT - 1) / TC_OUT);
   }
   RPK_CUDA(cudaSetDevice(N->device));
-  const int64_t nq = starts[nseq];
+  const int64_t nq = starts[nseq].x;
   rpk_status st = ensure_workspace(N, nq);
   if (st != RPK_OK) return st;
   if (nseq > N->cap_seq) {
     cudaFree(N->starts);
     N->starts = nullptr;
     N->cap_seq = 0;
-    st = net_alloc((void**)&N->starts, sizeof(int) * (nseq + 1));
+    st = net_alloc((void**)&N->starts, sizeof(int2) * (nseq + 1));
     if (st != RPK_OK) return st;
     N->cap_seq = nseq;
   }
-  RPK_CUDA(cudaMemcpyAsync(N->starts, starts.data(), sizeof(int) * (nseq + 1),
-                           cudaMemcpyHostToDevice, N->stream));
-  // tensor-core tiles: TC_OUT positions of one sequence each
-  std::vector<int4> tiles;
-  for (int s = 0; s < nseq; ++s)
-    for (int q = starts[s]; q < starts[s + 1]; q += TC_OUT)
-      tiles.push_back(make_int4(q, std::min(TC_OUT, starts[s + 1] - q), starts[s], starts[s + 1] - starts[s]));
-  if ((int)tiles.size() > N->cap_tiles) {
+  N->ntiles = starts[nseq].y;
+  if (N->ntiles > N->cap_tiles) {
     cudaFree(N->tiles);
     N->tiles = nullptr;
     N->cap_tiles = 0;
-    st = net_alloc((void**)&N->tiles, sizeof(int4) * tiles.size());
+    st = net_alloc((void**)&N->tiles, sizeof(int4) * N->ntiles);
     if (st != RPK_OK) return st;
-    N->cap_tiles = (int)tiles.size();
+    N->cap_tiles = N->ntiles;
   }
-  N->ntiles = (int)tiles.size();
-  RPK_CUDA(cudaMemcpyAsync(N->tiles, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice,
-                           N->stream));
-  k_fill_qseq<<<nseq, 256, 0, N->stream>>>(N->starts, N->qseq);
-  RPK_CUDA(cudaGetLastError());
-  st = forward(N, x, nq, 0, N->qseq, y, false);
-  // the host tables are read before they go away
-  if (st == RPK_OK) RPK_CUDA(cudaStreamSynchronize(N->stream));
-  if (st == RPK_OK) st = tc_status(N);
-  return st;
+  RPK_CUDA(cudaMemcpyAsync(N->starts, starts.data(), sizeof(int2) * (nseq + 1), cudaMemcpyHostToDevice, N->stream));
+  k_fill_sequences<<<nseq, 256, 0, N->stream>>>(N->starts, N->qseq, N->tiles);
+  cudaError_t err = cudaGetLastError();
+  if (err == cudaSuccess) st = forward(N, x, nq, 0, N->qseq, y, false);
+  // the table is read before it goes away, also after an error
+  if (err == cudaSuccess && st == RPK_OK) return tc_status(N);
+  cudaStreamSynchronize(N->stream);
+  return st != RPK_OK ? st : rpk::cuda_fail(err, "rpk_net_forward_ragged");
 }
 
 rpk_status rpk_net_loss_grad(rpk_net* N, const float* x, const float* target, const float* mask,
