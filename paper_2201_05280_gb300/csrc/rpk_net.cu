@@ -309,7 +309,11 @@ __global__ void __launch_bounds__(kConv1Threads) k_conv1(Conv1Args P) {
 // points (training, 96 tiles): 2 x 29.9 us -> 18.9 us. Tried: residual rows loaded
 // in the epilogue instead of copied ahead, 1715 against 1685 us a forward pass;
 // TMEM lane = channel with 2-byte stores into B2 and whole-block staging
-// barriers, 1863.
+// barriers, 1863; CTA pairs (M 256 over two SMs, each with half of the weights), 225 us a
+// block as before -- 450 with cluster-scope releases, which wait for the SM's global
+// stores -- since the epilogue's 10 k cycles a tile are the next bound; its residual
+// and output rows as bulk copies of 256 bytes, 223 alone and 220 with pairs; e1 moved
+// to the producers' warps, 260 with pairs.
 constexpr int TC_M = 128, TC_N = 128, TC_KC = 128, TC_TAPS = 5;
 constexpr int TC_OUT = TC_N - (TC_TAPS - 1);               // 124 output positions per tile
 constexpr int TC_ROWS = TC_N + TC_TAPS - 1;                // 132 staged rows
