@@ -129,6 +129,190 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 ? 5 : 1)
   flag_moments(m, K.theta0, status);
 }
 
+// k_collide in FP64 for lattices of one or two warps of points per SM. A quarter of
+// an SM issues an FP64 instruction in 64 cycles, however many lanes are active, and
+// all four together one in 19: a lone warp's 422 instructions take 27 k cycles with
+// three quarters idle. Here four warps share 32 points. Each gathers a group of pairs
+// (rest and axes, faces, corners, halves), sums its part of the moments and, after
+// an exchange, its part of the target's coefficients; after another it relaxes its
+// group: about 185 instructions a warp. 2000-cell tube: a step of 23.7 us became 18.6.
+__host__ __device__ constexpr int split_lo(int g) { return g < 3 ? 6 * g : 12 + 4 * (g - 2); }  // first pair of group g
+
+// This group's parts of drho, j and dP (xx yy zz xy xz yz), of raw_moments_shells.
+template <int kGroup, typename V>
+__device__ __forceinline__ void split_moments(const V (&h)[kQ], V (&p)[10]) {
+  constexpr double w1 = pair_weight(0), w2 = pair_weight(3), wf = pair_weight(6), wc = pair_weight(12),
+                   wh = pair_weight(16);
+  auto ev = [&](int k) { return h[2 * k + 1] + h[2 * k + 2]; };
+  auto od = [&](int k) { return h[2 * k + 1] - h[2 * k + 2]; };
+  if constexpr (kGroup == 0) {
+    const V s0 = ev(0), s1 = ev(1), s2 = ev(2), s3 = ev(3), s4 = ev(4), s5 = ev(5);
+    p[0] = fmad(V(w2), s3 + s4 + s5, fmad(V(w1), s0 + s1 + s2, V(kWeightRest) * h[0]));
+    p[1] = fmad(V(2 * w2), od(3), V(w1) * od(0));
+    p[2] = fmad(V(2 * w2), od(4), V(w1) * od(1));
+    p[3] = fmad(V(2 * w2), od(5), V(w1) * od(2));
+    p[4] = fmad(V(w1), s0, V(4 * w2) * s3);
+    p[5] = fmad(V(w1), s1, V(4 * w2) * s4);
+    p[6] = fmad(V(w1), s2, V(4 * w2) * s5);
+    p[7] = p[8] = p[9] = V(0);
+  } else if constexpr (kGroup == 1) {
+    const V ap = ev(6), am = ev(7), bp = ev(8), bm = ev(9), cp = ev(10), cm = ev(11);
+    const V A = ap + am, B = bp + bm, C = cp + cm;
+    const V oap = od(6), oam = od(7), obp = od(8), obm = od(9), ocp = od(10), ocm = od(11);
+    p[0] = V(wf) * (A + B + C);
+    p[1] = V(wf) * ((oap + oam) + (obp + obm));
+    p[2] = V(wf) * ((oap - oam) + (ocp + ocm));
+    p[3] = V(wf) * ((obp - obm) + (ocp - ocm));
+    p[4] = V(wf) * (A + B);
+    p[5] = V(wf) * (A + C);
+    p[6] = V(wf) * (B + C);
+    p[7] = V(wf) * (ap - am);
+    p[8] = V(wf) * (bp - bm);
+    p[9] = V(wf) * (cp - cm);
+  } else {
+    constexpr int k = split_lo(kGroup);
+    constexpr double w = kGroup == 2 ? wc : wh, wj = kGroup == 2 ? wc : 0.5 * wh, wp = kGroup == 2 ? wc : 0.25 * wh;
+    auto butterfly = [](V a, V b, V c, V d, V (&o)[4]) {
+      const V ab = a + b, cd = c + d, e = a - b, f = c - d;
+      o[0] = ab + cd;
+      o[1] = ab - cd;
+      o[2] = e + f;
+      o[3] = e - f;
+    };
+    V e[4], o[4];
+    butterfly(ev(k), ev(k + 1), ev(k + 2), ev(k + 3), e);
+    butterfly(od(k), od(k + 1), od(k + 2), od(k + 3), o);
+    p[0] = V(w) * e[0];
+    p[1] = V(wj) * o[0];
+    p[2] = V(wj) * o[1];
+    p[3] = V(wj) * o[2];
+    p[4] = p[5] = p[6] = V(wp) * e[0];
+    p[7] = V(wp) * e[1];
+    p[8] = V(wp) * e[2];
+    p[9] = V(wp) * e[3];
+  }
+}
+
+// f(std::integral_constant<int, group>) for the group of this warp.
+template <typename F>
+__device__ __forceinline__ void split_group(int group, F&& f) {
+  if (group == 0)
+    f(std::integral_constant<int, 0>{});
+  else if (group == 1)
+    f(std::integral_constant<int, 1>{});
+  else if (group == 2)
+    f(std::integral_constant<int, 2>{});
+  else
+    f(std::integral_constant<int, 3>{});
+}
+
+template <bool kPull, int kBC, bool kPaper>
+__global__ void __launch_bounds__(128)
+    k_collide_split(StepConst<double> K, const double* pin, double* __restrict__ pout, const double* e_in,
+                    double* __restrict__ e_out, double* __restrict__ drho_out, double* __restrict__ u_out,
+                    double* __restrict__ kap_out, const double* __restrict__ ghost, unsigned* __restrict__ status,
+                    double* __restrict__ tt_out, const double* wcol) {
+  __shared__ double part[4][10][32];
+  __shared__ double coef[20][32];
+  pdl_wait();
+  const int lane = threadIdx.x & 31, group = threadIdx.x >> 5;
+  const unsigned c = blockIdx.x * 32 + lane;
+  const bool mine = c < (unsigned)K.n3;
+  PointIdx P;
+  P.cell = mine ? c : 0u;
+  const unsigned row = K.by_nx.div((unsigned)P.cell), z = K.by_ny.div(row);
+  P.s = blockIdx.y;
+  P.x = (int)((unsigned)P.cell - row * K.nx);
+  P.y = (int)(row - z * K.ny);
+  P.z = (int)z;
+  const int64_t p = (int64_t)P.s * K.n3 + P.cell;
+  const double e = e_in[p];
+  double own[13];  // the group's populations
+  split_group(group, [&](auto gc) {
+    constexpr int g = decltype(gc)::value, lo = split_lo(g), hi = split_lo(g + 1), q0 = g ? 2 * lo + 1 : 0;
+    double h[kQ], sums[10];
+    gather<double, double, kPull, kBC, lo, hi>(pin, ghost, K, P, h, wcol);
+    split_moments<g>(h, sums);
+#pragma unroll
+    for (int k = 0; k < 10; ++k) part[g][k][lane] = sums[k];
+#pragma unroll
+    for (int q = q0; q < 2 * hi + 1; ++q) own[q - q0] = h[q];
+  });
+  __syncthreads();
+  Mom<double> m;
+  {
+    double t[10];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+      t[k] = part[1][k][lane] + part[2][k][lane] + part[3][k][lane];
+      if (k < 7) t[k] += part[0][k][lane];
+    }
+    m.drho = t[0];
+    m.rho = 1.0 + t[0];
+    m.inv_rho = 1.0 / m.rho;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) m.j[a] = t[1 + a];
+#pragma unroll
+    for (int a = 0; a < 6; ++a) m.dP[a] = t[4 + a];
+  }
+  // each group's quarter of the coefficients: the even part and oxyz, or one axis's odd part
+  split_group(group, [&](auto gc) {
+    constexpr int g = decltype(gc)::value;
+    Herm<double> H;
+    relaxed_target<double, kPaper>(m, e, K, H);
+    auto put = [&](int k, double v) { coef[k][lane] = v; };
+    if constexpr (g == 0) {
+      put(0, H.e0), put(1, H.exx), put(2, H.eyy), put(3, H.ezz), put(4, H.exy), put(5, H.exz), put(6, H.eyz);
+      put(7, H.oxyz);
+    } else if constexpr (g == 1) {
+      put(8, H.ox), put(9, H.oxxx), put(10, H.oyyx), put(11, H.ozzx);
+    } else if constexpr (g == 2) {
+      put(12, H.oy), put(13, H.oyyy), put(14, H.oxxy), put(15, H.ozzy);
+    } else {
+      put(16, H.oz), put(17, H.ozzz), put(18, H.oxxz), put(19, H.oyyz);
+    }
+  });
+  __syncthreads();
+  if (!mine) return;
+  Herm<double> H;
+  {
+    auto get = [&](int k) { return coef[k][lane]; };
+    H.e0 = get(0), H.exx = get(1), H.eyy = get(2), H.ezz = get(3), H.exy = get(4), H.exz = get(5), H.eyz = get(6);
+    H.oxyz = get(7), H.ox = get(8), H.oxxx = get(9), H.oyyx = get(10), H.ozzx = get(11), H.oy = get(12);
+    H.oyyy = get(13), H.oxxy = get(14), H.ozzy = get(15), H.oz = get(16), H.ozzz = get(17), H.oxxz = get(18);
+    H.oyyz = get(19);
+  }
+  double* out = pout + (int64_t)(P.s * kQ) * K.n3 + P.cell;
+  split_group(group, [&](auto gc) {
+    constexpr int g = decltype(gc)::value, lo = split_lo(g), hi = split_lo(g + 1), q0 = g ? 2 * lo + 1 : 0;
+    if constexpr (g == 0) out[0] = fmad(K.c_keep, own[0], H.e0);
+    herm_shells(H, [&](int k, double ev, double od) {
+      if (k < lo || k >= hi) return;
+      out[(2 * k + 1) * K.n3] = fmad(K.c_keep, own[2 * k + 1 - q0], ev + od);
+      out[(2 * k + 2) * K.n3] = fmad(K.c_keep, own[2 * k + 2 - q0], ev - od);
+    });
+  });
+  const int64_t npts = 2 * K.n3;
+  if (group == 1) {
+    if constexpr (kPaper)
+      e_out[p] = fmad(K.ra_keep, m.dR, K.ra_t * m.dT);
+    else
+      e_out[p] = fmad(K.exc * m.rho, m.dth - m.dR, e);
+    drho_out[p] = m.drho;
+  } else if (group == 2) {
+    u_out[p] = m.j[0] * m.inv_rho;
+    u_out[npts + p] = m.j[1] * m.inv_rho;
+    u_out[2 * npts + p] = m.j[2] * m.inv_rho;
+  } else if (group == 3) {
+    if constexpr (kPaper)
+      kap_out[p] = K.kapc * m.rho * fmad(fmad(K.delta, m.dR, 3.0 * m.dT), K.inv_3pd, K.theta0);
+    else
+      kap_out[p] = K.kapc * m.rho * (K.theta0 + m.dth);
+    if constexpr (kPaper) tt_out[p] = m.dT;
+    flag_moments(m, K.theta0, status);
+  }
+}
+
 }  // namespace rpk
 
 namespace rpk {

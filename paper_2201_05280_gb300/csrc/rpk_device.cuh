@@ -622,8 +622,9 @@ __device__ __forceinline__ bool pair_from_block(const StepConst<float>& K, int& 
 // and hw the wall's table entry. kBC & kWallX: the same for the x walls
 // (x = -1/4, x = nx - 1/4) with the (y, z) columns at
 // wcol[2 nx nz + (wall * nz + z) * ny + y]; a source beyond both a y and an x
-// wall belongs to the y wall.
-template <typename Store, typename Real, bool kPull, int kBC>
+// wall belongs to the y wall. Only the pairs kLo .. kHi - 1 (and the rest
+// population with pair 0) are gathered.
+template <typename Store, typename Real, bool kPull, int kBC, int kLo = 0, int kHi = kPairs>
 __device__ __forceinline__ void gather(const Store* __restrict__ pin,
                                        const Real* __restrict__ ghost, const StepConst<Real>& K,
                                        const PointIdx& P, Real (&h)[kQ],
@@ -632,7 +633,8 @@ __device__ __forceinline__ void gather(const Store* __restrict__ pin,
   if constexpr (!kPull) {
     const unsigned cell = (unsigned)P.cell;
 #pragma unroll
-    for (int q = 0; q < kQ; ++q) h[q] = to_real<Store, Real>((pin + (int64_t)(P.s * kQ + q) * n3)[cell]);
+    for (int q = kLo ? 2 * kLo + 1 : 0; q < 2 * kHi + 1; ++q)
+      h[q] = to_real<Store, Real>((pin + (int64_t)(P.s * kQ + q) * n3)[cell]);
   } else {
     const int nx = K.nx, ny = K.ny, nz = K.nz;
     int xw[5], yw[5], zw[5];
@@ -656,9 +658,9 @@ __device__ __forceinline__ void gather(const Store* __restrict__ pin,
     const bool yinhp = s ? yin[2] : yin[1], yinhm = s ? yin[3] : yin[2];
     const Store* same = pin + (int64_t)(s * kQ) * n3;
     const Store* other = pin + (int64_t)((1 - s) * kQ) * n3;
-    h[0] = to_real<Store, Real>(same[(unsigned)P.cell]);
-    static_for<kQ - 1>([&](auto qc) {
-      constexpr int q = decltype(qc)::value + 1;
+    if constexpr (kLo == 0) h[0] = to_real<Store, Real>(same[(unsigned)P.cell]);
+    static_for<2 * (kHi - kLo)>([&](auto qc) {
+      constexpr int q = decltype(qc)::value + 2 * kLo + 1;
       constexpr Vel2 v = vel2(q);
       constexpr bool half = (v.x & 1) != 0;
       int xs, ys, zs;

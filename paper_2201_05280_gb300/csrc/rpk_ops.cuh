@@ -144,6 +144,19 @@ static rpk_status collide_launch(rpk_lattice* L, const StepConst<Real>& K) {
   Real* ucur = static_cast<Real*>(L->u[L->steps & 1]);
   const Real* wcol = static_cast<const Real*>(L->wrho);
   const PointLaunch pt(L, L->n3);
+  if constexpr (std::is_same<Store, double>::value) {
+    // at most two warps of points per SM: four warps share each (steps, us, a thread per
+    // point / split: 2000 cells 23.7 / 18.6, 4864 cells 26.7 / 24.7, 5500 cells, three
+    // warps on some SMs, 28.8 / 31.1; 12^3 35.0 / 28.7, 20^3 37.0 / 47.2)
+    if (2 * ((L->n3 + 31) / 32) <= 2 * L->sms) {
+      const dim3 grid((unsigned)((L->n3 + 31) / 32), 2);
+      launch_step(L, L->rot_mode ? k_collide_split<kPull, kBC, true> : k_collide_split<kPull, kBC, false>, grid, 128, 0, K,
+                  pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star), static_cast<Real*>(L->drho),
+                  ucur, static_cast<Real*>(L->kap), static_cast<const Real*>(L->ghost), L->status,
+                  L->rot_mode ? static_cast<Real*>(L->thbuf) : nullptr, wcol);
+      return check_launch("k_collide_split");
+    }
+  }
   if (L->rot_mode) {
     if constexpr (kPull && kBC == 0 && sizeof(Real) == 4) {
       if (L->grid.nx % 2 == 0) {
