@@ -92,11 +92,25 @@ static inline rpk_status check_launch(const char* what) {
   return RPK_OK;
 }
 
+// FP64 lattices of at most two warps of points per SM: four warps share each
+// (k_collide_split; steps, us, a thread per point / split: 2000 cells 23.7 / 18.6, 4864
+// cells 26.7 / 24.7, 5500 cells, three warps on some SMs, 28.8 / 31.1; 12^3 35.0 / 28.7,
+// 20^3 37.0 / 47.2).
+static inline bool split_groups(const rpk_lattice* L) {
+  return L->store_elem == 8 && 2 * ((L->n3 + 31) / 32) <= 2 * (int64_t)L->sms;
+}
+
 // Launch a kernel of the step so that its blocks may become resident while the
 // previous kernel of the stream still runs (it waits in pdl_wait): 32^3 FP32 21.4
-// -> 17.4 us a step of four kernels. FP64 keeps ordinary launches: its pipe is
-// the bound, and blocks placed beside a running kernel's share SMs that would
-// otherwise have had one each (2000-cell tube: 27.7 against 30.5 us a step).
+// -> 17.4 us a step of four kernels. Larger FP64 lattices keep ordinary launches: their
+// pipe is the bound, and blocks placed beside a running kernel's share SMs that would
+// otherwise have had fewer (ordinary / overlapping, us a step: 1000 cells 16.5 / 13.1,
+// 12^3 28.8 / 25.1, 20^3 with 8 sub-steps 80 / 60, 26^3 59.5 / 52.6; but 36^3 125 / 136
+// and, one thread a point of a line, 5500 cells 28.8 / 38.1).
+static inline bool overlap_launches(const rpk_lattice* L) {
+  return L->real_elem == 4 || split_groups(L) || (L->grid.ny * L->grid.nz > 1 && L->n3 <= 128 * (int64_t)L->sms);
+}
+
 template <typename... KArgs, typename... Args>
 static void launch_step(rpk_lattice* L, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, Args... args) {
   cudaLaunchConfig_t c{};
@@ -108,7 +122,7 @@ static void launch_step(rpk_lattice* L, void (*kernel)(KArgs...), dim3 grid, dim
   a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   a.val.programmaticStreamSerializationAllowed = 1;
   c.attrs = &a;
-  c.numAttrs = L->real_elem == 4 ? 1 : 0;
+  c.numAttrs = overlap_launches(L) ? 1 : 0;
   cudaLaunchKernelEx(&c, kernel, static_cast<KArgs>(args)...);
 }
 
@@ -145,10 +159,7 @@ static rpk_status collide_launch(rpk_lattice* L, const StepConst<Real>& K) {
   const Real* wcol = static_cast<const Real*>(L->wrho);
   const PointLaunch pt(L, L->n3);
   if constexpr (std::is_same<Store, double>::value) {
-    // at most two warps of points per SM: four warps share each (steps, us, a thread per
-    // point / split: 2000 cells 23.7 / 18.6, 4864 cells 26.7 / 24.7, 5500 cells, three
-    // warps on some SMs, 28.8 / 31.1; 12^3 35.0 / 28.7, 20^3 37.0 / 47.2)
-    if (2 * ((L->n3 + 31) / 32) <= 2 * L->sms) {
+    if (split_groups(L)) {
       const dim3 grid((unsigned)((L->n3 + 31) / 32), 2);
       launch_step(L, L->rot_mode ? k_collide_split<kPull, kBC, true> : k_collide_split<kPull, kBC, false>, grid, 128, 0, K,
                   pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star), static_cast<Real*>(L->drho),
