@@ -380,34 +380,34 @@ __device__ __forceinline__ void hermite(V drho, V rho, V inv_rho, const V (&j)[3
 template <typename V>
 __device__ __forceinline__ void hermite_iso(V drho, V rho, V inv_rho, const V (&j)[3], V D, Herm<V>& H) {
   using S = scalar_t<V>;
-  constexpr double i1 = 1.0 / kTheta0, i2 = i1 * i1, i3 = i2 * i1;
+  constexpr S i1 = S(1) / S(kTheta0), i2 = i1 * i1, i3 = i2 * i1;
   const V jx = j[0], jy = j[1], jz = j[2];
   const V ux = jx * inv_rho, uy = jy * inv_rho, uz = jz * inv_rho;
   const V xx = jx * ux, yy = jy * uy, zz = jz * uz, xy = jx * uy;
   const V rD = rho * D, Dx = D * jx, Dy = D * jy, Dz = D * jz;
-  H.e0 = fmad(S(-0.5 * i1), (xx + yy + zz) + S(3) * rD, drho);
-  H.exx = S(0.5 * i2) * (xx + rD);
-  H.eyy = S(0.5 * i2) * (yy + rD);
-  H.ezz = S(0.5 * i2) * (zz + rD);
-  H.exy = S(i2) * xy;
-  H.exz = S(i2) * (jx * uz);
-  H.eyz = S(i2) * (jy * uz);
+  H.e0 = fmad(S(-0.5) * i1, (xx + yy + zz) + S(3) * rD, drho);
+  H.exx = S(0.5) * i2 * (xx + rD);
+  H.eyy = S(0.5) * i2 * (yy + rD);
+  H.ezz = S(0.5) * i2 * (zz + rD);
+  H.exy = i2 * xy;
+  H.exz = i2 * (jx * uz);
+  H.eyz = i2 * (jy * uz);
   const V xxx = fmad(xx, ux, S(3) * Dx), yyy = fmad(yy, uy, S(3) * Dy), zzz = fmad(zz, uz, S(3) * Dz);
   const V xxy = fmad(xx, uy, Dy), xxz = fmad(xx, uz, Dz), yyx = fmad(yy, ux, Dx), yyz = fmad(yy, uz, Dz),
           zzx = fmad(zz, ux, Dx), zzy = fmad(zz, uy, Dy);
-  H.ox = fmad(S(-0.5 * i2), xxx + yyx + zzx, S(i1) * jx);
-  H.oy = fmad(S(-0.5 * i2), xxy + yyy + zzy, S(i1) * jy);
-  H.oz = fmad(S(-0.5 * i2), xxz + yyz + zzz, S(i1) * jz);
-  H.oxxx = S(i3 / 6.0) * xxx;
-  H.oyyy = S(i3 / 6.0) * yyy;
-  H.ozzz = S(i3 / 6.0) * zzz;
-  H.oxxy = S(0.5 * i3) * xxy;
-  H.oxxz = S(0.5 * i3) * xxz;
-  H.oyyx = S(0.5 * i3) * yyx;
-  H.oyyz = S(0.5 * i3) * yyz;
-  H.ozzx = S(0.5 * i3) * zzx;
-  H.ozzy = S(0.5 * i3) * zzy;
-  H.oxyz = S(i3) * (xy * uz);
+  H.ox = fmad(S(-0.5) * i2, xxx + yyx + zzx, i1 * jx);
+  H.oy = fmad(S(-0.5) * i2, xxy + yyy + zzy, i1 * jy);
+  H.oz = fmad(S(-0.5) * i2, xxz + yyz + zzz, i1 * jz);
+  H.oxxx = i3 * S(1.0 / 6.0) * xxx;
+  H.oyyy = i3 * S(1.0 / 6.0) * yyy;
+  H.ozzz = i3 * S(1.0 / 6.0) * zzz;
+  H.oxxy = S(0.5) * i3 * xxy;
+  H.oxxz = S(0.5) * i3 * xxz;
+  H.oyyx = S(0.5) * i3 * yyx;
+  H.oyyz = S(0.5) * i3 * yyz;
+  H.ozzx = S(0.5) * i3 * zzx;
+  H.ozzy = S(0.5) * i3 * zzy;
+  H.oxyz = i3 * (xy * uz);
 }
 
 template <int VX, int VY, int VZ, typename V>
@@ -510,7 +510,9 @@ __device__ __forceinline__ void mix_coeffs(const Mom<V>& m, const StepConst<Real
 // stored rotational value, the f-level temperatures in m and the coefficients of
 // c_relax (f^mix/w - 1) in H. The products j_a u_b serve the temperature, the
 // stress and both orders of the expansion, and products of constants come from
-// the launch (about 130 operations instead of 240).
+// the launch (about 130 operations instead of 240). For FP64: the products of
+// constants, rounded to FP32, would shift an FP32 state's total momentum and mass by
+// parts in 1e8 a step.
 template <typename Real, bool kPaper, typename V>
 __device__ __forceinline__ void relaxed_target(Mom<V>& m, V e, const StepConst<Real>& K, Herm<V>& H) {
   using S = scalar_t<V>;
