@@ -470,7 +470,7 @@ def run_surrogate(args):
             "surrogate_parts_ms": dict(zip(("network", "spot_checks", "final_lbm", "reruns"), res["ms"].tolist())),
             "l1": {"mean": float(l1.mean()), "p90": float(np.percentile(l1, 90)), "max": float(l1.max()),
                    "frac_le_1pct": float((l1 <= 0.01).mean())},
-            "roofline": {"bound": "tensor", "kernel": "network forward (k_conv_tc + k_conv)",
+            "roofline": {"bound": "tensor", "kernel": "network forward (k_block_tc + k_conv1)",
                          "achieved": fwd_tflops, "peak": peak[0], "unit": "TFLOP/s",
                          "frac": fwd_tflops / peak[0], "peak_source": peak[1],
                          "flop_per_coarse_position": flop_pos, "positions": coarse,

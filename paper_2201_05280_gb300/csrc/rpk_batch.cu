@@ -10,7 +10,7 @@
 // and the FTCS sub-steps) costs no device-memory traffic. Tubes need no
 // synchronisation with each other, so the launch has no grid-wide barrier. The
 // arithmetic is that of the lattice kernels (k_collide, k_mac_pred,
-// k_mac_corr, k_ftcs_first, k_ftcs) on an nx x 1 x 1 grid, where every y and z
+// k_mac_corr, k_ftcs) on an nx x 1 x 1 grid, where every y and z
 // neighbour is the point itself and contributes exact zeros.
 #include <algorithm>
 #include <cmath>

@@ -47,13 +47,7 @@ __device__ __forceinline__ V collide_shells(const StepConst<Real>& K, const V (&
                                             Mom<V>& m) {
   raw_moments_shells(h, m);
   Herm<V> H;
-  if constexpr (sizeof(Real) == 8) {
-    relaxed_target<Real, kPaper>(m, e, K, H);
-  } else {
-    recover<Real, kPaper, true>(m, e, K);
-    mix_coeffs(m, K, H);
-    herm_scale(H, K.c_relax);
-  }
+  relaxed_target<Real, kPaper>(m, e, K, H);
   emit(0, fmad(K.c_keep, h[0], H.e0));
   herm_shells(H, [&](int k, V ev, V od) {
     emit(2 * k + 1, fmad(K.c_keep, h[2 * k + 1], ev + od));

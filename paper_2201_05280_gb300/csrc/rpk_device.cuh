@@ -261,9 +261,11 @@ __device__ __forceinline__ void raw_moments_shells(const V (&h)[kQ], Mom<V>& m) 
   m.dP[5] = fmad(whp, he[3], fmad(wc, ce[3], wf * (cp - cm)));
 }
 
-// Storage whose one-point kernels use the factored sums and targets.
+// Storage whose one-point kernels use the factored sums and targets: FP64. FP32 and
+// 16-bit lattices keep the rounding of the pair-by-pair form: the totals of a state
+// follow it to parts in 1e8 a step.
 template <typename Store>
-constexpr bool kShells = sizeof(Store) > 2;
+constexpr bool kShells = sizeof(Store) == 8;
 
 // f-level moments from g (Sec. 5, g/f relations) and the stored auxiliary
 // rotational energy e (deviation) -- or, in paper mode, the stored theta_R:
@@ -510,9 +512,8 @@ __device__ __forceinline__ void mix_coeffs(const Mom<V>& m, const StepConst<Real
 // stored rotational value, the f-level temperatures in m and the coefficients of
 // c_relax (f^mix/w - 1) in H. The products j_a u_b serve the temperature, the
 // stress and both orders of the expansion, and products of constants come from
-// the launch (about 130 operations instead of 240). For FP64: the products of
-// constants, rounded to FP32, would shift an FP32 state's total momentum and mass by
-// parts in 1e8 a step.
+// the launch (about 130 operations instead of 240). FP64 lattices and the batched
+// tubes use it; FP32 lattices keep the other rounding, as their totals do then.
 template <typename Real, bool kPaper, typename V>
 __device__ __forceinline__ void relaxed_target(Mom<V>& m, V e, const StepConst<Real>& K, Herm<V>& H) {
   using S = scalar_t<V>;

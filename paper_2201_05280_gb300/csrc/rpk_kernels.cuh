@@ -686,14 +686,11 @@ __global__ void __launch_bounds__(kTBX * kTBY)
 // g = f - (dt/2) Omega(f) with Omega = (f^Eq(rho, u, theta I) - f)/tau1 (the ES
 // term vanishes since sigma = 0), Er = E_R - (dt/2)(delta rho/2)(theta - theta_R)/tau1.
 // Outputs h = g/w - 1 and e = Er - delta theta0/2.
-// kSum: one expansion of the two targets' combined coefficients, shell by shell,
-// instead of two (half the operations; not for 16-bit storage, whose stored bits
-// depend on the rounding). In FP64 one isotropic expansion: f and f^Eq share rho and u
-// and the coefficients are linear in Lambda, so g/w - 1 = (1 + a) f/w - a fEq/w - 1,
-// a = dt/(2 tau1), is the expansion about theta_T + a (theta_T - theta). In FP32 the
-// first collision's rounding would follow that of the initial state and shift the
-// total momentum by a part in 1e7. 96^3 FP64: 2115 us pair by pair, 975 with
-// both expansions' coefficients combined, 677 now.
+// kSum (FP64 lattices, batched tubes): one isotropic expansion, shell by shell. f and
+// f^Eq share rho and u and the coefficients are linear in Lambda, so g/w - 1 = (1 + a)
+// f/w - a fEq/w - 1, a = dt/(2 tau1), is the expansion about theta_T + a (theta_T -
+// theta). FP32 and 16-bit lattices keep the rounding of the two expansions. 96^3 FP64:
+// 2115 us pair by pair, 975 with both expansions' coefficients combined, 677 now.
 template <typename Real, bool kSum = false>
 __device__ __forceinline__ void init_point(const StepConst<Real>& K, Real half_dt_over_tau1,
                                            double rho_d, double ux, double uy, double uz,
@@ -705,7 +702,7 @@ __device__ __forceinline__ void init_point(const StepConst<Real>& K, Real half_d
   const Real dR = round_to<Real>(R - to_double(K.theta0));
   const Real dth = (Real(3) * dT + K.delta * dR) * K.inv_3pd;
   const Real j[3] = {rho * round_to<Real>(ux), rho * round_to<Real>(uy), rho * round_to<Real>(uz)};
-  if constexpr (kSum && sizeof(Real) == 8) {
+  if constexpr (kSum) {
     Herm<Real> H;
     hermite_iso(drho, rho, inv_rho, j, fmad(half_dt_over_tau1, dT - dth, dT), H);
     h[0] = H.e0;
@@ -720,28 +717,16 @@ __device__ __forceinline__ void init_point(const StepConst<Real>& K, Real half_d
     hermite(drho, rho, inv_rho, j, Df, K.theta0, Hf);
     hermite(drho, rho, inv_rho, j, De, K.theta0, He);
     // g/w - 1 = (f/w - 1) - (dt/(2 tau1)) ((fEq/w - 1) - (f/w - 1))
-    if constexpr (kSum) {
-      Real* f = reinterpret_cast<Real*>(&Hf);
-      const Real* q = reinterpret_cast<const Real*>(&He);
-#pragma unroll
-      for (int i = 0; i < (int)(sizeof(Hf) / sizeof(Real)); ++i) f[i] = f[i] - half_dt_over_tau1 * (q[i] - f[i]);
-      h[0] = Hf.e0;
-      herm_shells(Hf, [&](int k, Real ev, Real od) {
-        h[2 * k + 1] = ev + od;
-        h[2 * k + 2] = ev - od;
-      });
-    } else {
-      h[0] = Hf.e0 - half_dt_over_tau1 * (He.e0 - Hf.e0);
-      static_for<kPairs>([&](auto kc) {
-        constexpr int k = decltype(kc)::value;
-        constexpr Vel2 v = kPairVel2[k];
-        const Real fe = herm_even<v.x, v.y, v.z>(Hf), fo = herm_odd<v.x, v.y, v.z>(Hf);
-        const Real ee = herm_even<v.x, v.y, v.z>(He), eo = herm_odd<v.x, v.y, v.z>(He);
-        const Real fp = fe + fo, fm = fe - fo, qp = ee + eo, qm = ee - eo;
-        h[2 * k + 1] = fp - half_dt_over_tau1 * (qp - fp);
-        h[2 * k + 2] = fm - half_dt_over_tau1 * (qm - fm);
-      });
-    }
+    h[0] = Hf.e0 - half_dt_over_tau1 * (He.e0 - Hf.e0);
+    static_for<kPairs>([&](auto kc) {
+      constexpr int k = decltype(kc)::value;
+      constexpr Vel2 v = kPairVel2[k];
+      const Real fe = herm_even<v.x, v.y, v.z>(Hf), fo = herm_odd<v.x, v.y, v.z>(Hf);
+      const Real ee = herm_even<v.x, v.y, v.z>(He), eo = herm_odd<v.x, v.y, v.z>(He);
+      const Real fp = fe + fo, fm = fe - fo, qp = ee + eo, qm = ee - eo;
+      h[2 * k + 1] = fp - half_dt_over_tau1 * (qp - fp);
+      h[2 * k + 2] = fm - half_dt_over_tau1 * (qm - fm);
+    });
   }
   // E_R = delta rho theta_R/2 as a deviation from delta theta0/2 (paper mode:
   // the state is theta_R - theta0)

@@ -10,9 +10,13 @@
 //   shuffle   (L/4, 4 Cout) -> (L, Cout)
 // Tensors are FP32 in memory, position-major ([position][channel]); every
 // contraction runs on the tensor cores with BF16 operands (converted while a
-// tile is staged in shared memory) and FP32 accumulation (mma.sync m16n8k16).
+// tile is staged in shared memory) and FP32 accumulation.
 //
-//   k_conv     out[q][m] = (sum_{t,j} A[m][t][j] * act(X[q + s (t - c)][j]) + bias)
+//   k_block_tc a whole residual block or its input gradient (tcgen05; C = 128)
+//   k_dw_tc    all blocks' weight and bias gradients in one launch (tcgen05; C = 128)
+//   k_conv1    one-tap layers (mma.sync m16n8k16)
+//   k_conv     the other layers and widths (mma.sync):
+//              out[q][m] = (sum_{t,j} A[m][t][j] * act(X[q + s (t - c)][j]) + bias)
 //              x (mask > 0) + residual; s = +1 forward, s = -1 input gradient
 //              (A = W transposed per tap), zero outside each sequence
 //   k_conv_dw  dW[o][t][i] += sum_q dY[q][o] * act(X[q + t - c][i])  (split over q)
