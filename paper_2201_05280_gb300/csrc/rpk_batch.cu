@@ -701,7 +701,7 @@ __global__ void k_batch_moments(const TubeDev<Real>* __restrict__ tubes, const S
       gather<Store, Real, true, 1>(pin, tb->ghost, K, P, h);
     Mom<Real> m;
     raw_moments_shells(h, m);
-    recover<Real, false, true>(m, e_state[off + p], K);
+    recover(m, e_state[off + p], K);
     const int64_t g = off + p;
     const double rh = 1.0 + to_double(m.drho), thR = to_double(K.theta0) + to_double(m.dR);
     out[g] = rh;

@@ -131,7 +131,6 @@ struct StepConst {
   Real exc;       // dt delta / (2 tau1)
   Real kapc;      // k_r 5 tau / (2 B), kappa_R = kapc * rho * theta
   Real E0;        // delta theta0 / 2
-  Real inv_delta; // 1 / delta
   // products of the above for the shell-wise collision (i = 1 / theta0)
   Real two_id;    // 2 / delta
   Real c_d, c_3;  // delta / (3 + delta), 3 / (3 + delta)
@@ -277,7 +276,7 @@ constexpr bool kShells = sizeof(Store) == 8;
 //   D = (theta_T(g) - Rt)/(1 + dt/(2 tau1)) = theta_T(f) - theta_R
 //   theta_T(f) = theta + delta D/(3 + delta),  theta_R = theta - 3 D/(3 + delta)
 //   sigma(f) = (P - jj/rho - rho theta_T(g) I)/(1 + dt/(2 tau*) - b dt/(2 tau))
-template <typename Real, bool kPaper = false, bool kInv = false, typename V>
+template <typename Real, bool kPaper = false, typename V>
 __device__ __forceinline__ void recover(Mom<V>& m, V e, const StepConst<Real>& K) {
   using S = scalar_t<V>;
   const S t0 = K.theta0;
@@ -290,11 +289,7 @@ __device__ __forceinline__ void recover(Mom<V>& m, V e, const StepConst<Real>& K
     m.dT = fmad(K.pa, m.dR, m.dTg) * K.inv_1pa;
     m.dth = fmad(K.delta, m.dR, S(3) * m.dT) * K.inv_3pd;
   } else {
-    V dRt = (S(2) * e - K.delta * t0 * m.drho) * m.inv_rho;
-    if constexpr (kInv)  // a product where the last bit is free
-      dRt = dRt * K.inv_delta;
-    else
-      dRt = dRt / K.delta;
+    const V dRt = (S(2) * e - K.delta * t0 * m.drho) * m.inv_rho / K.delta;
     m.dth = fmad(K.delta, dRt, S(3) * m.dTg) * K.inv_3pd;
     const V D = (m.dTg - dRt) * K.inv_d;
     m.dT = fmad(K.delta * K.inv_3pd, D, m.dth);

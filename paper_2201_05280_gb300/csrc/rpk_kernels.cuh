@@ -830,9 +830,9 @@ __global__ void __launch_bounds__(128)
   Mom<Real> m;
   raw_moments_shells(h, m);
   if (K.paper)
-    recover<Real, true, true>(m, e_in[p], K);
+    recover<Real, true>(m, e_in[p], K);
   else
-    recover<Real, false, true>(m, e_in[p], K);
+    recover<Real, false>(m, e_in[p], K);
   const double rho = 1.0 + to_double(m.drho), R = to_double(K.theta0) + to_double(m.dR);
   if (rho_o) rho_o[p] = rho;
   if (u_o) {
@@ -993,33 +993,26 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(Real) == 4 ? 4 : 1)
   diag_block_reduce(acc, partial);
 }
 
-// A running sum of two lanes in two FP32 words each (the rounding error of every
-// addition is kept exactly): 48 bits without the FP64 pipe, which issues two
-// lanes per cycle and SM. On 256^3 points its sums are those of FP64 additions to
-// 1e-13 of the sum of magnitudes, below the FP32 rounding of the terms.
-struct Sum2 {
-  F2 hi, lo;
-  __device__ __forceinline__ Sum2() : hi(0.f), lo(0.f) {}
-  __device__ __forceinline__ void add(F2 x) {
-    const F2 t = hi + x;
-    const F2 z = t - hi;
-    lo += (hi - (t - z)) + (x - z);
-    hi = t;
-  }
-  __device__ __forceinline__ double value() const {
-    return ((double)hi.v.x + (double)hi.v.y) + ((double)lo.v.x + (double)lo.v.y);
-  }
-};
+// x times 2^-896, exactly, for finite x: the bits of an FP32 value moved into an FP64
+// one's exponent and fraction fields, subnormals and zeros included. Three integer
+// operations, where a conversion takes the FP64 pipe.
+__device__ __forceinline__ double widen_scaled(float x) {
+  const unsigned b = __float_as_uint(x);
+  return __hiloint2double((int)((unsigned)((int)b >> 3) & 0x8fffffffu), (int)(b << 29));
+}
 
 // k_diag for two x-adjacent points per thread (periodic pull, FP32
 // arithmetic, nx even; kPaper: the state holds theta_R as in the paper's
 // solver): the moments and targets in packed FP32x2 form. Thread t handles pair
 // t of the field planes (sublattice t / (n3/2)).
-// Bound before: the FP64 pipe (12 additions and 9 conversions a point) and six
-// operations around each of the 41 logarithms; 256^3: 2.98 ms. Now the sums are
-// two-word FP32 (Sum2), sum f ln f takes one logarithm, a product and an FMA per
-// population (a logarithm of f <= 0 gives the NaN by itself, and sum f = rho),
-// and the smallest g comes from the smallest h of each shell: 1.52 ms.
+// Every sum is kept in FP64 from the point's FP32 values on, in units of 2^896 so
+// that widening them takes integer operations only (values that are not finite are
+// converted), and the two points of a thread are added before they join it. sum
+// f ln f takes one logarithm, a product and an FMA per population (a logarithm of
+// f <= 0 gives the NaN by itself, and sum f = rho), and the smallest g comes from the
+// smallest h of each shell. 256^3: 2.96 ms with 12 FP64 additions, 9 conversions and six
+// operations around each of the 41 logarithms a point, 1.54 ms now (paper's solver 3.25
+// and 1.58); with conversions by branching integer code 1.61 and 1.68.
 template <typename Store, bool kPaper>
 __global__ void __launch_bounds__(kDiagThreads, 3)
     k_diag_pair(StepConst<float> K, const Store* __restrict__ pin, const float* __restrict__ e_in,
@@ -1029,7 +1022,8 @@ __global__ void __launch_bounds__(kDiagThreads, 3)
   const double t0 = (double)K.theta0;
   int64_t npts_here = 0;
   const float beta = K.beta, keep = 1.f - K.beta;
-  Sum2 sM, sX, sY, sZ, sE, sH;
+  // sums of drho, j (3), the trace of dP, the rotational energy and H1 / ln 2
+  double sum[7] = {0, 0, 0, 0, 0, 0, 0};
   float gmin = INFINITY;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < 2 * n3p;
        t += (int64_t)gridDim.x * blockDim.x) {
@@ -1042,7 +1036,7 @@ __global__ void __launch_bounds__(kDiagThreads, 3)
     Mom<F2> m;
     raw_moments_shells(h, m);
     const F2 e(reinterpret_cast<const float2*>(e_in)[t]);
-    recover<float, kPaper, true>(m, e, K);
+    recover<float, kPaper>(m, e, K);
     // smallest g = w (1 + h): w (1 + smallest h) shell by shell (rounding is monotone)
     auto small = [&](int q) { return fminf(h[q].v.x, h[q].v.y); };
     float gm = float(kWeightRest) * (1.f + small(0));
@@ -1055,14 +1049,6 @@ __global__ void __launch_bounds__(kDiagThreads, 3)
       gm = fminf(gm, float(pair_weight(k0)) * (1.f + hm));
     });
     gmin = fminf(gmin, gm);
-    sM.add(m.drho);
-    sX.add(m.j[0]);
-    sY.add(m.j[1]);
-    sZ.add(m.j[2]);
-    // paper mode holds theta_R: its energy density delta rho theta_R / 2 (deviation)
-    const F2 Ee = kPaper ? (0.5f * K.delta) * fmad(K.theta0, m.drho, m.rho * m.dR) : e;
-    sE.add(0.5f * (m.dP[0] + m.dP[1] + m.dP[2]));
-    sE.add(Ee);
     // H1: sum f ln f - sum f - (delta/2) rho ln theta_R, f = (1 - beta*) g + beta* f^mix
     Herm<F2> H;
     mix_coeffs(m, K, H);
@@ -1077,20 +1063,43 @@ __global__ void __launch_bounds__(kDiagThreads, 3)
       Hl = fmad(w * fm, lg2(fm), Hl);
     });
     Hl = fmad((-0.5f * K.delta) * m.rho, lg2(m.dR + K.theta0), Hl);
-    // in units of ln 2, and rho as 1 + drho: the sums of -drho and -1 follow below
-    sH.add(Hl);
+    // H1 in units of ln 2, and rho as 1 + drho: the sums of -drho and -1 follow below
+    auto join = [&](auto&& w) {
+      auto both = [&](F2 a) { return w(a.v.x) + w(a.v.y); };
+      sum[0] += both(m.drho);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) sum[1 + a] += both(m.j[a]);
+      sum[4] += both(m.dP[0]) + both(m.dP[1]) + both(m.dP[2]);
+      if constexpr (kPaper) {
+        // paper mode holds theta_R: rho theta_R - theta0 (times delta / 2 below)
+        auto er = [&](float rho, float dR) { return fma(w(rho), fma(w(dR), 0x1p896, t0), -t0 * 0x1p-896); };
+        sum[5] += er(m.rho.v.x, m.dR.v.x) + er(m.rho.v.y, m.dR.v.y);
+      } else {
+        sum[5] += both(e);
+      }
+      sum[6] += both(Hl);
+    };
+    F2 nil = fmad(0.f, Hl, 0.f * m.drho);  // 0, or NaN where a term is not finite
+#pragma unroll
+    for (int a = 0; a < 3; ++a) nil = fmad(0.f, m.dP[a], fmad(0.f, m.j[a], nil));
+    nil = fmad(0.f, kPaper ? m.dR : e, nil);
+    if (nil.v.x + nil.v.y == 0.f)
+      join([](float x) { return widen_scaled(x); });
+    else
+      join([](float x) { return (double)x * 0x1p-896; });
     npts_here += 2;
   }
-  const double ln2 = 0.6931471805599453094, M = sM.value();
-  const double n = (double)npts_here;
+  const double ln2 = 0.6931471805599453094, n = (double)npts_here;
   double acc[kDiagVals - 1];
+#pragma unroll
+  for (int k = 0; k < 7; ++k) sum[k] *= 0x1p896;
   // the per-point constants: 1 (mass) and 3 theta0/2 + delta theta0/2 (energy)
-  acc[0] = M + n;
-  acc[1] = sX.value();
-  acc[2] = sY.value();
-  acc[3] = sZ.value();
-  acc[4] = sE.value() + n * (1.5 * t0 + 0.5 * (double)K.delta * t0);
-  acc[5] = ln2 * sH.value() - M - n;
+  acc[0] = sum[0] + n;
+  acc[1] = sum[1];
+  acc[2] = sum[2];
+  acc[3] = sum[3];
+  acc[4] = 0.5 * sum[4] + (kPaper ? 0.5 * (double)K.delta * sum[5] : sum[5]) + n * (1.5 * t0 + 0.5 * (double)K.delta * t0);
+  acc[5] = ln2 * sum[6] - sum[0] - n;
   acc[6] = (double)gmin;
   diag_block_reduce(acc, partial);
 }

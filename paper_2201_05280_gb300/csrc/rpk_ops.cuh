@@ -41,7 +41,6 @@ static StepConst<Real> make_step_const(const rpk_relax& r, int nsub, int nx, int
   K.exc = Real(r.dt * r.delta / (2.0 * r.tau1));
   K.kapc = Real(r.k_r * 5.0 * r.tau / (2.0 * B));
   K.E0 = Real(0.5 * r.delta * kTheta0);
-  K.inv_delta = Real(1.0 / r.delta);
   const double i1 = 1.0 / kTheta0, cr = 2.0 * beta;
   K.two_id = Real(2.0 / r.delta);
   K.c_d = Real(r.delta / (3.0 + r.delta));
