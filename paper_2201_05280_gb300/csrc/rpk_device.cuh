@@ -623,10 +623,10 @@ __device__ __forceinline__ bool pair_from_block(const StepConst<float>& K, int& 
 // wall belongs to the y wall. Only the pairs kLo .. kHi - 1 (and the rest
 // population with pair 0) are gathered.
 template <typename Store, typename Real, bool kPull, int kBC, int kLo = 0, int kHi = kPairs>
-__device__ __forceinline__ void gather(const Store* __restrict__ pin,
+__device__ __forceinline__ void gather(const Store* pin,
                                        const Real* __restrict__ ghost, const StepConst<Real>& K,
                                        const PointIdx& P, Real (&h)[kQ],
-                                       const Real* __restrict__ wcol = nullptr) {
+                                       const Real* wcol = nullptr) {
   const int64_t n3 = K.n3;
   if constexpr (!kPull) {
     const unsigned cell = (unsigned)P.cell;
@@ -727,7 +727,7 @@ __device__ __forceinline__ void gather(const Store* __restrict__ pin,
 // at once (the axis is a template argument: every trip count is known). 128 x 64
 // x 8 between y walls: 12.6 us with one load after the other, now 4.6 us.
 template <typename Store, typename Real, int kBC, bool kX>
-__device__ __forceinline__ Real wall_column(const StepConst<Real>& K, const Store* __restrict__ pin,
+__device__ __forceinline__ Real wall_column(const StepConst<Real>& K, const Store* pin,
                                             const Real* __restrict__ hw, int w, int ca, int z) {
   const int nx = K.nx, ny = K.ny, nn = kX ? nx : ny;  // cells along the wall normal
   const int64_t n3 = K.n3;

@@ -118,8 +118,7 @@ __device__ __forceinline__ Real wall_theta(const StepConst<Real>& K, const Real*
 
 // advecting velocity: second-order extrapolation to t + dt/2
 template <typename Real>
-__device__ __forceinline__ Real vadv(const Real* __restrict__ ucur, const Real* __restrict__ uprev,
-                                     int64_t idx) {
+__device__ __forceinline__ Real vadv(const Real* ucur, const Real* uprev, int64_t idx) {
   return Real(1.5) * ucur[idx] - Real(0.5) * uprev[idx];
 }
 
@@ -148,11 +147,11 @@ __global__ void __launch_bounds__(kTBX * kTBY)
   const int64_t p = (int64_t)P.s * K.n3 + P.cell;
   const NbOff no = nb_offsets(K, P);
   const Real ep0 = e[p];
-  Real div = Real(0);
+  Real div = Real(0), vs[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const Real vp = vadv(ucur, uprev, a * npts + p);
-    v[a * npts + p] = vp;
+    vs[a] = vp;  // stored at the end: a store here would hold back the next axis's loads
     const int gc = ghost_code<kBC>(K, P, a, +1);
     const int64_t q = gc < 0 ? (int64_t)gc : p + no.o[a][1];
     Real eq, vq;
@@ -167,6 +166,8 @@ __global__ void __launch_bounds__(kTBX * kTBY)
     div += K.E0 * (vq - vp) + (eq * vq - ep0 * vp);
   }
   ep[p] = ep0 - K.dt * div;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) v[a * npts + p] = vs[a];
 }
 
 template <typename Real, int kBC>
@@ -357,7 +358,7 @@ inline __device__ bool quad_from_block(const StepConst<float>& K, Quad& Q) {
   return true;
 }
 
-__device__ __forceinline__ float4 ld4(const float* __restrict__ a, int64_t i) {
+__device__ __forceinline__ float4 ld4(const float* a, int64_t i) {
   return *reinterpret_cast<const float4*>(a + i);
 }
 __device__ __forceinline__ void st4(float* __restrict__ a, int64_t i, const float (&v)[4]) {
@@ -624,7 +625,7 @@ static __global__ void __launch_bounds__(kTBX * kTBY)
 // wall's theta_R (its table entry holds theta_R - theta0 in this mode) at the
 // wall's distance, extrapolated from r at the point itself.
 template <typename Real, int kBC>
-__device__ __forceinline__ Real pm_nb(const StepConst<Real>& K, const PointIdx& P, const Real* __restrict__ r,
+__device__ __forceinline__ Real pm_nb(const StepConst<Real>& K, const PointIdx& P, const Real* r,
                                       const Real* __restrict__ ghost, int a, int d) {
   const int64_t q = axis_nb<kBC>(K, P, a, d);
   if (kBC == 1 && q < 0) return ghost[(q == -1 ? 0 : kGhostStride) + kGhE];

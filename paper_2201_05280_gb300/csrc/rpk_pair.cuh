@@ -57,7 +57,7 @@ struct PairIO<__nv_bfloat16> {
 // pulled from x - c_q on a periodic grid (the layout of gather(); nx even).
 // w: the population array as pair words, (s*41 + q)*n3/2 + ((z*ny + y)*nx)/2 + i.
 template <typename Store>
-__device__ __forceinline__ void gather_pair(const typename PairIO<Store>::Word* __restrict__ w,
+__device__ __forceinline__ void gather_pair(const typename PairIO<Store>::Word* w,
                                             const StepConst<float>& K, int s, int i, int y, int z,
                                             F2 (&h)[kQ]) {
   using IO = PairIO<Store>;
@@ -128,7 +128,7 @@ namespace rpk {
 // the pair (a straddled word is assembled from its two source words); the
 // layout and sources of gather_pair. 16-bit storage only.
 template <typename Store>
-__device__ __forceinline__ void gather_pair_words(const unsigned* __restrict__ w, const StepConst<float>& K,
+__device__ __forceinline__ void gather_pair_words(const unsigned* w, const StepConst<float>& K,
                                                   int s, int i, int y, int z, unsigned (&hw)[kQ]) {
   static_assert(sizeof(Store) == 2, "pair words of 16-bit storage");
   const int ny = K.ny, nz = K.nz, nxp = K.nx >> 1;

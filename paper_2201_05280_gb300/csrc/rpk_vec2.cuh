@@ -51,7 +51,8 @@ __device__ __forceinline__ F2 fmad(F2 a, float b, F2 c) { return fmad(a, F2(b), 
 // blocks become resident while their own still run, and wait here until the
 // kernel before has completed (a no-op for ordinary launches). Nothing that an
 // earlier kernel writes or reads may be touched before it, and what an earlier
-// kernel writes is not read through const __restrict__ parameters: those become
+// kernel writes is not read through const __restrict__ parameters, neither the
+// kernel's own nor those of the device functions that load for it: those become
 // non-coherent loads, which may find lines that a kernel of two launches ago left in
 // L1 while this one's blocks were already resident. The next kernel is let in after
 // the wait, so that no more than two of a chain are resident.
