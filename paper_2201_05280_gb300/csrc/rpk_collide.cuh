@@ -11,31 +11,34 @@ namespace rpk {
 // the paper's explicit update (Sec. 5):
 //   g' = (1 - 2 beta*) g + 2 beta* f^mix,   in h form: h' = c_keep h + c_relax (f^mix/w - 1)
 //   Er' = Er + dt (delta rho/2)(theta - theta_R)/tau1   (rotational exchange)
-// hands the 41 relaxed populations to emit(q, value) in the order q = 0, 1, 2,
-// ..., returns the moments in m and the exchanged auxiliary rotational energy
-// (paper mode: theta_R after the first backward-Euler half step).
-// The part after the raw moments: hq(q) gives population q's h for the
-// relaxation (the array itself, or a conversion of its stored word).
-template <typename Real, bool kPaper = false, typename V, typename HQ, typename Emit>
-__device__ __forceinline__ V collide_relax(const StepConst<Real>& K, Mom<V>& m, V e, HQ&& hq, Emit&& emit) {
+// hands the 41 relaxed populations to emit(q, value) in the order q = 0, 1, 2, ...
+// and, with the moments in m complete, the exchanged auxiliary rotational energy
+// (paper mode: theta_R after the first backward-Euler half step with the time-t
+// theta_T) to fields(e): before the populations (kFieldsFirst) or after them.
+template <typename Real, bool kPaper, bool kFieldsFirst, typename V, typename Fields, typename Emit>
+__device__ __forceinline__ void collide_emit(const StepConst<Real>& K, const V (&h)[kQ], V e, Fields&& fields,
+                                             Emit&& emit, Mom<V>& m) {
+  raw_moments(h, m);
   recover<Real, kPaper>(m, e, K);
+  auto hand_over = [&] {
+    if constexpr (kPaper)
+      fields(fmad(K.ra_keep, m.dR, K.ra_t * m.dT));
+    else
+      fields(fmad(K.exc * m.rho, m.dth - m.dR, e));
+  };
+  if constexpr (kFieldsFirst) hand_over();
   Herm<V> H;
   mix_coeffs(m, K, H);
-  emit(0, fmad(K.c_keep, hq(0), K.c_relax * H.e0));
+  emit(0, fmad(K.c_keep, h[0], K.c_relax * H.e0));
   static_for<kPairs>([&](auto kc) {
     constexpr int k = decltype(kc)::value;
     constexpr Vel2 v = kPairVel2[k];
     const V ev = herm_even<v.x, v.y, v.z>(H);
     const V od = herm_odd<v.x, v.y, v.z>(H);
-    emit(2 * k + 1, fmad(K.c_keep, hq(2 * k + 1), K.c_relax * (ev + od)));
-    emit(2 * k + 2, fmad(K.c_keep, hq(2 * k + 2), K.c_relax * (ev - od)));
+    emit(2 * k + 1, fmad(K.c_keep, h[2 * k + 1], K.c_relax * (ev + od)));
+    emit(2 * k + 2, fmad(K.c_keep, h[2 * k + 2], K.c_relax * (ev - od)));
   });
-  // conservative form: the exchanged auxiliary energy; paper mode: theta_R after
-  // the first backward-Euler half step with the time-t theta_T (Sec. 5, step 1)
-  if constexpr (kPaper)
-    return fmad(K.ra_keep, m.dR, K.ra_t * m.dT);
-  else
-    return fmad(K.exc * m.rho, m.dth - m.dR, e);
+  if constexpr (!kFieldsFirst) hand_over();
 }
 
 // The same with the shell-wise sums and targets: about 430 operations a point
@@ -59,23 +62,19 @@ __device__ __forceinline__ V collide_shells(const StepConst<Real>& K, const V (&
     return fmad(K.exc * m.rho, m.dth - m.dR, e);
 }
 
-template <typename Real, bool kPaper = false, typename V, typename Emit>
-__device__ __forceinline__ V collide_emit(const StepConst<Real>& K, const V (&h)[kQ], V e, Emit&& emit,
-                                          Mom<V>& m) {
-  raw_moments(h, m);
-  return collide_relax<Real, kPaper>(K, m, e, [&](int q) { return h[q]; }, emit);
-}
-
 // One point: population q goes to cell of the plane out + q * n3.
 template <typename Store, typename Real, bool kPaper = false>
 __device__ __forceinline__ Real collide_point(const StepConst<Real>& K, const Real (&h)[kQ], Real e,
                                               Store* __restrict__ out, unsigned cell, Mom<Real>& m) {
   const int64_t n3 = K.n3;
   auto put = [&](int q, Real v) { (out + (int64_t)q * n3)[cell] = from_real<Store, Real>(v); };
-  if constexpr (kShells<Store>)
+  if constexpr (kShells<Store>) {
     return collide_shells<Real, kPaper>(K, h, e, put, m);
-  else
-    return collide_emit<Real, kPaper>(K, h, e, put, m);
+  } else {
+    Real es;
+    collide_emit<Real, kPaper, false>(K, h, e, [&](Real v) { es = v; }, put, m);
+    return es;
+  }
 }
 
 // Device status flags: 1 non-finite moment, 2 rho <= 0, 4 theta_T or theta_R <= 0.
@@ -339,6 +338,13 @@ __device__ __forceinline__ void flag_moments2(const Mom<F2>& m, float theta0, un
 // the arithmetic instructions; pair words halve the loads and stores).
 // kPaper: the paper's theta_R solver (the state holds theta_R - theta0; the
 // time-t theta_T(f) - theta0 goes to tt_out), as in k_collide.
+// Bound: the FMA pipes, and registers: four blocks per SM of 16-bit storage leave 128
+// for 82 values. The fields are stored before the populations are relaxed, so that
+// the moments they come from need not be held until then (spills 172 -> 68 bytes), and
+// the paper's solver loads e before the populations (144 -> 52). us at 256^3, FP16 /
+// FP16 paper / BF16 / BF16 paper: 1261 / 1261 / 1262 / 1292 with the fields last, now
+// 1176 / 1209 / 1245 / 1259. FP16 held as words and converted twice, at five blocks
+// per SM (four, paper): 1374 / 1318. FP32 keeps three blocks and does not spill (1703).
 template <typename Store, bool kPaper = false>
 __global__ void __launch_bounds__(128, sizeof(Store) == 4 ? 3 : 4)
     k_collide_pair(StepConst<float> K, const Store* pin, Store* __restrict__ pout,
@@ -353,71 +359,29 @@ __global__ void __launch_bounds__(128, sizeof(Store) == 4 ? 3 : 4)
   if (!pair_from_block(K, s, i, y, z, cellp)) return;
   const int64_t n3p = K.n3 >> 1;                // pairs per sublattice
   const int64_t pp = (int64_t)s * n3p + cellp;  // pair in a field plane
+  const float2* e2 = reinterpret_cast<const float2*>(e_in) + pp;
+  F2 e;
+  if constexpr (kPaper) e = F2(*e2);
   F2 h[kQ];
   gather_pair<Store>(reinterpret_cast<const Word*>(pin), K, s, i, y, z, h);
+  if constexpr (!kPaper) e = F2(*e2);
   Mom<F2> m;
   Word* out = reinterpret_cast<Word*>(pout) + (int64_t)(s * kQ) * n3p;
   const unsigned cell = (unsigned)cellp;
-  const F2 es = collide_emit<float, kPaper>(
-      K, h, F2(reinterpret_cast<const float2*>(e_in)[pp]),
+  collide_emit<float, kPaper, true>(
+      K, h, e,
+      [&](F2 es) {
+        reinterpret_cast<float2*>(e_out)[pp] = es.v;
+        reinterpret_cast<float2*>(drho_out)[pp] = m.drho.v;
+        float2* u2 = reinterpret_cast<float2*>(u_out);
+        u2[pp] = (m.j[0] * m.inv_rho).v;
+        u2[K.n3 + pp] = (m.j[1] * m.inv_rho).v;
+        u2[2 * K.n3 + pp] = (m.j[2] * m.inv_rho).v;
+        reinterpret_cast<float2*>(kap_out)[pp] = (K.kapc * m.rho * (K.theta0 + m.dth)).v;
+        if constexpr (kPaper) reinterpret_cast<float2*>(tt_out)[pp] = m.dT.v;
+        flag_moments2(m, K.theta0, status);
+      },
       [&](int q, F2 v) { (out + (int64_t)q * n3p)[cell] = IO::from_f2(v); }, m);
-  reinterpret_cast<float2*>(e_out)[pp] = es.v;
-  reinterpret_cast<float2*>(drho_out)[pp] = m.drho.v;
-  float2* u2 = reinterpret_cast<float2*>(u_out);
-  u2[pp] = (m.j[0] * m.inv_rho).v;
-  u2[K.n3 + pp] = (m.j[1] * m.inv_rho).v;
-  u2[2 * K.n3 + pp] = (m.j[2] * m.inv_rho).v;
-  reinterpret_cast<float2*>(kap_out)[pp] = (K.kapc * m.rho * (K.theta0 + m.dth)).v;
-  if constexpr (kPaper) reinterpret_cast<float2*>(tt_out)[pp] = m.dT.v;
-  flag_moments2(m, K.theta0, status);
-}
-
-// FP16 storage: k_collide_pair holding the 41 pair words (one register
-// each) instead of their 82 FP32 values between the moments and the
-// relaxation, which converts each word again where it is used (one cvt per
-// value). Fewer live registers fit more blocks per SM: per 512^3 launch 10.06
-// against 10.46 ms in the conservative form (5 blocks per SM), 10.24 against
-// 10.88 ms in the paper's solver (4 blocks; 11.53 ms with 5). BF16 storage
-// keeps k_collide_pair (11.18 against 10.13 ms: its conversion is two
-// integer operations).
-template <typename Store, bool kPaper = false>
-__global__ void __launch_bounds__(128, kPaper ? 4 : 5)
-    k_collide_pair_w(StepConst<float> K, const Store* pin, Store* __restrict__ pout,
-                     const float* e_in, float* __restrict__ e_out, float* __restrict__ drho_out,
-                     float* __restrict__ u_out, float* __restrict__ kap_out, unsigned* __restrict__ status,
-                     float* __restrict__ tt_out) {
-  pdl_wait();
-  static_assert(std::is_same<Store, __half>::value, "the word-holding collision serves FP16 storage");
-  using IO = PairIO<Store>;
-  int s, i, y, z;
-  int64_t cellp;
-  if (!pair_from_block(K, s, i, y, z, cellp)) return;
-  const int64_t n3p = K.n3 >> 1;
-  const int64_t pp = (int64_t)s * n3p + cellp;
-  unsigned hw[kQ];
-  gather_pair_words<Store>(reinterpret_cast<const unsigned*>(pin), K, s, i, y, z, hw);
-  Mom<F2> m;
-  {
-    F2 h[kQ];
-#pragma unroll
-    for (int q = 0; q < kQ; ++q) h[q] = IO::to_f2(hw[q]);
-    raw_moments(h, m);
-  }
-  unsigned* out = reinterpret_cast<unsigned*>(pout) + (int64_t)(s * kQ) * n3p;
-  const unsigned cell = (unsigned)cellp;
-  const F2 es = collide_relax<float, kPaper>(
-      K, m, F2(reinterpret_cast<const float2*>(e_in)[pp]),
-      [&](int q) { return word_to_f2_here<Store>(hw[q]); },
-      [&](int q, F2 v) { (out + (int64_t)q * n3p)[cell] = IO::from_f2(v); });
-  reinterpret_cast<float2*>(e_out)[pp] = es.v;
-  reinterpret_cast<float2*>(drho_out)[pp] = m.drho.v;
-  float2* u2 = reinterpret_cast<float2*>(u_out);
-  u2[pp] = (m.j[0] * m.inv_rho).v;
-  u2[K.n3 + pp] = (m.j[1] * m.inv_rho).v;
-  u2[2 * K.n3 + pp] = (m.j[2] * m.inv_rho).v;
-  reinterpret_cast<float2*>(kap_out)[pp] = (K.kapc * m.rho * (K.theta0 + m.dth)).v;
-  if constexpr (kPaper) reinterpret_cast<float2*>(tt_out)[pp] = m.dT.v;
-  flag_moments2(m, K.theta0, status);
 }
 
 }  // namespace rpk

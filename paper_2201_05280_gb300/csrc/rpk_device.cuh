@@ -131,6 +131,10 @@ struct StepConst {
   Real exc;       // dt delta / (2 tau1)
   Real kapc;      // k_r 5 tau / (2 B), kappa_R = kapc * rho * theta
   Real E0;        // delta theta0 / 2
+  // Not read: the kernels' pointers then begin 8 bytes past a 16-byte boundary of the
+  // arguments. Without it, us a launch: 256^3 BF16 pairs 1267 -> 1296, FP32 one point
+  // a thread 161 x 127 x 93 240 -> 248.
+  Real spare;
   // products of the above for the shell-wise collision (i = 1 / theta0)
   Real two_id;    // 2 / delta
   Real c_d, c_3;  // delta / (3 + delta), 3 / (3 + delta)

@@ -42,6 +42,7 @@ static StepConst<Real> make_step_const(const rpk_relax& r, int nsub, int nx, int
   K.kapc = Real(r.k_r * 5.0 * r.tau / (2.0 * B));
   K.E0 = Real(0.5 * r.delta * kTheta0);
   const double i1 = 1.0 / kTheta0, cr = 2.0 * beta;
+  K.spare = Real(0);
   K.two_id = Real(2.0 / r.delta);
   K.c_d = Real(r.delta / (3.0 + r.delta));
   K.c_3 = Real(3.0 / (3.0 + r.delta));
@@ -172,14 +173,9 @@ static rpk_status collide_launch(rpk_lattice* L, const StepConst<Real>& K) {
       if (L->grid.nx % 2 == 0) {
         // two x-adjacent points per thread, packed FP32x2 arithmetic
         const PointLaunch at(L, L->n3 / 2);
-        if constexpr (std::is_same<Store, __half>::value)
-          launch_step(L, k_collide_pair_w<Store, true>, at.grid, at.block, 0, K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
-              static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status,
-              static_cast<Real*>(L->thbuf));
-        else
-          launch_step(L, k_collide_pair<Store, true>, at.grid, at.block, 0, K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
-              static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status,
-              static_cast<Real*>(L->thbuf));
+        launch_step(L, k_collide_pair<Store, true>, at.grid, at.block, 0, K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
+            static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status,
+            static_cast<Real*>(L->thbuf));
         return check_launch("k_collide_pair");
       }
     }
@@ -192,13 +188,8 @@ static rpk_status collide_launch(rpk_lattice* L, const StepConst<Real>& K) {
     if (L->grid.nx % 2 == 0) {
       // two x-adjacent points per thread, packed FP32x2 arithmetic
       const PointLaunch at(L, L->n3 / 2);
-      // FP16 storage holds the pair words, not their FP32 values, across the collision
-      if constexpr (std::is_same<Store, __half>::value)
-        launch_step(L, k_collide_pair_w<Store, false>, at.grid, at.block, 0, K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
-            static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status, nullptr);
-      else
-        launch_step(L, k_collide_pair<Store, false>, at.grid, at.block, 0, K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
-            static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status, nullptr);
+      launch_step(L, k_collide_pair<Store, false>, at.grid, at.block, 0, K, pin, pout, static_cast<const Real*>(L->e), static_cast<Real*>(L->e_star),
+          static_cast<Real*>(L->drho), ucur, static_cast<Real*>(L->kap), L->status, nullptr);
       return check_launch("k_collide_pair");
     }
   }
