@@ -795,11 +795,12 @@ constexpr uint32_t DW_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | 
                               ((uint32_t)(DW_N >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
 
 struct DwTcArgs {
-  const float* dY;    // layer l's output gradient at dY + l * stride
-  const float* h;     // even layers' inputs: block b's at h + b * stride
-  const float* z;     // odd layers' inputs
+  const float* dy_even;  // output gradients of even layers: block b's at dy_even + b * dy_stride
+  const float* dy_odd;   // and of odd layers
+  const float* h;        // even layers' inputs: block b's at h + b * stride
+  const float* z;        // odd layers' inputs
   float* g;           // layer l's weight gradient at g + l * gstride, then its bias gradient
-  int64_t stride, gstride;
+  int64_t stride, dy_stride, gstride;
   int ntiles, tiles_per_seq, seq_len, splits;
   unsigned* error;
 };
@@ -826,7 +827,7 @@ __global__ void __launch_bounds__(DW_THREADS, 1) k_dw_tc(DwTcArgs P) {
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot, bar0 = smem_u32(bars), base = smem_u32(tc_smem);
-  const float* dY = P.dY + layer * P.stride;
+  const float* dY = ((layer & 1) ? P.dy_odd : P.dy_even) + (layer >> 1) * P.dy_stride;
   const float* X = ((layer & 1) ? P.z : P.h) + (layer >> 1) * P.stride + half * DW_N;
   constexpr int kA = TC_N * (TC_M / 8) / DW_THREADS;                              // 4 dY elements per thread
   constexpr int kB = (TC_ROWS * (DW_N / 8) + DW_THREADS - 1) / DW_THREADS;        // 3 X elements
@@ -1145,7 +1146,8 @@ struct rpk_net {
   float* act = nullptr;   // h_0..h_B (B+1), z0 per block (B): (2B+1) x cap_q x width
   // training workspace for up to cap_t coarse positions
   int64_t cap_t = 0;
-  float* work = nullptr;  // (2B+1) x cap_t x width: slot 0 the lift's, slot l + 1 block layer l's output gradient
+  float* work = nullptr;  // output gradients, slots of nq x width (layout: backward)
+  int64_t work_floats = 0;
   float* headout = nullptr;
   float* dybuf = nullptr;
   double* loss = nullptr;
@@ -1186,6 +1188,16 @@ rpk_status ensure_workspace(rpk_net* N, int64_t nq) {
   return RPK_OK;
 }
 
+// Output gradients: one slot per layer (2 B + 1) lets one launch take every block's weight
+// gradients at the end; where they would take more than this, or do not fit the device,
+// two slots serve and each block's weight gradients follow its input gradient, so that
+// a batch is never refused for the sake of the slots. Batches that large fill the chip
+// with one block's layers: six blocks, a step of 204,800 coarse positions 3.31 ms with
+// all slots (1.4 GB) and 3.36 with two, of 768,000 11.37 (5.1 GB) and 11.32.
+constexpr int64_t kAllSlotsBytes = 4ll << 30;
+
+int64_t all_slots(const rpk_net* N, int64_t nq) { return (2 * (int64_t)N->nblocks + 1) * nq * N->width; }
+
 rpk_status ensure_training(rpk_net* N, int64_t nq) {
   rpk_status st = ensure_workspace(N, nq);
   if (st != RPK_OK || nq <= N->cap_t) return st;
@@ -1194,9 +1206,16 @@ rpk_status ensure_training(rpk_net* N, int64_t nq) {
   cudaFree(N->dybuf);
   N->work = N->headout = N->dybuf = nullptr;
   N->cap_t = 0;
-  st = net_alloc((void**)&N->work, sizeof(float) * (2 * N->nblocks + 1) * nq * N->width);
-  if (st == RPK_OK) st = net_alloc((void**)&N->headout, sizeof(float) * nq * R * N->cout);
+  st = net_alloc((void**)&N->headout, sizeof(float) * nq * R * N->cout);
   if (st == RPK_OK) st = net_alloc((void**)&N->dybuf, sizeof(float) * nq * R * N->cout);
+  if (st != RPK_OK) return st;
+  const int64_t two = std::min<int64_t>(2 * nq * N->width, all_slots(N, nq));
+  N->work_floats = std::max(two, std::min(all_slots(N, nq), kAllSlotsBytes / (int64_t)sizeof(float)));
+  st = net_alloc((void**)&N->work, sizeof(float) * N->work_floats);
+  if (st != RPK_OK && N->work_floats > two) {
+    N->work_floats = two;
+    st = net_alloc((void**)&N->work, sizeof(float) * two);
+  }
   if (st != RPK_OK) return st;
   N->cap_t = nq;
   return RPK_OK;
@@ -1339,15 +1358,18 @@ __global__ void k_fill_sequences(const int2* __restrict__ starts, int2* __restri
   }
 }
 
-// Gradients of every block convolution's weights and biases from the output
-// gradients in N->work (slot l + 1: block layer l).
-rpk_status block_grads(rpk_net* N, int64_t nq, int Lq) {
+// Gradients of the weights and biases of blocks b0 .. b0 + nb - 1 from the output
+// gradients of their even and odd layers (block b0's first, then dy_stride apart).
+rpk_status block_grads(rpk_net* N, int64_t nq, int Lq, int b0, int nb, const float* dy_even, const float* dy_odd,
+                       int64_t dy_stride) {
   const int64_t stride = nq * N->width;
-  const int nl = 2 * N->nblocks, W = N->width;
+  const int nl = 2 * nb, W = N->width;
   if (nl == 0) return RPK_OK;
-  const auto& first = N->layers[1];
+  const float* h = N->act + b0 * stride;
+  const float* z = N->act + (N->nblocks + 1 + b0) * stride;
+  const auto& first = N->layers[1 + 2 * b0];
   if (N->tc && (((uintptr_t)(N->g + first.w_off)) & 15) == 0) {
-    DwTcArgs P{N->work + stride, N->act, N->act + (N->nblocks + 1) * stride, N->g + first.w_off, stride,
+    DwTcArgs P{dy_even, dy_odd, h, z, N->g + first.w_off, stride, dy_stride,
                (int64_t)W * TC_K + W, 0, (Lq + TC_N - 1) / TC_N, Lq, 1, N->tc_error};
     P.ntiles = (int)(nq / Lq) * P.tiles_per_seq;
     // one CTA per SM: as many shares of the tiles as the SMs hold (layer, half) pairs
@@ -1357,9 +1379,9 @@ rpk_status block_grads(rpk_net* N, int64_t nq, int Lq) {
     return RPK_OK;
   }
   for (int l = 0; l < nl; ++l) {
-    const float* X = N->act + ((l & 1) ? N->nblocks + 1 + l / 2 : l / 2) * stride;
-    const float* dY = N->work + (l + 1) * stride;
-    const auto& L = N->layers[1 + l];
+    const float* X = ((l & 1) ? z : h) + (l >> 1) * stride;
+    const float* dY = ((l & 1) ? dy_odd : dy_even) + (l >> 1) * dy_stride;
+    const auto& L = N->layers[1 + 2 * b0 + l];
     rpk_status st = conv_dw(N, dY, W, X, W, K5, 1, N->g + L.w_off, nq, Lq);
     if (st != RPK_OK) return st;
     bias_grad(N, dY, nq, W, N->g + L.b_off);
@@ -1368,46 +1390,56 @@ rpk_status block_grads(rpk_net* N, int64_t nq, int Lq) {
   return RPK_OK;
 }
 
-// Backward pass from dy (fine layout == coarse layout), gradients into N->g:
-// the chain of input gradients first (each layer's output gradient kept in its
-// own slot of N->work), then the block layers' weight gradients together.
+// Backward pass from dy (fine layout == coarse layout), gradients into N->g. With
+// a slot of N->work per layer the chain of input gradients comes first (slot 0 the
+// lift's, slot l + 1 block layer l's output gradient) and the blocks' weight gradients
+// together after it. With two slots a block's weight gradients follow its input
+// gradient, whose output goes where an output gradient is no longer needed: slot 0
+// and the last block's output h_B in turn (h_B serves only the head).
 rpk_status backward(rpk_net* N, const float* x, const float* dy, int nseq, int L) {
   const int64_t nq = (int64_t)nseq * (L / R);
   const int Lq = L / R;
   const int64_t stride = nq * N->width;
   RPK_CUDA(cudaMemsetAsync(N->g, 0, sizeof(float) * N->nparams, N->stream));
+  const bool all = all_slots(N, nq) <= N->work_floats;
   auto slot = [&](int k) { return N->work + k * stride; };
   const int W = N->width;
   const auto& head = N->layers.back();
-  const float* hB = N->act + N->nblocks * stride;
+  float* hB = N->act + N->nblocks * stride;
   rpk_status st = conv_dw(N, dy, R * N->cout, hB, W, 1, 1, N->g + head.w_off, nq, Lq);
   bias_grad(N, dy, nq, R * N->cout, N->g + head.b_off);
   // d relu(h_B) = W_head^T dy, then mask by h_B > 0
+  float* dh = all ? slot(2 * N->nblocks) : slot(0);
+  float* spare = hB;
   if (st == RPK_OK)
-    st = conv(N, N->wtb + head.wb_off, W, 1, R * N->cout, -1, dy, 0, slot(2 * N->nblocks), nullptr, nullptr, hB, nq, Lq);
+    st = conv(N, N->wtb + head.wb_off, W, 1, R * N->cout, -1, dy, 0, dh, nullptr, nullptr, hB, nq, Lq);
   for (int b = N->nblocks - 1; b >= 0 && st == RPK_OK; --b) {
     const auto& c0 = N->layers[1 + 2 * b];
     const auto& c1 = N->layers[2 + 2 * b];
     const float* hb = N->act + b * stride;
     const float* z0 = N->act + (N->nblocks + 1 + b) * stride;
-    const float* dh = slot(2 * b + 2);  // z1 = conv(relu(z0)); d z1 = dh
-    float* dz = slot(2 * b + 1);        // z0 = conv(relu(h_b)); d z0
+    // z1 = conv(relu(z0)): d z1 = dh; z0 = conv(relu(h_b)): d z0 = dz; d h_b = dp
+    float* dz = all ? slot(2 * b + 1) : slot(1);
+    float* dp = all ? slot(2 * b) : spare;
     if (N->tc) {
-      st = block_tc(N, BlockArgs{N->wtb + c1.wb_off, N->wtb + c0.wb_off, dh, dz, slot(2 * b), nullptr, nullptr, z0, hb,
+      st = block_tc(N, BlockArgs{N->wtb + c1.wb_off, N->wtb + c0.wb_off, dh, dz, dp, nullptr, nullptr, z0, hb,
                                  nullptr, 0, 0, 0, -1, 0, nullptr},
                     nq, Lq, nullptr);
-      continue;
+    } else {
+      st = conv(N, N->wtb + c1.wb_off, W, K5, W, -1, dh, 0, dz, nullptr, nullptr, z0, nq, Lq);
+      // d h_b = dh + (W0^T dz) masked by h_b > 0
+      if (st == RPK_OK)
+        st = conv(N, N->wtb + c0.wb_off, W, K5, W, -1, dz, 0, dp, nullptr, dh, hb, nq, Lq);
     }
-    st = conv(N, N->wtb + c1.wb_off, W, K5, W, -1, dh, 0, dz, nullptr, nullptr, z0, nq, Lq);
-    // d h_b = dh + (W0^T dz) masked by h_b > 0
-    if (st == RPK_OK)
-      st = conv(N, N->wtb + c0.wb_off, W, K5, W, -1, dz, 0, slot(2 * b), nullptr, dh, hb, nq, Lq);
+    if (!all && st == RPK_OK) st = block_grads(N, nq, Lq, b, 1, dz, dh, 0);
+    spare = dh;
+    dh = dp;
   }
-  if (st == RPK_OK) st = block_grads(N, nq, Lq);
+  if (all && st == RPK_OK) st = block_grads(N, nq, Lq, 0, N->nblocks, slot(1), slot(2), 2 * stride);
   if (st != RPK_OK) return st;
   const auto& lift = N->layers[0];
-  st = conv_dw(N, slot(0), W, x, R * N->cin, 1, 0, N->g + lift.w_off, nq, Lq);
-  bias_grad(N, slot(0), nq, W, N->g + lift.b_off);
+  st = conv_dw(N, dh, W, x, R * N->cin, 1, 0, N->g + lift.w_off, nq, Lq);
+  bias_grad(N, dh, nq, W, N->g + lift.b_off);
   RPK_CUDA(cudaGetLastError());
   return st;
 }
