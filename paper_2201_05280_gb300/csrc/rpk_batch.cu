@@ -665,7 +665,7 @@ __global__ void k_batch_init(TubeDev<Real>* __restrict__ tubes, const double* __
     const int side = threadIdx.x;
     const double* st = res + 12 * (int64_t)blockIdx.x + 6 * side;
     Real h[kQ], e;
-    init_point(K, hdt, st[0], st[1], st[2], st[3], st[4], st[5], h, e);
+    init_point<Real, true>(K, hdt, st[0], st[1], st[2], st[3], st[4], st[5], h, e);
     Real* gg = tb->ghost + side * kGhostStride;
     for (int q = 0; q < kQ; ++q) gg[q] = h[q];
     gg[kGhE] = e;

@@ -794,7 +794,8 @@ __global__ void __launch_bounds__(128)
 
 // Reservoir table: for the low (side 0) and high (side 1) x end, the h of the
 // equilibrium state (post-collision equals pre-collision there), its e, rho - 1,
-// u and kappa_R. states: rho, ux, uy, uz, theta_T, theta_R per side.
+// u and kappa_R, in the expansion of the points (k_init), so that the same state has
+// the same bits on both sides of an end. states: rho, ux, uy, uz, theta_T, theta_R per side.
 template <typename Real>
 __global__ void k_ghost(StepConst<Real> K, Real half_dt_over_tau1, const double* __restrict__ st,
                         Real* __restrict__ ghost) {
@@ -802,7 +803,7 @@ __global__ void k_ghost(StepConst<Real> K, Real half_dt_over_tau1, const double*
   if (side >= 2) return;
   const double* s = st + 6 * side;
   Real h[kQ], e;
-  init_point(K, half_dt_over_tau1, s[0], s[1], s[2], s[3], s[4], s[5], h, e);
+  init_point<Real, kShells<Real>>(K, half_dt_over_tau1, s[0], s[1], s[2], s[3], s[4], s[5], h, e);
   Real* g = ghost + side * kGhostStride;
 #pragma unroll
   for (int q = 0; q < kQ; ++q) g[q] = h[q];
