@@ -433,8 +433,9 @@ __device__ __forceinline__ int ftcs_width(int nx, int nwarps) {
   return -best;
 }
 
-template <typename Store, typename Real, int kThreads, bool kImplicit>
-__global__ void __launch_bounds__(kThreads)
+// kCtas: CTAs per SM that must fit its registers (see BatchOps); 0 leaves it open.
+template <typename Store, typename Real, int kThreads, bool kImplicit, int kCtas>
+__global__ void __launch_bounds__(kThreads, kCtas)
     k_batch(TubeDev<Real>* __restrict__ tubes, const int* __restrict__ order, int ntubes,
             int* __restrict__ counter, Store* __restrict__ pop0, Store* __restrict__ pop1,
             Real* __restrict__ e_state, Real* __restrict__ ux_state, float* __restrict__ snaps,
@@ -802,19 +803,27 @@ namespace {
 template <typename Store, typename Real>
 struct BatchOps {
   // one kernel per thread count and diffusion, so that neither form's registers
-  // bind the other
+  // bind the other. 256 threads in FP32 take 254 registers; several CTAs per SM of
+  // tubes up to kTwoCtaCells take a kernel held to the 128 that two leave. Two CTAs
+  // of 256 per SM, ms, backward Euler / FTCS: 1216 tubes of 60 to 150 cells 2.16 / 1.43
+  // -> 1.56 / 1.02, of 500 to 700 6.30 / 6.49 -> 5.74 / 5.44; 456 of 1000 to 1500 5.04 /
+  // 5.49 -> 5.17 / 5.55, so longer tubes keep the kernel with all registers.
+  static constexpr int kTwoCtaCells = 1000;
   template <bool kImplicit>
-  static void* kernel_of(int threads) {
+  static void* kernel_of(int threads, bool two) {
+    constexpr int kTwo = sizeof(Real) == 4 ? 2 : 0;
     switch (threads) {
-      case 128: return (void*)k_batch<Store, Real, 128, kImplicit>;
-      case 256: return (void*)k_batch<Store, Real, 256, kImplicit>;
-      case 384: return (void*)k_batch<Store, Real, 384, kImplicit>;
-      case 512: return (void*)k_batch<Store, Real, 512, kImplicit>;
+      case 128: return (void*)k_batch<Store, Real, 128, kImplicit, 0>;
+      case 256:
+        return two ? (void*)k_batch<Store, Real, 256, kImplicit, kTwo> : (void*)k_batch<Store, Real, 256, kImplicit, 0>;
+      case 384: return (void*)k_batch<Store, Real, 384, kImplicit, 0>;
+      case 512: return (void*)k_batch<Store, Real, 512, kImplicit, 0>;
       default: return nullptr;
     }
   }
-  static void* kernel(int threads, int implicit) {
-    return implicit ? kernel_of<true>(threads) : kernel_of<false>(threads);
+  static void* kernel(const rpk_batch* B, int threads, int ctas) {
+    const bool two = ctas >= 2 && B->max_nx <= kTwoCtaCells;
+    return B->implicit ? kernel_of<true>(threads, two) : kernel_of<false>(threads, two);
   }
 };
 
@@ -896,8 +905,8 @@ rpk_status upload_tubes(rpk_batch* B) {
 
 // Shared-memory limit of the kernel variant (outside any stream capture).
 template <typename Store, typename Real>
-rpk_status prepare_batch(rpk_batch* B, int threads) {
-  void* kfn = BatchOps<Store, Real>::kernel(threads, B->implicit);
+rpk_status prepare_batch(rpk_batch* B, int threads, int ctas_per_sm) {
+  void* kfn = BatchOps<Store, Real>::kernel(B, threads, ctas_per_sm);
   if (!kfn) return fail(RPK_ERR_ARG, "unsupported thread count");
   RPK_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)batch_smem(B)));
@@ -917,7 +926,7 @@ rpk_status launch_batch(rpk_batch* B, cudaStream_t stream, int threads, int ctas
   Real* es = static_cast<Real*>(B->e_state);
   Real* us = static_cast<Real*>(B->ux_state);
   const int max_np = 2 * B->max_nx;
-  void* kfn = BatchOps<Store, Real>::kernel(threads, B->implicit);
+  void* kfn = BatchOps<Store, Real>::kernel(B, threads, ctas_per_sm);
   int ntubes = B->ntubes, save_every = B->save_every;
   // both population buffers of the tubes that run at a time, against L2
   int l2 = 0;
@@ -1187,7 +1196,7 @@ rpk_status rpk_batch_run(rpk_batch* B) {
     }
     rpk_status pst = with_batch_types(B->precision, [&](auto ops, auto* real_tag) {
       using Real = std::remove_pointer_t<decltype(real_tag)>;
-      return prepare_batch<Real, Real>(B, B->threads);
+      return prepare_batch<Real, Real>(B, B->threads, B->ctas_per_sm);
     });
     if (pst != RPK_OK) return pst;
     cudaStream_t cap = nullptr;
@@ -1291,7 +1300,7 @@ rpk_status rpk_batch_autotune(rpk_batch* B, int64_t out[3]) {
         float ms = 0.f;
         st = with_batch_types(B->precision, [&](auto ops, auto* real_tag) {
           using Real = std::remove_pointer_t<decltype(real_tag)>;
-          return prepare_batch<Real, Real>(S, t);
+          return prepare_batch<Real, Real>(S, t, c);
         });
         for (int rep = 0; rep < 2 && st == RPK_OK; ++rep) {
           cudaEventRecord(e0, B->stream);
