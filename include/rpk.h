@@ -259,8 +259,10 @@ rpk_status rpk_get_info(rpk_lattice* lat, int64_t out[4]);
 /* Kernel timing (a tracing aid; the paper has no counterpart). While enabled,
  * rpk_step brackets each kernel class with CUDA events recorded on the
  * lattice's stream: RPK_KC_COLLIDE (pull-stream + collide + exchange) and
- * RPK_KC_TRANSPORT (MacCormack advection and all FTCS sub-steps of E_R). rpk_timing(lat, 1) clears the counters and starts;
- * rpk_timing(lat, 0) stops. rpk_timing_read synchronises the stream and
+ * RPK_KC_TRANSPORT (MacCormack advection and all FTCS sub-steps of E_R).
+ * rpk_timing(lat, 1) clears the counters and starts; rpk_timing(lat, 2) does too and
+ * keeps the kernels of a step from overlapping (each starts when the one before has
+ * ended); rpk_timing(lat, 0) stops. rpk_timing_read synchronises the stream and
  * returns the summed milliseconds and the number of kernel launches per class
  * since the last start (arrays of RPK_KC_COUNT entries). */
 enum { RPK_KC_COLLIDE = 0, RPK_KC_TRANSPORT = 1, RPK_KC_COUNT = 2 };

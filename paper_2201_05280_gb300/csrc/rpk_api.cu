@@ -680,6 +680,7 @@ rpk_status rpk_load(rpk_lattice* L, const char* path) {
 rpk_status rpk_timing(rpk_lattice* L, int enable) {
   if (!L) return fail(RPK_ERR_ARG, "lattice is NULL");
   L->timing = enable != 0;
+  L->apart = enable == 2;
   L->ev_used = 0;
   return RPK_OK;
 }

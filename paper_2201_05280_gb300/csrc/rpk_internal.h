@@ -64,6 +64,7 @@ struct rpk_lattice {
   BrickPlan brick;
   // kernel timing: event pairs recorded around each kernel class
   bool timing = false;
+  bool apart = false;  // launches of a step one after the other
   std::vector<cudaEvent_t> events;
   std::vector<int> ev_class;   // class of each recorded pair
   std::vector<int> ev_kernels; // kernel launches inside each pair

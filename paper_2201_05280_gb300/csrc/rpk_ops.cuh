@@ -122,7 +122,7 @@ static void launch_step(rpk_lattice* L, void (*kernel)(KArgs...), dim3 grid, dim
   a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   a.val.programmaticStreamSerializationAllowed = 1;
   c.attrs = &a;
-  c.numAttrs = overlap_launches(L) ? 1 : 0;
+  c.numAttrs = overlap_launches(L) && !L->apart ? 1 : 0;
   cudaLaunchKernelEx(&c, kernel, static_cast<KArgs>(args)...);
 }
 
