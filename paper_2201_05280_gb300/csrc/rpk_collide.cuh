@@ -14,7 +14,7 @@ namespace rpk {
 // hands the 41 relaxed populations to emit(q, value) in the order q = 0, 1, 2, ...
 // and, with the moments in m complete, the exchanged auxiliary rotational energy
 // (paper mode: theta_R after the first backward-Euler half step with the time-t
-// theta_T) to fields(e): before the populations (kFieldsFirst) or after them.
+// theta_T) to fields(e, m): before the populations (kFieldsFirst) or after them.
 template <typename Real, bool kPaper, bool kFieldsFirst, typename V, typename Fields, typename Emit>
 __device__ __forceinline__ void collide_emit(const StepConst<Real>& K, const V (&h)[kQ], V e, Fields&& fields,
                                              Emit&& emit, Mom<V>& m) {
@@ -22,9 +22,9 @@ __device__ __forceinline__ void collide_emit(const StepConst<Real>& K, const V (
   recover<Real, kPaper>(m, e, K);
   auto hand_over = [&] {
     if constexpr (kPaper)
-      fields(fmad(K.ra_keep, m.dR, K.ra_t * m.dT));
+      fields(fmad(K.ra_keep, m.dR, K.ra_t * m.dT), m);
     else
-      fields(fmad(K.exc * m.rho, m.dth - m.dR, e));
+      fields(fmad(K.exc * m.rho, m.dth - m.dR, e), m);
   };
   if constexpr (kFieldsFirst) hand_over();
   Herm<V> H;
@@ -72,7 +72,7 @@ __device__ __forceinline__ Real collide_point(const StepConst<Real>& K, const Re
     return collide_shells<Real, kPaper>(K, h, e, put, m);
   } else {
     Real es;
-    collide_emit<Real, kPaper, false>(K, h, e, [&](Real v) { es = v; }, put, m);
+    collide_emit<Real, kPaper, false>(K, h, e, [&](Real v, const Mom<Real>&) { es = v; }, put, m);
     return es;
   }
 }
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(128, sizeof(Store) == 4 ? 3 : 4)
   const unsigned cell = (unsigned)cellp;
   collide_emit<float, kPaper, true>(
       K, h, e,
-      [&](F2 es) {
+      [&](F2 es, const Mom<F2>& m) {
         reinterpret_cast<float2*>(e_out)[pp] = es.v;
         reinterpret_cast<float2*>(drho_out)[pp] = m.drho.v;
         float2* u2 = reinterpret_cast<float2*>(u_out);
