@@ -243,11 +243,12 @@ static inline bool brick_block(const rpk_lattice* L, int open, const int (&own)[
     b.halo[a] = !op && (int64_t)own[a] + 2 * h > n[a] ? 0 : h;
     b.ext[a] = op ? std::min(own[a] + 2 * h, n[a] + 2) : b.halo[a] ? own[a] + 2 * h : n[a];
   }
-  const int64_t area = (int64_t)b.ext[0] * b.ext[1], Z = b.ext[2];
-  if (area > kBrickThreads || Z > kBrickMaxP * (kBrickThreads / area)) return false;
-  b.planes = (int)((Z + kBrickThreads / area - 1) / (kBrickThreads / area));
-  b.groups = (int)((Z + b.planes - 1) / b.planes);
-  b.threads = (int)((area * b.groups + 31) / 32 * 32);
+  if ((int64_t)b.ext[0] * b.ext[1] > kBrickThreads) return false;
+  const int area = b.ext[0] * b.ext[1], Z = b.ext[2], columns = kBrickThreads / area;
+  if (Z > kBrickMaxP * columns) return false;
+  b.planes = (Z + columns - 1) / columns;
+  b.groups = (Z + b.planes - 1) / b.planes;
+  b.threads = (area * b.groups + 31) / 32 * 32;
   b.smem = sizeof(float) * kBrickArrays * kBrickThreads * b.planes;
   return true;
 }
@@ -279,15 +280,27 @@ static inline rpk_status make_brick_plan(rpk_lattice* L, int open) {
   if (L->n3 > (int64_t)kBrickMaxP * kBrickThreads * L->sms) return RPK_OK;
   const int n[3] = {L->grid.nx, L->grid.ny, L->grid.nz};
   static constexpr int kCuts[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32, 48, 64, 96, 128};
+  // the cuts of an axis that give tiles of different length, fewest first
+  struct Cut {
+    int count, own;
+  } cuts[3][sizeof(kCuts) / sizeof(int)];
+  int ncuts[3] = {0, 0, 0};
+  for (int a = 0; a < 3; ++a)
+    for (int c : kCuts) {
+      const int own = (n[a] + c - 1) / c;
+      if (c <= n[a] && (ncuts[a] == 0 || cuts[a][ncuts[a] - 1].own != own)) cuts[a][ncuts[a]++] = {c, own};
+    }
   // best tile of a launch of m sub-steps
   auto best = [&](int m, bool first, BrickPlan::Part& part) {
     double cost = 1e30;
-    for (int cz : kCuts)
-      for (int cy : kCuts)
-        for (int cx : kCuts) {
-          if (cx > n[0] || cy > n[1] || cz > n[2] || cx * cy * cz > 2 * L->sms) break;
-          const int own[3] = {(n[0] + cx - 1) / cx, (n[1] + cy - 1) / cy, (n[2] + cz - 1) / cz};
+    for (int kz = 0; kz < ncuts[2]; ++kz)
+      for (int ky = 0; ky < ncuts[1]; ++ky)
+        for (int kx = 0; kx < ncuts[0]; ++kx) {
+          const int cx = cuts[0][kx].count, cy = cuts[1][ky].count, cz = cuts[2][kz].count;
+          if (cx * cy * cz > 2 * L->sms) break;
+          const int own[3] = {cuts[0][kx].own, cuts[1][ky].own, cuts[2][kz].own};
           BrickBlock b;
+          if (cost <= 7000.0 + 600.0 * m) return cost;  // the least of any tile
           if (!brick_block(L, open, own, m + (first ? 1 : 0), b)) continue;
           const int blocks = (2 * cx * cy * cz + L->sms - 1) / L->sms;  // of the busiest SM
           const int rounds = (blocks * b.threads + kBrickThreads - 1) / kBrickThreads;
@@ -305,6 +318,7 @@ static inline rpk_status make_brick_plan(rpk_lattice* L, int open) {
   for (int m = std::min(L->nsub, kBrickSub); m >= 1; --m) {
     const int parts = (L->nsub + m - 1) / m;
     if (m > 1 && (L->nsub + m - 2) / (m - 1) == parts) continue;  // as many launches of fewer sub-steps
+    if (7000.0 * parts + 600.0 * L->nsub >= cost) continue;        // their least cost
     BrickPlan::Part first, full, rest;
     // parts of m or m - 1 sub-steps, the first with the deeper halo a short one
     const int shorter = parts * m - L->nsub, m0 = m - (shorter ? 1 : 0);
