@@ -306,15 +306,15 @@ void rpk_batch_destroy(rpk_batch* b);
 rpk_status rpk_batch_init(rpk_batch* b, const double* rho, const double* u, const double* theta_T,
                           const double* theta_R);
 
-/* Launch configuration of the persistent kernel: threads per CTA (a multiple
- * of 32 in [64, 512]) and CTAs per SM (>= 1, limited by shared memory). */
+/* Launch configuration of the persistent kernel: threads per CTA (128,
+ * 256, 384 or 512) and CTAs per SM (>= 1, limited by shared memory). */
 rpk_status rpk_batch_set_config(rpk_batch* b, int threads, int ctas_per_sm);
 /* Rotational diffusion of the batch: mode 0 (default) the nsub FTCS sub-steps
  * of the paper's scheme (Sec. 5, rotational step 3); mode 1 a variant that
  * takes the same flux-form equation in one backward-Euler step per time step,
  * (delta rho / 2) theta' - dt [K+ (theta'_+ - theta') - K- (theta' - theta'_-)]
- * = E_R, solved per sublattice line by cyclic reduction (unconditionally
- * stable: nsub is ignored). Takes effect at the next rpk_batch_run. */
+ * = E_R, solved per sublattice line by substructuring: blocks of points, their
+ * end points, then all points (unconditionally stable: nsub is ignored). Takes effect at the next rpk_batch_run. */
 rpk_status rpk_batch_set_diffusion(rpk_batch* b, int mode);
 
 /* Time every supported launch configuration on a sample of the batch's own

@@ -9,9 +9,10 @@
 // live in shared memory for the whole time loop, so the transport (MacCormack
 // and the FTCS sub-steps) costs no device-memory traffic. Tubes need no
 // synchronisation with each other, so the launch has no grid-wide barrier. The
-// arithmetic is that of the lattice kernels (k_collide, k_mac_pred,
-// k_mac_corr, k_ftcs) on an nx x 1 x 1 grid, where every y and z
-// neighbour is the point itself and contributes exact zeros.
+// method is that of the lattice kernels on an nx x 1 x 1 grid, where every y and z
+// neighbour is the point itself and contributes exact zeros; the collision is the
+// factored form of FP64 lattices in FP32 too, so FP32 tubes and FP32 lattices agree to
+// rounding, not bit for bit.
 #include <algorithm>
 #include <cmath>
 #include <cstring>

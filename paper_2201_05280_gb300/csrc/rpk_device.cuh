@@ -99,8 +99,10 @@ __device__ __forceinline__ void static_for(F&& f) {
 // ---------------------------------------------------------------------------
 // per-launch constants (host fills them in double, then casts)
 
-// Division of a 32-bit index by a launch constant: n / d = (umulhi(m, n) + n) >> l
-// for n < 2^31 (m = floor(2^32 (2^l - d) / d) + 1, l = ceil(log2 d)).
+// Division of a 32-bit index by a launch constant, after Granlund and Montgomery
+// (Division by invariant integers using multiplication, PLDI 1994): n / d =
+// (umulhi(m, n) + n) >> l for n < 2^31, m = floor(2^32 (2^l - d) / d) + 1, l =
+// ceil(log2 d).
 struct FastDiv {
   unsigned m, l;
   FastDiv() = default;
@@ -213,8 +215,8 @@ __device__ __forceinline__ void raw_moments(const V (&h)[kQ], Mom<V>& m) {
 // sums once instead of every pair, and the sign patterns of the (1, 1, 1) and
 // (1/2, 1/2, 1/2) pairs, (+++), (++-), (+-+), (+--), are one 4-point butterfly for
 // the even and one for the odd parts: 138 operations instead of 214. For
-// storage of 32 bits and more (another order of rounding flips last bits of
-// 16-bit values).
+// FP64 and batched collisions, and for moments and diagnostics of every storage; the
+// collisions of FP32 and 16-bit lattices keep raw_moments (see kShells).
 template <typename V>
 __device__ __forceinline__ void raw_moments_shells(const V (&h)[kQ], Mom<V>& m) {
   using S = scalar_t<V>;
@@ -265,8 +267,9 @@ __device__ __forceinline__ void raw_moments_shells(const V (&h)[kQ], Mom<V>& m) 
 }
 
 // Storage whose one-point kernels use the factored sums and targets: FP64. FP32 and
-// 16-bit lattices keep the rounding of the pair-by-pair form: the totals of a state
-// follow it to parts in 1e8 a step.
+// 16-bit lattices keep the pair-by-pair form so that their stored states keep their
+// bits, not for accuracy: over random states both forms shift mass and energy by the
+// same parts in 1e8 a step, which come from the rounded constants they share.
 template <typename Store>
 constexpr bool kShells = sizeof(Store) == 8;
 
@@ -512,7 +515,7 @@ __device__ __forceinline__ void mix_coeffs(const Mom<V>& m, const StepConst<Real
 // c_relax (f^mix/w - 1) in H. The products j_a u_b serve the temperature, the
 // stress and both orders of the expansion, and products of constants come from
 // the launch (about 130 operations instead of 240). FP64 lattices and the batched
-// tubes use it; FP32 lattices keep the other rounding, as their totals do then.
+// tubes use it; FP32 and 16-bit lattices keep their bits (see kShells).
 template <typename Real, bool kPaper, typename V>
 __device__ __forceinline__ void relaxed_target(Mom<V>& m, V e, const StepConst<Real>& K, Herm<V>& H) {
   using S = scalar_t<V>;

@@ -274,7 +274,7 @@ __global__ void k_line_transport(StepConst<Real> K, const Real* e, const Real* u
   pdl_wait();
   extern __shared__ __align__(16) unsigned char line_smem[];
   const int T = blockDim.x, l = threadIdx.x, nx = K.nx;
-  Real* s0 = reinterpret_cast<Real*>(line_smem);  // two slots per thread, one spare at each end
+  Real* s0 = reinterpret_cast<Real*>(line_smem);  // two slots per thread
   Real* s1 = s0 + T;
   const int lo = nsub + (kFirst ? 1 : 0), hi = nsub + (kFirst ? 1 : 0);
   const int own = T - lo - hi;  // points this tile writes
