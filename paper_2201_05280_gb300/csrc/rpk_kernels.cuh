@@ -1013,8 +1013,9 @@ __device__ __forceinline__ double widen_scaled(float x) {
 // f ln f takes one logarithm, a product and an FMA per population (a logarithm of
 // f <= 0 gives the NaN by itself, and sum f = rho), and the smallest g comes from the
 // smallest h of each shell. 256^3: 2.96 ms with 12 FP64 additions, 9 conversions and six
-// operations around each of the 41 logarithms a point, 1.54 ms now (paper's solver 3.25
-// and 1.58); with conversions by branching integer code 1.61 and 1.68.
+// operations around each of the 41 logarithms a point, 1.51 ms now (paper's solver 3.25
+// and 1.53); with every value joining its sum after the logarithms 1.54 and 1.58 (more
+// spills), with conversions by branching integer code 1.61 and 1.68.
 template <typename Store, bool kPaper>
 __global__ void __launch_bounds__(kDiagThreads, 3)
     k_diag_pair(StepConst<float> K, const Store* __restrict__ pin, const float* __restrict__ e_in,
@@ -1051,6 +1052,31 @@ __global__ void __launch_bounds__(kDiagThreads, 3)
       gm = fminf(gm, float(pair_weight(k0)) * (1.f + hm));
     });
     gmin = fminf(gmin, gm);
+    // the point's values join the sums by w: integer widening, or where a value is not
+    // finite (0 times it is NaN) a conversion
+    auto join = [&](F2 nil, auto&& add) {
+      if (nil.v.x + nil.v.y == 0.f)
+        add([](float x) { return widen_scaled(x); });
+      else
+        add([](float x) { return (double)x * 0x1p-896; });
+    };
+    F2 nil = 0.f * m.drho;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) nil = fmad(0.f, m.dP[a], fmad(0.f, m.j[a], nil));
+    join(fmad(0.f, kPaper ? m.dR : e, nil), [&](auto&& w) {
+      auto both = [&](F2 a) { return w(a.v.x) + w(a.v.y); };
+      sum[0] += both(m.drho);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) sum[1 + a] += both(m.j[a]);
+      sum[4] += both(m.dP[0]) + both(m.dP[1]) + both(m.dP[2]);
+      if constexpr (kPaper) {
+        // paper mode holds theta_R: rho theta_R - theta0 (times delta / 2 below)
+        auto er = [&](float rho, float dR) { return fma(w(rho), fma(w(dR), 0x1p896, t0), -t0 * 0x1p-896); };
+        sum[5] += er(m.rho.v.x, m.dR.v.x) + er(m.rho.v.y, m.dR.v.y);
+      } else {
+        sum[5] += both(e);
+      }
+    });
     // H1: sum f ln f - sum f - (delta/2) rho ln theta_R, f = (1 - beta*) g + beta* f^mix
     Herm<F2> H;
     mix_coeffs(m, K, H);
@@ -1065,30 +1091,8 @@ __global__ void __launch_bounds__(kDiagThreads, 3)
       Hl = fmad(w * fm, lg2(fm), Hl);
     });
     Hl = fmad((-0.5f * K.delta) * m.rho, lg2(m.dR + K.theta0), Hl);
-    // H1 in units of ln 2, and rho as 1 + drho: the sums of -drho and -1 follow below
-    auto join = [&](auto&& w) {
-      auto both = [&](F2 a) { return w(a.v.x) + w(a.v.y); };
-      sum[0] += both(m.drho);
-#pragma unroll
-      for (int a = 0; a < 3; ++a) sum[1 + a] += both(m.j[a]);
-      sum[4] += both(m.dP[0]) + both(m.dP[1]) + both(m.dP[2]);
-      if constexpr (kPaper) {
-        // paper mode holds theta_R: rho theta_R - theta0 (times delta / 2 below)
-        auto er = [&](float rho, float dR) { return fma(w(rho), fma(w(dR), 0x1p896, t0), -t0 * 0x1p-896); };
-        sum[5] += er(m.rho.v.x, m.dR.v.x) + er(m.rho.v.y, m.dR.v.y);
-      } else {
-        sum[5] += both(e);
-      }
-      sum[6] += both(Hl);
-    };
-    F2 nil = fmad(0.f, Hl, 0.f * m.drho);  // 0, or NaN where a term is not finite
-#pragma unroll
-    for (int a = 0; a < 3; ++a) nil = fmad(0.f, m.dP[a], fmad(0.f, m.j[a], nil));
-    nil = fmad(0.f, kPaper ? m.dR : e, nil);
-    if (nil.v.x + nil.v.y == 0.f)
-      join([](float x) { return widen_scaled(x); });
-    else
-      join([](float x) { return (double)x * 0x1p-896; });
+    // in units of ln 2, and rho as 1 + drho: the sums of -drho and -1 follow below
+    join(0.f * Hl, [&](auto&& w) { sum[6] += w(Hl.v.x) + w(Hl.v.y); });
     npts_here += 2;
   }
   const double ln2 = 0.6931471805599453094, n = (double)npts_here;
