@@ -19,7 +19,11 @@ struct BrickPlan {
     int own[3];
   };
   int nsub = 0, open = -1;
-  std::vector<Part> parts;
+  // the first launch, then equal ones, then equal ones of a sub-step less
+  Part part[3];
+  int times[3] = {0, 0, 0};
+  int launches() const { return times[0] + times[1] + times[2]; }
+  const Part& at(int i) const { return part[i < times[0] ? 0 : i < times[0] + times[1] ? 1 : 2]; }
 };
 
 struct rpk_lattice {

@@ -274,10 +274,13 @@ static inline auto brick_kernel(bool first, int planes) {
 static inline rpk_status make_brick_plan(rpk_lattice* L, int open) {
   BrickPlan& B = L->brick;
   if (B.nsub == L->nsub && B.open == open) return RPK_OK;
-  B.nsub = L->nsub;
-  B.open = open;
-  B.parts.clear();
-  if (L->n3 > (int64_t)kBrickMaxP * kBrickThreads * L->sms) return RPK_OK;
+  B = BrickPlan();
+  auto made = [&] {
+    B.nsub = L->nsub;
+    B.open = open;
+    return RPK_OK;
+  };
+  if (L->n3 > (int64_t)kBrickMaxP * kBrickThreads * L->sms) return made();
   const int n[3] = {L->grid.nx, L->grid.ny, L->grid.nz};
   static constexpr int kCuts[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32, 48, 64, 96, 128};
   // the cuts of an axis that give tiles of different length, fewest first
@@ -328,25 +331,24 @@ static inline rpk_status make_brick_plan(rpk_lattice* L, int open) {
     if (shorter > 1) c += (shorter - 1) * best(m - 1, false, rest);
     if (c < cost) {
       cost = c;
-      B.parts.assign(1, first);
-      for (int i = 0; i < nfull / m; ++i) B.parts.push_back(full);
-      for (int i = 1; i < shorter; ++i) B.parts.push_back(rest);
+      B.part[0] = first, B.part[1] = full, B.part[2] = rest;
+      B.times[0] = 1, B.times[1] = nfull / m, B.times[2] = std::max(0, shorter - 1);
     }
   }
-  if (B.parts.empty()) return RPK_OK;
+  if (!B.launches()) return made();
   for (int planes = 1; planes <= kBrickMaxP; ++planes)
     for (bool first : {true, false})
       RPK_CUDA(cudaFuncSetAttribute(brick_kernel(first, planes), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBrickSmem));
-  return RPK_OK;
+  return made();
 }
 
 // Transport of a small lattice in FP32 by its plan (conservative form).
 static inline rpk_status brick_launch(rpk_lattice* L, const StepConst<float>& K, int open) {
   const float* src = static_cast<const float*>(L->e_star);
   RPK_CUDA(timing_begin(L));
-  const size_t parts = L->brick.parts.size();
-  for (size_t i = 0; i < parts; ++i) {
-    const BrickPlan::Part& part = L->brick.parts[i];
+  const int parts = L->brick.launches();
+  for (int i = 0; i < parts; ++i) {
+    const BrickPlan::Part& part = L->brick.at(i);
     BrickArgs B{};
     B.nsub = part.nsub;
     B.open = open;
@@ -374,7 +376,7 @@ static inline rpk_status brick_launch(rpk_lattice* L, const StepConst<float>& K,
                 static_cast<const float*>(L->ghost));
     src = dst;
   }
-  RPK_CUDA(timing_end(L, RPK_KC_TRANSPORT, (int)parts));
+  RPK_CUDA(timing_end(L, RPK_KC_TRANSPORT, parts));
   return check_launch("rotational transport (brick)");
 }
 
@@ -478,7 +480,7 @@ rpk_status Ops<Store, Real>::step(rpk_lattice* L, int64_t n) {
     if (!L->rot_mode && (wm || L->grid.ny > 1 || L->grid.nz > 1)) {
       const rpk_status st = make_brick_plan(L, res ? 1 : wm);
       if (st != RPK_OK) return st;
-      brick = !L->brick.parts.empty();
+      brick = L->brick.launches() > 0;
     }
   }
   for (int64_t t = 0; t < n; ++t) {
